@@ -5,7 +5,7 @@ import subprocess
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 LIB = os.path.join(PKG, "libccsd_gb300.so")
-SOURCES = [os.path.join(PKG, "csrc", f) for f in ("ccsd_api.cu", "ccsd_noalloc.cu", "peak_probe.cu")]
+SOURCES = [os.path.join(PKG, "csrc", f) for f in ("ccsd_api.cu", "zgemm_launch.cu", "ccsd_noalloc.cu", "peak_probe.cu")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

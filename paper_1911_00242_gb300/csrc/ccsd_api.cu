@@ -28,7 +28,7 @@
 #include "ccsd_kernels.cuh"
 #include "tcgemm.cuh"
 #include "ozaki.cuh"
-#include "zgemm_kb.cuh"
+#include "zgemm_launch.h"
 #include "diis.h"
 #include "grouped.cuh"
 #include "kgrid.h"
@@ -66,12 +66,15 @@ enum Buf {
     NBUF
 };
 
+struct GemmVar {        // launch shape of one contraction in one arithmetic
+    int shape, nsplit, tiles_m, tiles_n;
+    long long blocks;   // tiles x batches
+};
+
 struct GemmPlan {
     int a, b, c;
-    GemmArgs args;      // device tables filled; A/B/C pointers resolved at launch
-    GemmArgs args32;    // the same for the FP32 instance: shorter FP32 partial sums (split-K)
-    int cfg;            // tile configuration
-    int blocks;
+    GemmArgs args;      // device tables filled; pointers, tiles and splits resolved at launch
+    GemmVar var[ZG_ARITH];
 };
 
 struct CopyPlan {       // dst = (conj) src, n elements
@@ -139,6 +142,8 @@ struct ccsd_ctx {
     int* kb_of = nullptr;            // fourth momentum of doubles blocks
     double2* work = nullptr;         // split-K partials
     size_t work_elems = 0;
+    int* cnt = nullptr;              // finished splits per output tile of a split contraction
+    size_t cnt_need = 0;
     double* red = nullptr;           // reduction partials
     double* red_out = nullptr;       // scalars
     double2* cred = nullptr;
@@ -266,13 +271,6 @@ struct GemmSpec {
     double ar = 1.0, ai = 0.0;
 };
 
-// Tile configurations: (BM, BN, BK, TM, TN[, KS]), 256 threads each.  The two K-split
-// shapes (KS thread groups share each K step) serve skinny contractions with K >= 32.
-enum { CFG_64x64 = 0, CFG_64x32 = 1, CFG_128x16 = 2, CFG_16x16 = 3, CFG_32x16 = 4, CFG_16x16K = 5, CFG_32x16K = 6,
-       CFG_COUNT = 7 };
-const int CFG_BM[CFG_COUNT] = {64, 64, 128, 16, 32, 16, 32};
-const int CFG_BN[CFG_COUNT] = {64, 32, 16, 16, 16, 16, 16};
-
 const int kSMs = 152;
 const int kRedBlocks = kSMs * 4;    // blocks of the reductions (max|R|, inner products, energy)
 
@@ -289,9 +287,10 @@ int finalize_gemm(ccsd_ctx* h, Alloc& al, GemmSpec s, size_t& work_need) {
         // an empty contraction (no momentum blocks for this shape): kept as a no-op step
         // so that every problem has the same step sequence (batched form)
         GemmPlan p{};
-        p.a = s.a; p.b = s.b; p.c = s.c; p.cfg = CFG_16x16; p.blocks = 0;
+        p.a = s.a; p.b = s.b; p.c = s.c;
         p.args.M = std::max(s.M, 1); p.args.N = std::max(s.N, 1); p.args.K = s.K;
-        p.args.nbatch = 0; p.args.nchunk = std::max(s.nchunk, 1); p.args.nsplit = 1; p.args.chunks_per_split = 1;
+        p.args.nbatch = 0; p.args.nchunk = std::max(s.nchunk, 1); p.args.nsplit = 1;
+        for (GemmVar& w : p.var) w = GemmVar{3, 1, 1, 1, 0};
         h->gemms.push_back(p);
         h->seq.push_back({0, (int)h->gemms.size() - 1, h->cur_name, 0.0, 0.0});
         return 0;
@@ -352,26 +351,28 @@ int finalize_gemm(ccsd_ctx* h, Alloc& al, GemmSpec s, size_t& work_need) {
         g0.a0 = g0.affA ? (long long)s.rowA[0] + s.colA[0] : 0;
         g0.b0 = g0.affB ? (long long)s.rowB[0] + s.colB[0] : 0;
     }
-    if (s.N >= 48) p.cfg = CFG_64x64;
-    else if (s.N > 16) p.cfg = CFG_64x32;
-    else if (s.M > 64) p.cfg = CFG_128x16;
-    else if (s.M > 16) p.cfg = s.K >= 32 ? CFG_32x16K : CFG_32x16;
-    else p.cfg = s.K >= 32 ? CFG_16x16K : CFG_16x16;
     GemmArgs& g = p.args;
     g.M = s.M; g.N = s.N; g.K = s.K; g.nbatch = s.nbatch; g.nchunk = s.nchunk;
     g.conjA = s.conjA; g.conjB = s.conjB; g.accumulate = s.acc ? 1 : 0;
     g.alpha_re = s.ar; g.alpha_im = s.ai;
-    g.tiles_m = (s.M + CFG_BM[p.cfg] - 1) / CFG_BM[p.cfg];
-    g.tiles_n = (s.N + CFG_BN[p.cfg] - 1) / CFG_BN[p.cfg];
-    const long long ctas = (long long)g.tiles_m * g.tiles_n * s.nbatch;
-    int nsplit = 1;
-    if (ctas < 2 * kSMs && s.nchunk > 1) {
-        nsplit = (int)std::min<long long>(s.nchunk, (4 * kSMs + ctas - 1) / ctas);
+    // Tile shape and K split for each arithmetic the step may run in (zgemm_shapes.h); the
+    // operands with a complex64 copy in mixed iterations are those to_c64 refreshes
+    for (int w = 0; w < ZG_ARITH; ++w) {
+        if (w == ZG_FP32 && h->cfg.precision != CCSD_MIXED) { p.var[w] = p.var[ZG_FP64]; continue; }
+        if (w == ZG_DF && !h->has_oz) { p.var[w] = p.var[ZG_FP64]; continue; }
+        auto wide = [&](int b) { return w == ZG_FP32 ? h->shadow[b] == nullptr : !h->in32[b]; };
+        const ZgChoice ch = zg_choose(w, s.M, s.N, s.K, s.nchunk, s.nbatch, (wide(s.a) ? 1 : 0) + (wide(s.b) ? 1 : 0),
+                                      kSMs);
+        const ZgShape& sh = kZgShapes[ch.shape];
+        GemmVar& v = p.var[w];
+        v.shape = ch.shape; v.nsplit = ch.nsplit;
+        v.tiles_m = (s.M + sh.bm - 1) / sh.bm; v.tiles_n = (s.N + sh.bn - 1) / sh.bn;
+        v.blocks = (long long)v.tiles_m * v.tiles_n * s.nbatch;
+        if (v.nsplit > 1) {
+            work_need = std::max(work_need, (size_t)v.nsplit * s.nbatch * s.M * s.N);
+            h->cnt_need = std::max(h->cnt_need, (size_t)v.blocks);
+        }
     }
-    g.chunks_per_split = (s.nchunk + nsplit - 1) / nsplit;
-    g.nsplit = (s.nchunk + g.chunks_per_split - 1) / g.chunks_per_split;
-    if (g.nsplit > 1) work_need = std::max(work_need, (size_t)g.nsplit * s.nbatch * s.M * s.N);
-    p.blocks = (int)ctas;
     g.offA = upload(al, s.offA, h->st); g.offB = upload(al, s.offB, h->st); g.offC = upload(al, s.offC, h->st);
     g.rowA = upload(al, s.rowA, h->st); g.colA = upload(al, s.colA, h->st);
     g.rowB = upload(al, s.rowB, h->st); g.colB = upload(al, s.colB, h->st);
@@ -380,18 +381,6 @@ int finalize_gemm(ccsd_ctx* h, Alloc& al, GemmSpec s, size_t& work_need) {
     g.offC2 = s.offC2.empty() ? nullptr : upload(al, s.offC2, h->st);
     g.colC2 = s.colC2.empty() ? nullptr : upload(al, s.colC2, h->st);
     if (al.err) return al.err;
-    // FP32 instance (mixed form): an FP32 partial sum runs over at most kFp32Chain terms
-    // (or one momentum chunk); the chunk partials are added in FP64 by the split-K
-    // reduction, so the FP32 rounding error stays that of a short sum
-    p.args32 = g;
-    {
-        const long long kFp32Chain = 8192;
-        GemmArgs& g32 = p.args32;
-        if ((long long)g32.chunks_per_split * s.K > kFp32Chain && s.nchunk > 1) {
-            g32.chunks_per_split = (int)std::max<long long>(1, kFp32Chain / std::max(1, s.K));
-            g32.nsplit = (s.nchunk + g32.chunks_per_split - 1) / g32.chunks_per_split;
-        }   // its split-K workspace is sized in setup_handle, for the steps that run in FP32
-    }
     h->gemms.push_back(p);
     double chunks = (double)s.nchunk * s.nbatch;
     if (!s.nchunk_b.empty()) { chunks = 0.0; for (int x : s.nchunk_b) chunks += x; }
@@ -1832,53 +1821,27 @@ dim3 ew_grid(long long n) {
     return dim3((unsigned)b);
 }
 
+// A contraction's arguments in one arithmetic, with the handle's buffers resolved.
+GemmArgs gemm_args(const ccsd_ctx* h, const GemmPlan& p, int arith) {
+    const GemmVar& v = p.var[arith];
+    const bool fp32 = arith == ZG_FP32;
+    GemmArgs g = p.args;
+    g.A = h->buf[p.a]; g.B = h->buf[p.b]; g.C = h->buf[p.c]; g.work = h->work; g.cnt = h->cnt;
+    g.A32 = (fp32 || h->in32[p.a]) ? h->shadow[p.a] : nullptr;
+    g.B32 = (fp32 || h->in32[p.b]) ? h->shadow[p.b] : nullptr;
+    g.tiles_m = v.tiles_m; g.tiles_n = v.tiles_n; g.nsplit = v.nsplit;
+    return g;
+}
+
+// Arithmetic of the contractions left off the tensor cores in the current iteration.
+int gemm_arith(const ccsd_ctx* h) { return h->oz_on ? ZG_DF : h->fp32 ? ZG_FP32 : ZG_FP64; }
+
 int launch_gemm(ccsd_ctx* h, GemmPlan& p) {
-    if (p.blocks == 0) return 0;
-    GemmArgs g = h->fp32 ? p.args32 : p.args;
-    g.A = h->buf[p.a]; g.B = h->buf[p.b]; g.C = h->buf[p.c]; g.work = h->work;
-    g.A32 = (h->fp32 || h->in32[p.a]) ? h->shadow[p.a] : nullptr;
-    g.B32 = (h->fp32 || h->in32[p.b]) ? h->shadow[p.b] : nullptr;
-    dim3 grid((unsigned)p.blocks, (unsigned)g.nsplit);
-    // the K-split tile shapes pay off in FP32 only (measured on GB300: the double-float
-    // instance ran slower with them, the FP64 one no faster); the other instances take
-    // the plain shape with the same tile, so the plan's tiling and split-K stand
-    const int cfg = h->fp32 ? p.cfg : p.cfg == CFG_16x16K ? CFG_16x16 : p.cfg == CFG_32x16K ? CFG_32x16 : p.cfg;
-    if (h->oz_on) {         // Ozaki form: the GEMMs left off the tensor cores run in double-float
-        switch (cfg) {
-            case CFG_64x64:  zgemm_kb_kernel<64, 64, 8, 4, 4, df><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_64x32:  zgemm_kb_kernel<64, 32, 8, 4, 2, df><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_128x16: zgemm_kb_kernel<128, 16, 8, 8, 1, df><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_32x16:  zgemm_kb_kernel<32, 16, 8, 2, 1, df><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_32x16K: zgemm_kb_kernel<32, 16, 32, 2, 2, df, 2><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_16x16K: zgemm_kb_kernel<16, 16, 32, 2, 2, df, 4><<<grid, 256, 0, h->st>>>(g); break;
-            default:         zgemm_kb_kernel<16, 16, 8, 1, 1, df><<<grid, 256, 0, h->st>>>(g); break;
-        }
-    } else if (h->fp32) {
-        switch (cfg) {
-            case CFG_64x64:  zgemm_kb_kernel<64, 64, 8, 4, 4, float><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_64x32:  zgemm_kb_kernel<64, 32, 8, 4, 2, float><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_128x16: zgemm_kb_kernel<128, 16, 8, 8, 1, float><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_32x16:  zgemm_kb_kernel<32, 16, 8, 2, 1, float><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_32x16K: zgemm_kb_kernel<32, 16, 32, 2, 2, float, 2><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_16x16K: zgemm_kb_kernel<16, 16, 32, 2, 2, float, 4><<<grid, 256, 0, h->st>>>(g); break;
-            default:         zgemm_kb_kernel<16, 16, 8, 1, 1, float><<<grid, 256, 0, h->st>>>(g); break;
-        }
-    } else {
-        switch (cfg) {
-            case CFG_64x64:  zgemm_kb_kernel<64, 64, 8, 4, 4><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_64x32:  zgemm_kb_kernel<64, 32, 8, 4, 2><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_128x16: zgemm_kb_kernel<128, 16, 8, 8, 1><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_32x16:  zgemm_kb_kernel<32, 16, 8, 2, 1><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_32x16K: zgemm_kb_kernel<32, 16, 32, 2, 2, double, 2><<<grid, 256, 0, h->st>>>(g); break;
-            case CFG_16x16K: zgemm_kb_kernel<16, 16, 32, 2, 2, double, 4><<<grid, 256, 0, h->st>>>(g); break;
-            default:         zgemm_kb_kernel<16, 16, 8, 1, 1><<<grid, 256, 0, h->st>>>(g); break;
-        }
-    }
+    const int arith = gemm_arith(h);
+    const GemmVar& v = p.var[arith];
+    if (v.blocks == 0) return 0;
+    launch_zgemm(arith, v.shape, gemm_args(h, p, arith), (int)v.blocks, h->st);
     ++h->launches;
-    if (g.nsplit > 1) {
-        zgemm_split_reduce<<<ew_grid((long long)g.nbatch * g.M * g.N), 256, 0, h->st>>>(g);
-        ++h->launches;
-    }
     return 0;
 }
 
@@ -2157,13 +2120,11 @@ int run_residual(ccsd_ctx* h) {
 //   * max|R| per member, and the update of the members not yet converged.
 // The group's launch descriptors are built once per membership on the host.
 struct BatchGroup {
-    int cfg = CFG_64x64;
+    int cfg = 0;                      // tile shape of the launch
     std::vector<GemmArgs> args;       // per member, tiles for `cfg`, pointers resolved
     GemmArgs* d_args = nullptr;
     long long* d_prefix = nullptr;
     long long total = 0;
-    std::vector<int> split_members;
-    std::function<void(cudaStream_t)> reduce;   // grouped split-K reduction (members that split)
 };
 
 // One grouped launch: enqueues itself on a stream (no host synchronization).
@@ -2287,86 +2248,76 @@ int make_grouped(Group& G, const std::vector<Op>& ops, const std::vector<long lo
 }
 
 long long tiles_for(const GemmArgs& a, int cfg, int* tm, int* tn) {
-    *tm = (a.M + CFG_BM[cfg] - 1) / CFG_BM[cfg];
-    *tn = (a.N + CFG_BN[cfg] - 1) / CFG_BN[cfg];
+    *tm = (a.M + kZgShapes[cfg].bm - 1) / kZgShapes[cfg].bm;
+    *tn = (a.N + kZgShapes[cfg].bn - 1) / kZgShapes[cfg].bn;
     return (long long)*tm * *tn * a.nbatch;
+}
+
+// A member's split-K workspace and tile counters, grown to what a grouped launch needs.
+int member_split_space(ccsd_ctx* h, size_t work, size_t tiles, cudaStream_t st) {
+    if (work > h->work_elems) {
+        void* w = nullptr;
+        if (cudaMalloc(&w, work * 16) != cudaSuccess) { cudaGetLastError(); return CCSD_ERR_OOM; }
+        h->owned.push_back(w);
+        h->owned_bytes += work * 16;
+        h->work = (double2*)w;
+        h->work_elems = work;
+    }
+    if (tiles > h->cnt_need) {
+        void* w = nullptr;
+        if (cudaMalloc(&w, tiles * sizeof(int)) != cudaSuccess) { cudaGetLastError(); return CCSD_ERR_OOM; }
+        h->owned.push_back(w);
+        h->owned_bytes += tiles * sizeof(int);
+        CK(cudaMemsetAsync(w, 0, tiles * sizeof(int), st));
+        h->cnt = (int*)w;
+        h->cnt_need = tiles;
+    }
+    return 0;
 }
 
 int group_gemm_descriptors(Group& G, BatchGroup& bg, size_t si, int cfg, cudaStream_t st, bool own_split = false) {
     const int n = (int)G.m.size();
+    const int arith = G.fp32 ? ZG_FP32 : ZG_FP64;
     bg.cfg = cfg;
     bg.args.clear();
-    bg.split_members.clear();
     // Split-K by load balance: the persistent CTAs stride one work list, so no work item
-    // (a tile and its share of the chunks) should hold more than half the mean load of a
-    // CTA.  Skinny contractions (a few tiles over a long K, like the F~ and R1 sums) are
-    // then spread over many CTAs even when the whole group has plenty of tiles.
+    // (a tile and its share of the sum) should hold more than half the mean load of a
+    // CTA.  Contractions with few outputs (a few tiles over a long K, like the F~ and R1
+    // sums) are then spread over many CTAs even when the whole group has plenty of tiles.
     double total_work = 0.0;             // sum over members of tiles x K x chunks
     for (int i = 0; i < n; ++i) {
         int tm, tn;
         const GemmArgs& a0 = G.m[i]->gemms[G.m[i]->seq[si].idx].args;
         total_work += (double)tiles_for(a0, cfg, &tm, &tn) * a0.K * a0.nchunk;
     }
-    const double item_cap = std::max(1.0, 0.5 * total_work / (double)(kSMs * 8));
+    const double item_cap = std::max(4.0 * kZgUnit, 0.5 * total_work / (double)(kSMs * 8));
     long long tot = 0;
     std::vector<long long> prefix;
-    std::vector<SplitReduceOp> red;
-    std::vector<long long> red_blocks;
     for (int i = 0; i < n; ++i) {
         ccsd_ctx* h = G.m[i];
         const GemmPlan& p = h->gemms[h->seq[si].idx];
-        GemmArgs a = G.fp32 ? p.args32 : p.args;
-        int tm, tn;
-        tiles_for(a, cfg, &tm, &tn);
+        const GemmVar& v = p.var[arith];
+        int tm, tn, ns = v.nsplit;
+        tiles_for(p.args, cfg, &tm, &tn);
         if (own_split) {
-            if (cfg != p.cfg) { refuse("members of a split-keeping group must share each step's tile shape"); return CCSD_ERR_INVALID; }
-            a.A = h->buf[p.a]; a.B = h->buf[p.b]; a.C = h->buf[p.c]; a.work = h->work;
-            a.A32 = (G.fp32 || h->in32[p.a]) ? h->shadow[p.a] : nullptr;
-            a.B32 = (G.fp32 || h->in32[p.b]) ? h->shadow[p.b] : nullptr;
-            if (a.nsplit > 1) {
-                bg.split_members.push_back(i);
-                red.push_back(SplitReduceOp{a});
-                red_blocks.push_back(grid_blocks(ew_grid((long long)a.nbatch * a.M * a.N)));
-            }
-            prefix.push_back(tot);
-            tot += (long long)tm * tn * a.nbatch * a.nsplit;
-            bg.args.push_back(a);
-            continue;
-        }
-        a.tiles_m = tm; a.tiles_n = tn;
-        const int ns = std::max(1, std::min(a.nchunk, (int)std::ceil((double)a.K * a.nchunk / item_cap)));
-        a.chunks_per_split = (a.nchunk + ns - 1) / ns;
-        a.nsplit = (a.nchunk + a.chunks_per_split - 1) / a.chunks_per_split;
-        if (G.fp32) {        // the FP32 instance keeps its partial sums short (see finalize_gemm)
-            const GemmArgs& g32 = p.args32;
-            if (g32.chunks_per_split < a.chunks_per_split) {
-                a.chunks_per_split = g32.chunks_per_split;
-                a.nsplit = (a.nchunk + a.chunks_per_split - 1) / a.chunks_per_split;
+            if (cfg != v.shape && v.blocks > 0) { refuse("members of a split-keeping group must share each step's tile shape"); return CCSD_ERR_INVALID; }
+        } else {
+            const long long units = (long long)p.args.nchunk * ((p.args.K + kZgUnit - 1) / kZgUnit);
+            ns = (int)std::max<long long>(1, std::min<long long>(std::min<long long>(units, kZgMaxSplit),
+                                              (long long)std::ceil((double)p.args.K * p.args.nchunk / item_cap)));
+            if (G.fp32) ns = std::max(ns, (int)zg_fp32_splits(p.args.K, p.args.nchunk));   // short FP32 partial sums
+            if (p.args.nbatch == 0) ns = 1;
+            if (ns > 1) {
+                const int rc = member_split_space(h, (size_t)ns * p.args.nbatch * p.args.M * p.args.N,
+                                                  (size_t)tm * tn * p.args.nbatch, st);
+                if (rc) return rc;
             }
         }
-        if (a.nbatch == 0) a.nsplit = 1;
-        if (a.nsplit > 1) {
-            const size_t need = (size_t)a.nsplit * a.nbatch * a.M * a.N;
-            if (need > h->work_elems) {          // the handle owns its split-K workspace
-                void* w = nullptr;
-                if (cudaMalloc(&w, need * 16) != cudaSuccess) { cudaGetLastError(); return CCSD_ERR_OOM; }
-                h->owned.push_back(w);
-                h->owned_bytes += need * 16;
-                h->work = (double2*)w;
-                h->work_elems = need;
-            }
-            bg.split_members.push_back(i);
-        }
-        a.A = h->buf[p.a]; a.B = h->buf[p.b]; a.C = h->buf[p.c]; a.work = h->work;
-        a.A32 = (G.fp32 || h->in32[p.a]) ? h->shadow[p.a] : nullptr;
-        a.B32 = (G.fp32 || h->in32[p.b]) ? h->shadow[p.b] : nullptr;
+        GemmArgs a = gemm_args(h, p, arith);
+        a.tiles_m = tm; a.tiles_n = tn; a.nsplit = ns;
         prefix.push_back(tot);
         tot += (long long)tm * tn * a.nbatch * a.nsplit;
         bg.args.push_back(a);
-        if (a.nsplit > 1) {
-            red.push_back(SplitReduceOp{a});
-            red_blocks.push_back(grid_blocks(ew_grid((long long)a.nbatch * a.M * a.N)));
-        }
     }
     prefix.push_back(tot);
     bg.total = tot;
@@ -2380,38 +2331,22 @@ int group_gemm_descriptors(Group& G, BatchGroup& bg, size_t si, int cfg, cudaStr
     }
     CK(cudaMemcpyAsync(bg.d_args, bg.args.data(), sizeof(GemmArgs) * n, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(bg.d_prefix, prefix.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, st));
-    bg.reduce = nullptr;
-    if (!red.empty()) {
-        GLaunch gl;
-        int rc = make_grouped(G, red, red_blocks, st, gl);
-        if (rc) return rc;
-        bg.reduce = gl.fn;
-    }
     return 0;
-}
-
-template <int BM, int BN, int BK, int TM, int TN, int KS = 1>
-void grouped_gemm_launch(const BatchGroup& bg, int fp32, cudaStream_t st, int n) {
-    const long long ctas = std::min<long long>(bg.total, (long long)kSMs * 8);
-    if (fp32)
-        zgemm_grouped_kernel<BM, BN, BK, TM, TN, float, KS><<<(unsigned)ctas, 256, 0, st>>>(bg.d_args, bg.d_prefix, n, bg.total);
-    else
-        zgemm_grouped_kernel<BM, BN, BK, TM, TN, double, KS><<<(unsigned)ctas, 256, 0, st>>>(bg.d_args, bg.d_prefix, n, bg.total);
 }
 
 void launch_gemm_group(const BatchGroup& bg, int fp32, cudaStream_t st, int n) {
     if (bg.total <= 0 || !bg.d_args) return;
-    const int cfg = fp32 ? bg.cfg : bg.cfg == CFG_16x16K ? CFG_16x16 : bg.cfg == CFG_32x16K ? CFG_32x16 : bg.cfg;
-    switch (cfg) {
-        case CFG_64x64: grouped_gemm_launch<64, 64, 8, 4, 4>(bg, fp32, st, n); break;
-        case CFG_64x32: grouped_gemm_launch<64, 32, 8, 4, 2>(bg, fp32, st, n); break;
-        case CFG_128x16: grouped_gemm_launch<128, 16, 8, 8, 1>(bg, fp32, st, n); break;
-        case CFG_32x16: grouped_gemm_launch<32, 16, 8, 2, 1>(bg, fp32, st, n); break;
-        case CFG_32x16K: grouped_gemm_launch<32, 16, 32, 2, 2, 2>(bg, fp32, st, n); break;
-        case CFG_16x16K: grouped_gemm_launch<16, 16, 32, 2, 2, 4>(bg, fp32, st, n); break;
-        default: grouped_gemm_launch<16, 16, 8, 1, 1>(bg, fp32, st, n); break;
+    launch_zgemm_grouped(fp32 ? ZG_FP32 : ZG_FP64, bg.cfg, bg.d_args, bg.d_prefix, n, bg.total,
+                         (int)std::min<long long>(bg.total, (long long)kSMs * 8), st);
+}
+
+// Tile shape of a grouped contraction before any autotuning: the first member's with work.
+int group_shape(const Group& G, size_t si, int arith) {
+    for (const ccsd_ctx* h : G.m) {
+        const GemmVar& v = h->gemms[h->seq[si].idx].var[arith];
+        if (v.blocks > 0) return v.shape;
     }
-    if (bg.reduce) bg.reduce(st);
+    return 3;
 }
 
 // Builds every grouped launch of one iteration of the group's members.  d_norms[i]
@@ -2444,11 +2379,11 @@ int group_build(Group& G, int fp32, const std::vector<int>& cfgs, double* d_norm
         GLaunch gl;
         switch (s0.kind) {
             case 0: {
-                const int cfg = gi < (int)cfgs.size() ? cfgs[gi] : h0->gemms[s0.idx].cfg;
+                const int cfg = gi < (int)cfgs.size() ? cfgs[gi] : group_shape(G, si, fp32 ? ZG_FP32 : ZG_FP64);
                 if ((rc = group_gemm_descriptors(G, G.gemms[gi], si, cfg, st, own_split))) return rc;
                 const BatchGroup* bg = &G.gemms[gi];
                 gl.gemm = gi;
-                gl.launches = (bg->total > 0 ? 1 : 0) + (bg->reduce ? 1 : 0);
+                gl.launches = bg->total > 0 ? 1 : 0;
                 gl.fn = [bg, fp32, n](cudaStream_t s) { launch_gemm_group(*bg, fp32, s, n); };
                 ++gi;
                 break;
@@ -2694,10 +2629,12 @@ void batch_iteration_body(ccsd_batch* B) {
     }
 }
 
-// Autotuner: times every tile shape on every grouped contraction and keeps the
-// fastest.  Safe at any time: each residual re-initializes what it accumulates.
+// Autotuner: times the kTuneShapes tile shapes that the shape rule's model ranks first
+// for every grouped contraction (its ranking is within a few percent of the measured one,
+// so timing all shapes would only lengthen the first iteration) and keeps the fastest.
+// Safe at any time: each residual re-initializes what it accumulates.
+constexpr int kTuneShapes = 4;
 int batch_autotune(ccsd_batch* B) {
-    const int cands[CFG_COUNT] = {CFG_64x64, CFG_64x32, CFG_128x16, CFG_32x16, CFG_16x16, CFG_32x16K, CFG_16x16K};
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
@@ -2712,7 +2649,24 @@ int batch_autotune(ccsd_batch* B) {
             const size_t si = G.steps[k];
             int best = bg.cfg;
             float best_ms = 1e30f;
-            for (int c : cands) {
+            std::vector<std::pair<double, int>> order;
+            for (int c = 0; c < kZgShapeCount; ++c) {
+                double est = 0.0;               // the members' tiles share the launch
+                for (const ccsd_ctx* h : G.m) {
+                    const GemmPlan& p = h->gemms[h->seq[si].idx];
+                    if (p.args.nbatch == 0) continue;
+                    const int c128 = (h->in32[p.a] ? 0 : 1) + (h->in32[p.b] ? 0 : 1);
+                    double one = 1e300;
+                    for (int ns : {1, 4, 16, kZgMaxSplit})
+                        one = std::min(one, zg_estimate(B->fp32 ? ZG_FP32 : ZG_FP64, c, ns, p.args.M, p.args.N,
+                                                        p.args.K, p.args.nchunk, p.args.nbatch, c128, kSMs));
+                    est += one;
+                }
+                order.emplace_back(est, c);
+            }
+            std::sort(order.begin(), order.end());
+            for (int q = 0; q < kTuneShapes; ++q) {
+                const int c = order[(size_t)q].second;
                 if ((rc = group_gemm_descriptors(G, bg, si, c, B->st))) break;
                 launch_gemm_group(bg, B->fp32, B->st, n);     // warm
                 cudaEventRecord(e0, B->st);
@@ -2727,7 +2681,7 @@ int batch_autotune(ccsd_batch* B) {
                 if (ms < best_ms) { best_ms = ms; best = c; }
             }
             if (!rc) rc = group_gemm_descriptors(G, bg, si, best, B->st);
-            G.res[k].launches = (bg.total > 0 ? 1 : 0) + (bg.reduce ? 1 : 0);
+            G.res[k].launches = bg.total > 0 ? 1 : 0;
             ++gi;
         }
         if (rc) break;
@@ -2932,17 +2886,14 @@ int setup_handle(ccsd_ctx* h, Alloc& al, const void* const* ins, const bool* on_
     size_t work_need = 0;
     int rc = build_plan(h, al, work_need);
     if (rc) return rc;
-    if (h->cfg.precision == CCSD_MIXED) {
-        // GEMM steps that a mixed handle runs in FP32 (all but the FP64-only ones)
-        for (const Step& st : h->seq) {
-            if (st.kind != 0 || st.mode == 1 || st.mode == 4) continue;
-            const GemmArgs& g32 = h->gemms[st.idx].args32;
-            if (g32.nsplit > 1) work_need = std::max(work_need, (size_t)g32.nsplit * g32.nbatch * g32.M * g32.N);
-        }
-    }
     if (work_need) { h->work = dalloc((long long)work_need); if (!h->work) return al.err; }
     if (h->oz_work_elems) { h->oz_work = dalloc(h->oz_work_elems); if (!h->oz_work) return al.err; }
     h->work_elems = work_need;
+    if (h->cnt_need) {
+        h->cnt = (int*)al.get(h->cnt_need * sizeof(int));
+        if (!h->cnt) return al.err;
+        if (!al.dry && cudaMemsetAsync(h->cnt, 0, h->cnt_need * sizeof(int), h->st) != cudaSuccess) return CCSD_ERR_CUDA;
+    }
     h->red_blocks = kRedBlocks;
     h->red = (double*)al.get(sizeof(double) * h->red_blocks);
     h->red_out = (double*)al.get(sizeof(double) * 4);
@@ -3178,7 +3129,10 @@ std::vector<long long> server_key(const ccsd_ctx* h) {
     std::vector<long long> k{h->fp32, h->oz_on, h->cfg.precision};
     for (const Step& st : h->seq) {
         k.push_back(st.kind * 16 + st.mode);
-        if (st.kind == 0) k.push_back(h->gemms[st.idx].cfg);
+        if (st.kind == 0) {
+            const GemmVar& v = h->gemms[st.idx].var[h->fp32 ? ZG_FP32 : ZG_FP64];
+            k.push_back(v.blocks > 0 ? v.shape : -1);
+        }
     }
     return k;
 }
@@ -3474,8 +3428,7 @@ int ccsd_plan_check(const ccsd_config* cfg, long long* n_launches, size_t* table
     const int rc = build_plan(h, al, work_need);
     long long n = 0;
     for (const Step& st : h->seq)
-        n += ((st.kind == 0 && h->gemms[st.idx].args.nsplit > 1) || (st.kind == 6 && h->tcs[st.idx].oz &&
-              h->tcs[st.idx].z.nsplit > 1)) ? 2 : 1;
+        n += (st.kind == 6 && h->tcs[st.idx].oz && h->tcs[st.idx].z.nsplit > 1) ? 2 : 1;
     if (n_launches) *n_launches = n;
     if (table_bytes) *table_bytes = h->owned_bytes;
     delete h;
@@ -3520,6 +3473,11 @@ int tc_selftest_impl(int M, int Ncols, int K, int nterms, unsigned long long see
     int rc = finalize_gemm(h, al, g, work_need);
     if (rc) return fail(rc);
     if (work_need) { h->work = (double2*)al.get(work_need * 16); if (!h->work) return fail(al.err); }
+    if (h->cnt_need) {
+        h->cnt = (int*)al.get(h->cnt_need * sizeof(int));
+        if (!h->cnt) return fail(al.err);
+        if (cudaMemsetAsync(h->cnt, 0, h->cnt_need * sizeof(int), h->st) != cudaSuccess) return fail(CCSD_ERR_CUDA);
+    }
     // tensor cores: embed, GEMM
     const int kpad = (2 * K + TC_BK - 1) / TC_BK * TC_BK;
     TcBuf ta{}, tb{};

@@ -84,7 +84,7 @@ __device__ __forceinline__ df2 ld_df2(const df2* p) { return *p; }
 
 // dst = src as double-float pairs (the split costs FP64 operations, so constant inputs
 // are converted once)
-__global__ void to_df2_kernel(df2* __restrict__ dst, const double2* __restrict__ src, long long n)
+static __global__ void to_df2_kernel(df2* __restrict__ dst, const double2* __restrict__ src, long long n)
 {
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
          e += (long long)gridDim.x * blockDim.x)
