@@ -464,16 +464,24 @@ int encode_map_bf16(CUtensorMap* m, const uint16_t* base, long long rows, int kp
 int tc_mode(const ccsd_ctx* h) { return h->cur_oz ? 5 : 2; }
 
 // A tensor-core operand: split-TF32 parts (big, small: rows x kpad floats each), or for
-// the Ozaki form BF16 slice planes (sl: planes x rows x kpad) and row scales (sc).
-struct TcBuf { float* big; float* small; long long rows; int kpad; uint16_t* sl = nullptr; float* sc = nullptr; };
+// the Ozaki form BF16 slice planes (sl: planes x rows x kpad) and row scales (sc, sc_rows
+// of them).
+struct TcBuf {
+    float* big; float* small; long long rows; int kpad;
+    uint16_t* sl = nullptr;
+    float* sc = nullptr;
+    long long sc_rows = 0;
+};
 
-int tc_alloc(ccsd_ctx* h, Alloc& al, TcBuf& t, long long rows, int kpad) {
+// sc_rows: row scales to hold, if the buffer is also viewed with shorter (more) rows.
+int tc_alloc(ccsd_ctx* h, Alloc& al, TcBuf& t, long long rows, int kpad, long long sc_rows = 0) {
     t.rows = rows; t.kpad = kpad;
+    t.sc_rows = std::max(rows, sc_rows);
     if (h->cur_oz) {
         const size_t bytes = (size_t)rows * kpad * 2 * h->oz_slices;
         t.big = t.small = nullptr;
         t.sl = (uint16_t*)al.get(bytes);
-        t.sc = (float*)al.get((size_t)rows * 4);
+        t.sc = (float*)al.get((size_t)t.sc_rows * 4);
         if (al.err) return al.err;
         if (!al.dry && cudaMemsetAsync(t.sl, 0, bytes, h->st) != cudaSuccess) return CCSD_ERR_CUDA;
         return 0;
@@ -500,7 +508,10 @@ int add_embed(ccsd_ctx* h, Alloc& al, int src, const TcBuf& dst, int mode, int R
     const long long lo = *std::min_element(srcoff.begin(), srcoff.end()) + *std::min_element(srow.begin(), srow.end()) +
                          *std::min_element(scol.begin(), scol.end());
     if (lo < 0 || hi >= h->bufsize[src]) { refuse("an operand gather offset is out of range (32-bit tables)"); return CCSD_ERR_INVALID; }
-    if (nblk * R * (mode == 0 ? 1 : 2) > dst.rows) { refuse("an embedded operand exceeds its buffer"); return CCSD_ERR_INVALID; }
+    if (nblk * R * (mode == 0 ? 1 : 2) > dst.rows || (h->cur_oz && dst.rows > dst.sc_rows)) {
+        refuse("an embedded operand exceeds its buffer");
+        return CCSD_ERR_INVALID;
+    }
     EmbedPlan e{};
     e.src = src;
     e.a.srcoff = upload(al, srcoff, h->st);
@@ -758,8 +769,8 @@ int oz_convert_gemms(ccsd_ctx* h, Alloc& al, std::map<int, GemmSpec>& specs, boo
             std::vector<long long> offa((size_t)ia.size()), offb((size_t)ib.size());
             for (auto& kv : ia) offa[(size_t)kv.second] = kv.first;
             for (auto& kv : ib) offb[(size_t)kv.second] = kv.first;
-            TcBuf A{nullptr, nullptr, (long long)ia.size() * s.M, kpad, ga, gasc};
-            TcBuf B{nullptr, nullptr, (long long)ib.size() * 2 * s.N, kpad, gb, gbsc};
+            TcBuf A{nullptr, nullptr, (long long)ia.size() * s.M, kpad, ga, gasc, capRA};
+            TcBuf B{nullptr, nullptr, (long long)ib.size() * 2 * s.N, kpad, gb, gbsc, capRB};
             int rc;
             if ((rc = add_embed(h, al, s.a, A, 0, s.M, s.K, offa, s.rowA, s.colA, false, s.conjA)) ||
                 (rc = add_embed(h, al, s.b, B, 1, s.N, s.K, offb, s.colB, s.rowB, false, s.conjB)))
@@ -812,6 +823,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
         long long epb;                       // bytes per operand element
         TcBuf la, lap, lb, ra, rb, b1, ha, hb, h2a, h2b;
         long long lb_floats;                 // ladder B capacity (elements per part / slice plane)
+        long long lb_sc_rows;                // and its row scales (Ozaki): the (e < f) rows are shorter
         long long lad_max, lad_cap, pa, pb;  // sizes in elements per part / plane
     };
     std::vector<TcSet> sets;
@@ -896,13 +908,14 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
                 T.lb_floats = std::max(1LL, std::min(T.lad_max, T.lad_cap));
                 if ((rc = tc_alloc(h, al, T.la, N3l * oo, T.kpl)) ||
                     (rc = tc_alloc(h, al, T.lap, N3l * oo, std::max(T.kplp, T.KQ))) ||
-                    (rc = tc_alloc(h, al, T.lb, T.lb_floats / T.kpl + 1, T.kpl)) ||
+                    (rc = tc_alloc(h, al, T.lb, T.lb_floats / T.kpl + 1, T.kpl, T.lb_floats / std::max(T.kplp, T.KQ) + 1)) ||
                     (rc = tc_alloc(h, al, T.ra, N3l * ov, T.kpr)) || (rc = tc_alloc(h, al, T.rb, N3l * 2 * ov, T.kpr)) ||
                     (rc = tc_alloc(h, al, T.b1, N3l * 2 * ov, T.kpr)) ||
                     (rc = tc_alloc(h, al, T.ha, N3l * oo, T.kpl)) || (rc = tc_alloc(h, al, T.hb, N3l * 2 * oo, T.kpl)) ||
                     (rc = tc_alloc(h, al, T.h2a, N3l * oo, T.kpo)) || (rc = tc_alloc(h, al, T.h2b, N3l * 2 * vv, T.kpo)))
                     return rc;
                 T.lb_floats = T.lb.rows * T.kpl;
+                T.lb_sc_rows = T.lb.sc_rows;
             }
         } else {
             // Large problems: every tensor-core step embeds its operands into one of two pools
@@ -928,7 +941,9 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
                 float* scB = nullptr;
                 if (T.oz) {   // row scales of the largest A-side and B-side operands
                     const long long ra = N3l * std::max(oo, ov);
-                    const long long rb = std::max({N3l * 2 * ov, N3l * 2 * oo, N3l * 2 * vv, pb / T.kpl + 1});
+                    const long long rb = std::max({N3l * 2 * ov, N3l * 2 * oo, N3l * 2 * vv,
+                                                   pb / std::max(T.kplp, T.KQ) + 1});
+                    T.lb_sc_rows = rb;
                     scA = (float*)al.get((size_t)ra * 4);
                     scB = (float*)al.get((size_t)rb * 4);
                     if (al.err) return al.err;
@@ -936,20 +951,20 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
                 }
                 T.lb_floats = pb;
                 const bool zo = T.oz;
-                auto view = [zo](float* base, float* sc, long long floats, long long rows, int kpad) {
+                auto view = [&](float* base, float* sc, long long scr, long long floats, long long rows, int kpad) {
                     if (zo) {
-                        TcBuf t{nullptr, nullptr, rows, kpad, (uint16_t*)base, sc};
+                        TcBuf t{nullptr, nullptr, rows, kpad, (uint16_t*)base, sc, scr};
                         return t;
                     }
                     TcBuf t{base, base + floats, rows, kpad};
                     return t;
                 };
-                T.la = view(pool_a, scA, pa, N3l * oo, T.kpl); T.lap = view(pool_a, scA, pa, N3l * oo, std::max(T.kplp, T.KQ));
-                T.ra = view(pool_a, scA, pa, N3l * ov, T.kpr); T.ha = view(pool_a, scA, pa, N3l * oo, T.kpl);
-                T.h2a = view(pool_a, scA, pa, N3l * oo, T.kpo);
-                T.rb = view(pool_b, scB, pb, N3l * 2 * ov, T.kpr); T.b1 = view(pool_b, scB, pb, N3l * 2 * ov, T.kpr);
-                T.hb = view(pool_b, scB, pb, N3l * 2 * oo, T.kpl); T.h2b = view(pool_b, scB, pb, N3l * 2 * vv, T.kpo);
-                T.lb = view(pool_b, scB, pb, pb / T.kpl, T.kpl);
+                T.la = view(pool_a, scA, pool_ar, pa, N3l * oo, T.kpl); T.lap = view(pool_a, scA, pool_ar, pa, N3l * oo, std::max(T.kplp, T.KQ));
+                T.ra = view(pool_a, scA, pool_ar, pa, N3l * ov, T.kpr); T.ha = view(pool_a, scA, pool_ar, pa, N3l * oo, T.kpl);
+                T.h2a = view(pool_a, scA, pool_ar, pa, N3l * oo, T.kpo);
+                T.rb = view(pool_b, scB, pool_br, pb, N3l * 2 * ov, T.kpr); T.b1 = view(pool_b, scB, pool_br, pb, N3l * 2 * ov, T.kpr);
+                T.hb = view(pool_b, scB, pool_br, pb, N3l * 2 * oo, T.kpl); T.h2b = view(pool_b, scB, pool_br, pb, N3l * 2 * vv, T.kpo);
+                T.lb = view(pool_b, scB, pool_br, pb, pb / T.kpl, T.kpl);
             }
             h->buf[B_WAB] = (double2*)pool_b;
         }
@@ -1458,8 +1473,11 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
                         rows += (long long)chunks[b1].size() * rows_per_block;
                         ++b1;
                     }
-                    if (rows > cap_rows) return CCSD_ERR_INVALID;
-                    TcBuf B{T.lb.big, T.lb.big + T.lb_floats, std::max(rows, 1LL), A.kpad};
+                    if (rows > cap_rows || (T.oz && rows > T.lb_sc_rows)) {
+                        refuse("the ladder's W' exceeds its operand buffer or row scales");
+                        return CCSD_ERR_INVALID;
+                    }
+                    TcBuf B{T.lb.big, T.lb.big + T.lb_floats, std::max(rows, 1LL), A.kpad, nullptr, nullptr, T.lb_sc_rows};
                     if (!pooled) B.small = T.lb.small;
                     if (T.oz) { B.big = B.small = nullptr; B.sl = T.lb.sl; B.sc = T.lb.sc; }
                     int nchmax = 0;

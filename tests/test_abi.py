@@ -131,6 +131,22 @@ def test_mixed_plan_indices_in_bounds(libpath, grid, o, v, lean):
 
 
 @pytest.mark.parametrize("lean", [0, 1])
+@pytest.mark.parametrize("grid,o,v", [((1, 1, 1), 2, 33), ((1, 1, 1), 9, 15), ((2, 1, 1), 8, 9), ((2, 1, 1), 3, 31)])
+def test_ozaki_row_scales_in_bounds(libpath, grid, o, v, lean):
+    """With one and two k points the ladder's largest W' class has e < f only: its rows are
+    half as long as the (e, f) rows the buffer is counted in, so there are twice as many
+    row scales.  ccsd_plan_check refuses a plan whose rows exceed its row scales."""
+    from paper_1911_00242_gb300 import binding
+    lib = binding.load(libpath)
+    n = ctypes.c_longlong(0)
+    tb = ctypes.c_size_t(0)
+    for more in (dict(precision=binding.CCSD_OZAKI),
+                 dict(precision=binding.CCSD_MIXED, polish_precision=binding.CCSD_OZAKI)):
+        cfg = binding.make_config(grid, o, v, lean=lean, **more)
+        assert lib.ccsd_plan_check(ctypes.byref(cfg), ctypes.byref(n), ctypes.byref(tb)) == 0, binding.load().ccsd_last_error()
+
+
+@pytest.mark.parametrize("lean", [0, 1])
 @pytest.mark.parametrize("slices", [0, 3, 8])
 @pytest.mark.parametrize("grid,o,v", [((1, 1, 1), 3, 5), ((2, 1, 1), 2, 3), ((3, 2, 1), 5, 7),
                                       ((2, 2, 2), 8, 32), ((3, 3, 3), 8, 24), ((2, 2, 1), 8, 32),
