@@ -69,12 +69,15 @@ enum Buf {
 struct GemmVar {        // launch shape of one contraction in one arithmetic
     int shape, nsplit, tiles_m, tiles_n;
     long long blocks;   // tiles x batches
+    long long work_off, cnt_off;   // this step's own split partials and tile counters (0: shared)
 };
 
 struct GemmPlan {
     int a, b, c;
     GemmArgs args;      // device tables filled; pointers, tiles and splits resolved at launch
     GemmVar var[ZG_ARITH];
+    int part = 0;       // momentum blocks of C written: 0 all, 1 those with equal pair momenta
+                        // (ka = kb or km = kn), 2 the others
 };
 
 struct CopyPlan {       // dst = (conj) src, n elements
@@ -118,6 +121,10 @@ struct TcPlan {
     OzArgs z;
     int c;
     int blocks;
+    const void* opA = nullptr;     // operand buffers read
+    const void* opB = nullptr;
+    long long work_off = 0;        // this step's own split partials in oz_work (0: shared)
+    int split_cap = 1;             // most splits at any slice count (sizes the workspace)
 };
 
 }  // namespace
@@ -188,6 +195,13 @@ struct ccsd_ctx {
     std::vector<WListPlan> wlists;
     std::vector<int> const_embeds;   // embeds of constant inputs, run once at creation
     int* tc_err = nullptr;
+    // Problems of up to kGraphElems replay the residual as a CUDA graph whose edges are the
+    // plan's data dependencies.  [0]: on the handle's amplitudes, with max|R| and the error
+    // word copied to the host; [1]: on `stage` (ccsd_residual's arguments are copied in and out).
+    bool graphable = false;
+    double2* stage = nullptr;        // [t1 | t2]
+    cudaGraphExec_t graph[2][ZG_ARITH] = {};
+    long long graph_launches[2][ZG_ARITH] = {};
     // tracing: CUDA events around every step of the residual plan
     int trace = 0;
     std::vector<cudaEvent_t> ev0, ev1;
@@ -272,6 +286,14 @@ struct GemmSpec {
 };
 
 const int kSMs = 152;
+// Largest t2 (elements, 16 bytes each) of a problem whose residual is replayed as a graph.
+// A replay saves about 2 us of host time per launch and runs independent steps side by
+// side: a chain of 4 k points (n2 = 65 k) takes 0.72 ms step by step and 0.35 ms replayed,
+// one Ozaki iteration at 2x2x1/o8/v32 (n2 = 4 M) 9.0 and 8.1 ms, with equal bits.  At
+// 2x2x2/o8/v32 (n2 = 34 M) each step fills the chip (87.9 and 87.8 ms), and ccsd_residual's
+// arguments, copied in and out, cost memory and time.
+const long long kGraphElems = 1LL << 24;
+const size_t kGraphWorkBytes = 1ull << 30;    // most split workspace for a region per step
 const int kRedBlocks = kSMs * 4;    // blocks of the reductions (max|R|, inner products, energy)
 
 // Momentum pairs (ka <= kb) whose ladder W' blocks one slab holds: as many as fit in
@@ -290,7 +312,7 @@ int finalize_gemm(ccsd_ctx* h, Alloc& al, GemmSpec s, size_t& work_need) {
         p.a = s.a; p.b = s.b; p.c = s.c;
         p.args.M = std::max(s.M, 1); p.args.N = std::max(s.N, 1); p.args.K = s.K;
         p.args.nbatch = 0; p.args.nchunk = std::max(s.nchunk, 1); p.args.nsplit = 1;
-        for (GemmVar& w : p.var) w = GemmVar{3, 1, 1, 1, 0};
+        for (GemmVar& w : p.var) w = GemmVar{3, 1, 1, 1, 0, 0, 0};
         h->gemms.push_back(p);
         h->seq.push_back({0, (int)h->gemms.size() - 1, h->cur_name, 0.0, 0.0});
         return 0;
@@ -576,6 +598,8 @@ int add_tc(ccsd_ctx* h, Alloc& al, const TcBuf& A, const TcBuf& B, int c, int M,
     }
     TcPlan t{};
     t.c = c;
+    t.opA = oz ? (const void*)A.sl : (const void*)A.big;
+    t.opB = oz ? (const void*)B.sl : (const void*)B.big;
     TcArgs& a = t.a;
     a.rowA = upload(al, rowA, h->st); a.rowB = upload(al, rowB, h->st);
     a.offC = upload(al, offC, h->st); a.colC = upload(al, colC, h->st);
@@ -607,6 +631,9 @@ int add_tc(ccsd_ctx* h, Alloc& al, const TcBuf& A, const TcBuf& B, int c, int M,
         const long long tiles = (long long)z.tiles_m * z.tiles_n * nbatch;
         const int units = nchunk * oz_nwin(z.kstages, h->oz_slices);
         z.nsplit = 1;
+        if (tiles < 2 * kSMs)
+            t.split_cap = (int)std::min<long long>(std::min<long long>((long long)nchunk * z.kstages, OZ_MAX_SPLIT),
+                                                   (2 * kSMs + tiles - 1) / tiles);
         if (tiles < 2 * kSMs) z.nsplit = (int)std::min<long long>(std::min(units, OZ_MAX_SPLIT), (2 * kSMs + tiles - 1) / tiles);
         t.blocks = (int)(tiles * z.nsplit);
         if (z.nsplit > 1)
@@ -1232,6 +1259,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
             s.rowC = tab({{(int)oo, 1}});
             for (int x : nc) { s.colC.push_back(x * (int)oo); s.colC2.push_back(swap_pair(x, o) * (int)oo); }
             if ((rc = G(s))) return rc;
+            h->gemms.back().part = diag_mn ? 1 : 2;
             if (tcp) h->seq.back().mode = 1;
         }
     }
@@ -1294,6 +1322,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
             s.rowC = tab({{(int)oo, vv}}); s.colC = nc;
             for (int x : nc) s.colC2.push_back(swap_pair(x, v));
             if ((rc = G(s))) return rc;
+            h->gemms.back().part = diag_ab ? 1 : 2;
             if (tcp) h->seq.back().mode = 1;
         }
     }
@@ -1423,6 +1452,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
                     // block for ka = kb
                     for (int x : ncols) s.colC2.push_back(swapped[x]);
                     if ((rc = G(s))) return rc;
+                    h->gemms.back().part = diag_ab ? 1 : 2;
                 }
             }
             // the tensor-core path forms W' inside its operand embedding
@@ -1848,6 +1878,7 @@ GemmArgs gemm_args(const ccsd_ctx* h, const GemmPlan& p, int arith) {
     g.A32 = (fp32 || h->in32[p.a]) ? h->shadow[p.a] : nullptr;
     g.B32 = (fp32 || h->in32[p.b]) ? h->shadow[p.b] : nullptr;
     g.tiles_m = v.tiles_m; g.tiles_n = v.tiles_n; g.nsplit = v.nsplit;
+    if (v.nsplit > 1) { g.work += v.work_off; g.cnt += v.cnt_off; }
     return g;
 }
 
@@ -1958,7 +1989,7 @@ void launch_tc(ccsd_ctx* h, TcPlan& t) {
         ensure_smem_attr(SMEM_OZ);
         OzArgs z = t.z;
         z.C = h->buf[t.c];
-        z.work = z.nsplit > 1 ? h->oz_work : nullptr;
+        z.work = z.nsplit > 1 ? h->oz_work + t.work_off : nullptr;
         oz_gemm_kernel<<<t.blocks, OZ_THREADS, OZ_SMEM_BYTES, h->st>>>(t.mA_big, t.mB_big, z);
         ++h->launches;
         if (z.work) {
@@ -2100,18 +2131,203 @@ int run_residual_async(ccsd_ctx* h) {
     return 0;
 }
 
-// A bounded wait inside a tensor-core GEMM gave up: report, clear, fail (synchronizes).
-int check_tc_err(ccsd_ctx* h) {
-    if (!((h->fp32 && h->cfg.precision == CCSD_MIXED) || h->oz_on) || !h->tc_err) return 0;
-    int flag = 0;
-    CK(cudaMemcpyAsync(&flag, h->tc_err, sizeof(int), cudaMemcpyDeviceToHost, h->st));
-    CK(cudaStreamSynchronize(h->st));
+// The handle's host words, pinned: max|R| of the last iteration and the tensor-core error
+// word, copied together.
+bool tc_active(const ccsd_ctx* h) { return ((h->fp32 && h->cfg.precision == CCSD_MIXED) || h->oz_on) && h->tc_err; }
+
+int copy_host_words(ccsd_ctx* h, bool norm) {
+    if (norm) CK(cudaMemcpyAsync(h->norm_host, h->red_out, sizeof(double), cudaMemcpyDeviceToHost, h->st));
+    if (tc_active(h)) CK(cudaMemcpyAsync(h->norm_host + 1, h->tc_err, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+    return 0;
+}
+
+// max|R| of h->res into red_out.
+void launch_norm(ccsd_ctx* h) {
+    maxabs_partial<<<h->red_blocks, 256, 0, h->st>>>(MaxabsOp{h->res, h->n1 + h->n2, h->red});
+    final_max<<<1, 32, 0, h->st>>>(h->red, h->red_blocks, h->red_out);
+    h->launches += 2;
+}
+
+// What a plan step reads and writes, as base addresses (buffers that share memory, like
+// the pooled operands, share the address).  R2 and W~_mnij count as two buffers each, the
+// blocks with equal pair momenta and the others: the packed contractions into the two run
+// side by side.
+struct StepAccess { std::vector<const void*> rd, wr; };
+
+StepAccess step_access(const ccsd_ctx* h, const Step& st) {
+    StepAccess a;
+    auto add = [&](std::vector<const void*>& v, int id, int part) {
+        const char* p = (const char*)h->buf[id];
+        if (!p) return;
+        const bool halves = id == B_R2 || id == B_WHH;
+        if (!halves || part != 2) v.push_back(p);
+        if (halves && part != 1) v.push_back(p + 1);
+    };
+    auto rd = [&](int id) { add(a.rd, id, 0); if (h->shadow[id]) a.rd.push_back(h->shadow[id]); };
+    auto wr = [&](int id, int part = 0) { add(a.wr, id, part); };
+    switch (st.kind) {
+        case 0: { const GemmPlan& p = h->gemms[st.idx]; rd(p.a); rd(p.b); wr(p.c, p.part); break; }
+        case 1: rd(h->copies[st.idx].src); wr(h->copies[st.idx].dst); break;
+        case 2: rd(h->perms[st.idx].src); wr(h->perms[st.idx].dst); break;
+        case 3:
+            add(a.rd, B_T1, 0); add(a.rd, B_T2, 0); wr(B_TAU); wr(B_TAUT);
+            if (h->shadow[B_T2]) { a.wr.push_back(h->shadow[B_T2]); a.wr.push_back(h->shadow[B_TAUT]); }
+            break;
+        case 4: rd(B_ZR); wr(B_R2); break;
+        case 5: {
+            const EmbedPlan& e = h->embeds[st.idx];
+            rd(e.src);
+            a.wr.push_back(e.oz ? (const void*)e.z.sl : (const void*)e.a.big);
+            break;
+        }
+        case 6: { const TcPlan& t = h->tcs[st.idx]; a.rd.push_back(t.opA); a.rd.push_back(t.opB); wr(t.c); break; }
+        case 7: wr(st.idx); break;
+        case 9: case 12: add(a.rd, st.idx, 0); a.wr.push_back(h->shadow[st.idx]); break;
+        case 10: {
+            const WListPlan& w = h->wlists[st.idx];
+            rd(B_VVVV); rd(B_OVVV); rd(B_T1);
+            a.wr.push_back(w.oz ? (const void*)w.z.sl : (const void*)w.a.big);
+            break;
+        }
+        case 11: rd(B_T2); rd(B_T1); rd(B_FVVP); rd(B_FOOP); rd(B_OOOV); rd(B_OVVV); wr(B_ZR); break;
+        case 13:
+            for (const void* p : {(const void*)h->t2_df, (const void*)h->t1_df, (const void*)h->fvvpT_df,
+                                  (const void*)h->foop_df}) a.rd.push_back(p);
+            rd(B_OOOV); rd(B_OVVV); wr(B_ZR);
+            break;
+        case 14:
+            rd(B_T2); rd(B_T1); rd(B_FVVP); rd(B_FOOP);
+            for (const void* p : {(const void*)h->t2_df, (const void*)h->t1_df, (const void*)h->fvvpT_df,
+                                  (const void*)h->foop_df}) a.wr.push_back(p);
+            break;
+    }
+    return a;
+}
+
+// Order of the active steps: for each, the earlier steps it must follow (read after
+// write, write after read, write after write).  An accumulation is a write, so the sums
+// into one buffer keep their order and the results do not depend on the replay.
+struct HazardMap {
+    struct Last { int writer = -1; std::vector<int> readers; };
+    std::map<const void*, Last> last;
+    std::vector<int> add(int i, const StepAccess& a) {
+        std::set<int> pre;
+        for (const void* p : a.rd) if (last[p].writer >= 0) pre.insert(last[p].writer);
+        for (const void* p : a.wr) {
+            Last& l = last[p];
+            if (l.writer >= 0) pre.insert(l.writer);
+            pre.insert(l.readers.begin(), l.readers.end());
+        }
+        for (const void* p : a.rd) last[p].readers.push_back(i);
+        for (const void* p : a.wr) { last[p].writer = i; last[p].readers.clear(); }
+        pre.erase(i);
+        return std::vector<int>(pre.begin(), pre.end());
+    }
+};
+
+// Captures the residual (and, norm set, max|R| and the host copies) into a graph.
+int build_graph(ccsd_ctx* h, bool norm, cudaGraphExec_t* out, long long* launches) {
+    cudaGraph_t g = nullptr;
+    cudaStream_t cs = nullptr;
+    if (cudaGraphCreate(&g, 0) != cudaSuccess) { last_err(cudaGetLastError()); return CCSD_ERR_CUDA; }
+    if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
+        last_err(cudaGetLastError());
+        cudaGraphDestroy(g);
+        return CCSD_ERR_CUDA;
+    }
+    const cudaStream_t own = h->st;
+    const long long before = h->launches;
+    h->st = cs;
+    cudaError_t err = cudaSuccess;
+    // one captured piece: launches of `fn` after the nodes `pre`; returns its last nodes
+    auto piece = [&](const std::vector<cudaGraphNode_t>& pre, const std::function<void()>& fn) {
+        std::vector<cudaGraphNode_t> ends;
+        if (err != cudaSuccess) return ends;
+        err = cudaStreamBeginCaptureToGraph(cs, g, pre.data(), nullptr, pre.size(), cudaStreamCaptureModeThreadLocal);
+        if (err != cudaSuccess) return ends;
+        fn();
+        cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+        const cudaGraphNode_t* nodes = nullptr;
+        size_t n = 0;
+        err = cudaStreamGetCaptureInfo(cs, &status, nullptr, nullptr, &nodes, nullptr, &n);
+        if (err == cudaSuccess) ends.assign(nodes, nodes + n);
+        cudaGraph_t same = nullptr;
+        const cudaError_t e2 = cudaStreamEndCapture(cs, &same);
+        if (err == cudaSuccess) err = e2;
+        return ends;
+    };
+    HazardMap hz;
+    std::vector<std::vector<cudaGraphNode_t>> ends(h->seq.size());
+    auto after = [&](const std::vector<int>& steps) {
+        std::set<cudaGraphNode_t> pre;
+        for (int i : steps) pre.insert(ends[(size_t)i].begin(), ends[(size_t)i].end());
+        return std::vector<cudaGraphNode_t>(pre.begin(), pre.end());
+    };
+    for (size_t si = 0; si < h->seq.size() && err == cudaSuccess; ++si) {
+        if (!step_active(h, h->seq[si])) continue;
+        ends[si] = piece(after(hz.add((int)si, step_access(h, h->seq[si]))), [&]() { launch_step(h, si); });
+    }
+    if (norm && err == cudaSuccess) {
+        std::vector<int> all;                 // every step: the error word is any of theirs
+        for (size_t si = 0; si < h->seq.size(); ++si) if (!ends[si].empty()) all.push_back((int)si);
+        StepAccess r;
+        for (int id : {B_R1, B_R2}) { r.rd.push_back(h->buf[id]); r.rd.push_back((const char*)h->buf[id] + 1); }
+        int rc = 0;
+        const std::vector<cudaGraphNode_t> nodes = piece(after(hz.add((int)h->seq.size(), r)), [&]() { launch_norm(h); });
+        std::vector<cudaGraphNode_t> pre = after(all);
+        pre.insert(pre.end(), nodes.begin(), nodes.end());
+        piece(pre, [&]() { rc = copy_host_words(h, true); });
+        if (rc && err == cudaSuccess) err = cudaErrorUnknown;
+    }
+    h->st = own;
+    *launches = h->launches - before;
+    h->launches = before;
+    if (err == cudaSuccess) err = cudaGetLastError();
+    if (err == cudaSuccess) err = cudaGraphInstantiate(out, g, 0);
+    cudaGraphDestroy(g);
+    cudaStreamDestroy(cs);
+    if (err != cudaSuccess) { cudaGetLastError(); last_err(err); *out = nullptr; return CCSD_ERR_CUDA; }
+    return 0;
+}
+
+// True if this call replays the graph: problems up to its size, except while tracing and while the
+// caller captures the handle's stream (the launches then become part of that capture).
+bool use_graph(const ccsd_ctx* h) {
+    if (!h->graphable || h->trace) return false;
+    if (!h->st) return true;
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->st, &s) != cudaSuccess) { cudaGetLastError(); return false; }
+    return s == cudaStreamCaptureStatusNone;
+}
+
+int replay_graph(ccsd_ctx* h, int which) {
+    const int w = gemm_arith(h);
+    if (!h->graph[which][w]) {
+        const int rc = build_graph(h, which == 0, &h->graph[which][w], &h->graph_launches[which][w]);
+        if (rc) return rc;
+    }
+    CK(cudaGraphLaunch(h->graph[which][w], h->st));
+    h->launches += h->graph_launches[which][w];
+    return 0;
+}
+
+// A bounded wait inside a tensor-core GEMM gave up (flag: the error word): report, clear, fail.
+int report_tc_err(ccsd_ctx* h, int flag) {
     if (flag) {
         snprintf(g_errbuf, sizeof g_errbuf, "tensor-core GEMM wait timed out (code %d)", flag);
         CK(cudaMemsetAsync(h->tc_err, 0, sizeof(int), h->st));
         return CCSD_ERR_TIMEOUT;
     }
     return 0;
+}
+
+// Reads the error word of the last residual (synchronizes, if tensor cores ran).
+int check_tc_err(ccsd_ctx* h) {
+    if (!tc_active(h)) return 0;
+    const int rc = copy_host_words(h, false);
+    if (rc) return rc;
+    CK(cudaStreamSynchronize(h->st));
+    return report_tc_err(h, *(const int*)(h->norm_host + 1));
 }
 
 int run_residual(ccsd_ctx* h) {
@@ -2332,6 +2548,7 @@ int group_gemm_descriptors(Group& G, BatchGroup& bg, size_t si, int cfg, cudaStr
             }
         }
         GemmArgs a = gemm_args(h, p, arith);
+        if (!own_split) { a.work = h->work; a.cnt = h->cnt; }   // the group's steps run one after another
         a.tiles_m = tm; a.tiles_n = tn; a.nsplit = ns;
         prefix.push_back(tot);
         tot += (long long)tm * tn * a.nbatch * a.nsplit;
@@ -2904,6 +3121,44 @@ int setup_handle(ccsd_ctx* h, Alloc& al, const void* const* ins, const bool* on_
     size_t work_need = 0;
     int rc = build_plan(h, al, work_need);
     if (rc) return rc;
+    if (h->n2 <= kGraphElems) {
+        // the steps of a graph run side by side: they have their own split partials and counters (one
+        // arithmetic is active at a time, so the arithmetics share the space)
+        size_t work = 0, cnt = 0, ozw = 0;
+        auto lay_out = [&](bool assign) {
+            for (int w = 0; w < ZG_ARITH; ++w) {
+                size_t wk = 0, ct = 0;
+                for (GemmPlan& p : h->gemms) {
+                    GemmVar& v = p.var[w];
+                    if (v.nsplit < 2) continue;
+                    if (assign) { v.work_off = (long long)wk; v.cnt_off = (long long)ct; }
+                    wk += (size_t)v.nsplit * p.args.nbatch * p.args.M * p.args.N;
+                    ct += (size_t)v.blocks;
+                }
+                work = std::max(work, wk);
+                cnt = std::max(cnt, ct);
+            }
+            size_t oz = 0;
+            for (TcPlan& t : h->tcs) {
+                if (!t.oz || t.split_cap < 2) continue;
+                if (assign) t.work_off = (long long)oz;
+                oz += (size_t)t.split_cap * t.z.nbatch * t.z.M * (t.z.Nr / 2);
+            }
+            ozw = std::max(ozw, oz);
+        };
+        lay_out(false);
+        if ((work + ozw) * 16 <= kGraphWorkBytes) {
+            lay_out(true);
+            h->graphable = true;
+            work_need = std::max(work_need, work);
+            h->cnt_need = std::max(h->cnt_need, cnt);
+            h->oz_work_elems = std::max(h->oz_work_elems, (long long)ozw);
+        }
+    }
+    if (h->graphable) {
+        h->stage = dalloc(h->n1 + h->n2);
+        if (!h->stage) return al.err;
+    }
     if (work_need) { h->work = dalloc((long long)work_need); if (!h->work) return al.err; }
     if (h->oz_work_elems) { h->oz_work = dalloc(h->oz_work_elems); if (!h->oz_work) return al.err; }
     h->work_elems = work_need;
@@ -2955,13 +3210,14 @@ size_t footprint_bytes(const ccsd_config* c, const bool* on_dev, int int_dtype, 
 // First half of an iteration: residual and max|R| on the device, the norm
 // copied into pinned host memory; returns without waiting.
 int iter_begin(ccsd_ctx* h) {
-    int rc = run_residual_async(h);
-    if (rc) return rc;
-    const long long n = h->n1 + h->n2;
-    maxabs_partial<<<h->red_blocks, 256, 0, h->st>>>(MaxabsOp{h->res, n, h->red});
-    final_max<<<1, 32, 0, h->st>>>(h->red, h->red_blocks, h->red_out);
-    h->launches += 2;
-    CK(cudaMemcpyAsync(h->norm_host, h->red_out, sizeof(double), cudaMemcpyDeviceToHost, h->st));
+    int rc;
+    if (use_graph(h)) {
+        if ((rc = replay_graph(h, 0))) return rc;
+    } else {
+        if ((rc = run_residual_async(h))) return rc;
+        launch_norm(h);
+        if ((rc = copy_host_words(h, true))) return rc;
+    }
     CK(cudaEventRecord(h->ev_norm, h->st));
     return 0;
 }
@@ -2982,7 +3238,7 @@ int iter_test(const ccsd_ctx* h, double mr, int* done) {
 int iter_end(ccsd_ctx* h, int* done, double* max_resid) {
     *done = 0;
     CK(cudaEventSynchronize(h->ev_norm));
-    int rc = check_tc_err(h);
+    int rc = tc_active(h) ? report_tc_err(h, *(const int*)(h->norm_host + 1)) : 0;
     if (rc) return rc;
     if (h->trace && (rc = trace_collect(h, 0, h->seq.size()))) return rc;
     const double mr = *h->norm_host;
@@ -3635,7 +3891,7 @@ int ccsd_create(const ccsd_config* cfg, const ccsd_inputs* in, void* stream, ccs
     int rc = setup_handle(h, al, ins, on_dev, in->int_dtype, in->vvvv_on_host != 0);
     if (rc) return fail(rc);
     for (int ei : h->const_embeds) launch_embed(h, h->embeds[ei]);
-    if (cudaMallocHost(&h->norm_host, sizeof(double)) != cudaSuccess) { cudaGetLastError(); h->norm_host = nullptr; return fail(CCSD_ERR_OOM); }
+    if (cudaMallocHost(&h->norm_host, 2 * sizeof(double)) != cudaSuccess) { cudaGetLastError(); h->norm_host = nullptr; return fail(CCSD_ERR_OOM); }
     if (cudaEventCreateWithFlags(&h->ev_norm, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); h->ev_norm = nullptr; return fail(CCSD_ERR_CUDA); }
     if (cudaStreamSynchronize(h->st) != cudaSuccess) return fail(CCSD_ERR_CUDA);
     *out = h;
@@ -3648,6 +3904,22 @@ int ccsd_residual(ccsd_t h, const void* t1, const void* t2, void* r1, void* r2) 
     // the kernels read and write these directly: host memory is refused, not faulted on
     if (!is_device_ptr(t1) || !is_device_ptr(t2) || !is_device_ptr(r1) || !is_device_ptr(r2)) return CCSD_ERR_INVALID;
     h->launches = 0;
+    if (use_graph(h)) {
+        // the graph reads the staged amplitudes and writes the handle's residual buffer
+        // (scratch between calls): one copy in, one out
+        const PairCopyOp in{h->stage, h->stage + h->n1, (const double2*)t1, (const double2*)t2, h->n1, h->n2};
+        const PairCopyOp back{(double2*)r1, (double2*)r2, h->res, h->res + h->n1, h->n1, h->n2};
+        op_kernel<PairCopyOp><<<ew_grid(h->n1 + h->n2), 256, 0, h->st>>>(in);
+        double2* amp[2] = {h->buf[B_T1], h->buf[B_T2]};
+        h->buf[B_T1] = h->stage; h->buf[B_T2] = h->stage + h->n1;
+        int rc = replay_graph(h, 1);
+        h->buf[B_T1] = amp[0]; h->buf[B_T2] = amp[1];
+        if (rc) return rc;
+        op_kernel<PairCopyOp><<<ew_grid(h->n1 + h->n2), 256, 0, h->st>>>(back);
+        h->launches += 2;
+        CK(cudaGetLastError());
+        return check_tc_err(h);
+    }
     double2* save[4] = {h->buf[B_T1], h->buf[B_T2], h->buf[B_R1], h->buf[B_R2]};
     h->buf[B_T1] = (double2*)t1; h->buf[B_T2] = (double2*)t2;
     h->buf[B_R1] = (double2*)r1; h->buf[B_R2] = (double2*)r2;
@@ -4119,6 +4391,7 @@ int ccsd_destroy(ccsd_t h) {
     ApiScope api_scope_;
     if (!h) return CCSD_ERR_INVALID;
     if (h->st) cudaStreamSynchronize(h->st); else cudaDeviceSynchronize();
+    for (auto& src : h->graph) for (cudaGraphExec_t g : src) if (g) cudaGraphExecDestroy(g);
     for (void* p : h->owned) cudaFree(p);
     for (cudaEvent_t e : h->ev0) cudaEventDestroy(e);
     for (cudaEvent_t e : h->ev1) cudaEventDestroy(e);

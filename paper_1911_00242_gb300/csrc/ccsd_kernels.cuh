@@ -79,6 +79,17 @@ struct CopyOp {
 };
 __global__ void copy_kernel(const CopyOp op) { op.run(blockIdx.x, gridDim.x); }
 
+// Two arrays in one pass: a1 = b1 (n1 elements), a2 = b2 (n2 elements).
+struct PairCopyOp {
+    double2* a1; double2* a2; const double2* b1; const double2* b2; long long n1, n2;
+    __device__ void run(long long vb, long long nvb) const {
+        for (long long e = vb * blockDim.x + threadIdx.x; e < n1 + n2; e += nvb * blockDim.x) {
+            if (e < n1) a1[e] = b1[e];
+            else a2[e - n1] = b2[e - n1];
+        }
+    }
+};
+
 // Batched 4-index permuted copy:
 //   dst[offD[b] + i0*d0 + i1*d1 + i2*d2 + i3*d3] = src[offS[b] + i0*s0 + i1*s1 + i2*s2 + i3*s3]
 struct Perm4 {
