@@ -340,7 +340,7 @@ const char* ccsd_last_error(void);
  *   f_ov, oovv, t1, t2   device pointers in the layout above (complex128)
  *   e_out                device pointer to 2 doubles: real, imaginary part
  *   stream               cudaStream_t the work is enqueued on (asynchronous)
- * It allocates nothing: its scratch (one partial sum per momentum block) is a
+ * It allocates nothing: its scratch (a few partial sums per momentum block) is a
  * fixed 512 KiB device array inside the library, which every GPU that loads
  * the library keeps until the process exits.  Requires N_k^3 + 1 <= 32768
  * (N_k <= 31); larger grids return CCSD_ERR_INVALID before any launch.  The

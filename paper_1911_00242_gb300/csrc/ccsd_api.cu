@@ -155,7 +155,8 @@ struct ccsd_ctx {
     double* red_out = nullptr;       // scalars
     double2* cred = nullptr;
     double2* cred_out = nullptr;
-    double* norm_host = nullptr;     // pinned: max|R| of the last iteration
+    double* norm_host = nullptr;     // pinned, two words: max|R| of the last iteration and the
+                                     // tensor-core error word, or the energy
     cudaEvent_t ev_norm = nullptr;
     std::vector<double2*> hx, he;    // DIIS history on canonical blocks: [t1 | nc blocks of t2]
     long long nc = 0;                // canonical t2 blocks (ki <= kj, ka <= kb)
@@ -1938,6 +1939,11 @@ UpdateOp update_op(const ccsd_ctx* h, const int* skip) {
                     h->N, h->o, h->v, nullptr, nullptr, skip};
 }
 
+DiisPackOp diis_pack_op(const ccsd_ctx* h, const int* skip) {
+    return DiisPackOp{h->amp, h->res, h->d_diis, h->d_cblk, h->nc, h->d_rden, h->N, h->o, h->v,
+                      h->d_cw, h->d_diis_part, h->red_blocks, skip};
+}
+
 void launch_embed(ccsd_ctx* h, EmbedPlan& e) {
     if (e.oz) {
         OzEmbedArgs z = e.z;
@@ -2763,31 +2769,21 @@ int group_build(Group& G, int fp32, const std::vector<int>& cfgs, double* d_norm
             // pack, inner products, Pulay solve, extrapolation -- the kernels and grids of
             // ccsd_iterate, so a member's iterates are those it has alone
             std::vector<DiisPackOp> pk;
-            std::vector<DiisDotOp> dt;
-            std::vector<DiisSolveOp> sv;
             std::vector<DiisComboOp> cb;
-            std::vector<long long> bp, bd, bs, bc;
+            std::vector<long long> bp, bc;
             for (int i = 0; i < n; ++i) {
                 ccsd_ctx* h = G.m[i];
                 if (!h->d_diis) { refuse("a group member has no DIIS state"); return CCSD_ERR_INVALID; }
                 const int* skip = d_skip ? d_skip + i : nullptr;
-                const long long blk = (long long)h->o * h->o * h->v * h->v;
-                pk.push_back(DiisPackOp{h->amp, h->res, h->d_diis, h->d_cblk, h->nc, h->d_rden, h->N, h->o, h->v,
-                                        skip});
-                bp.push_back(grid_blocks(ew_grid(h->n1 + h->nc * blk)));
-                dt.push_back(DiisDotOp{h->d_diis, h->n1, blk, h->nc, h->d_cw, h->d_diis_part, h->red_blocks, skip});
-                bd.push_back(h->red_blocks);
-                sv.push_back(DiisSolveOp{h->d_diis, h->d_diis_part, h->red_blocks, skip});
-                bs.push_back(1);
+                pk.push_back(diis_pack_op(h, skip));
+                bp.push_back(h->red_blocks);
                 cb.push_back(DiisComboOp{h->amp, h->d_diis, h->d_ctgt, h->nc, h->N, h->o, h->v, skip});
                 bc.push_back(std::min<long long>(cb.back().units(), 8LL * kSMs));
             }
-            GLaunch g1, g2, g3, g4;
-            if ((rc = make_grouped(G, pk, bp, st, g1)) || (rc = make_grouped(G, dt, bd, st, g2)) ||
-                (rc = make_grouped(G, sv, bs, st, g3)) || (rc = make_grouped(G, cb, bc, st, g4)))
-                return rc;
-            G.update.launches = g1.launches + g2.launches + g3.launches + g4.launches;
-            G.update.fn = [g1, g2, g3, g4](cudaStream_t s) { g1.fn(s); g2.fn(s); g3.fn(s); g4.fn(s); };
+            GLaunch g1, g2;
+            if ((rc = make_grouped(G, pk, bp, st, g1)) || (rc = make_grouped(G, cb, bc, st, g2))) return rc;
+            G.update.launches = g1.launches + g2.launches;
+            G.update.fn = [g1, g2](cudaStream_t s) { g1.fn(s); g2.fn(s); };
         }
     }
     CK(cudaStreamSynchronize(st));
@@ -3261,18 +3257,12 @@ int iter_finish(ccsd_ctx* h, double mr, int* done) {
         ++h->launches;
         if (h->trace) { cudaEventRecord(h->ev1[tu], h->st); if ((rc = trace_collect(h, tu, tu + 1))) return rc; }
     } else {
-        // DIIS on the device: pack x = t + R/D and e = R/D into the history, inner products
-        // of e with the filled slots, the Pulay solve, the extrapolation (no host round trip)
-        const long long blk = (long long)h->o * h->o * h->v * h->v;
-        const long long np = h->n1 + h->nc * blk;
-        op_kernel<DiisPackOp><<<ew_grid(np), 256, 0, h->st>>>(DiisPackOp{h->amp, h->res, h->d_diis, h->d_cblk, h->nc,
-                                                                          h->d_rden, h->N, h->o, h->v, nullptr});
-        op_kernel<DiisDotOp><<<(unsigned)h->red_blocks, 256, 0, h->st>>>(
-            DiisDotOp{h->d_diis, h->n1, blk, h->nc, h->d_cw, h->d_diis_part, h->red_blocks, nullptr});
-        op_kernel<DiisSolveOp><<<1, 32, 0, h->st>>>(DiisSolveOp{h->d_diis, h->d_diis_part, h->red_blocks, nullptr});
+        // DIIS on the device: one pass packs x = t + R/D and e = R/D into the history, forms the
+        // inner products and solves the Pulay system; a second extrapolates (no host round trip)
+        op_kernel<DiisPackOp><<<(unsigned)h->red_blocks, 256, 0, h->st>>>(diis_pack_op(h, nullptr));
         const DiisComboOp cb{h->amp, h->d_diis, h->d_ctgt, h->nc, h->N, h->o, h->v, nullptr};
         op_kernel<DiisComboOp><<<(unsigned)std::min<long long>(cb.units(), 8LL * kSMs), 256, 0, h->st>>>(cb);
-        h->launches += 4;
+        h->launches += 2;
         if (h->trace) { cudaEventRecord(h->ev1[tu], h->st); if ((rc = trace_collect(h, tu, tu + 1))) return rc; }
     }
     cudaError_t ce = cudaGetLastError();
@@ -4018,11 +4008,10 @@ int ccsd_energy(ccsd_t h, double* e_real, double* e_imag) {
         energy_partial<<<h->red_blocks, 256, 0, h->st>>>(h->buf[B_T1], h->buf[B_T2], h->buf[B_FOV_IN], h->buf[B_OOVV],
                                                          h->N, h->o, h->v, h->cred);
     final_csum<<<1, 32, 0, h->st>>>(h->cred, h->red_blocks, h->cred_out);
-    double2 e;
-    CK(cudaMemcpyAsync(&e, h->cred_out, sizeof(double2), cudaMemcpyDeviceToHost, h->st));
+    CK(cudaMemcpyAsync(h->norm_host, h->cred_out, sizeof(double2), cudaMemcpyDeviceToHost, h->st));   // pinned
     CK(cudaStreamSynchronize(h->st));
-    if (e_real) *e_real = e.x / h->N;
-    if (e_imag) *e_imag = e.y / h->N;
+    if (e_real) *e_real = h->norm_host[0] / h->N;
+    if (e_imag) *e_imag = h->norm_host[1] / h->N;
     return CCSD_OK;
 }
 

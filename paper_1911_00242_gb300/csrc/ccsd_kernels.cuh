@@ -150,40 +150,47 @@ struct AntisymOp {
 __global__ void antisym_kernel(const AntisymOp op) { op.run(blockIdx.x, gridDim.x); }
 
 // Block-wise max |R| partials over an array (grid-stride; fixed per-thread order).
-// part[vb] = max over this block's elements (blocks of 256 threads).
+// part[vb] = max over this block's elements (blocks of 256 threads).  The square root is
+// taken once, of the largest square (it is monotone, so the result is the same): one per
+// element is some 20 operations on the FP64 pipe, 1.3 ms for the 34 M elements of
+// 2x2x2/o8/v32, where the read takes 0.08 ms.
 struct MaxabsOp {
     const double2* x; long long n; double* part;
     __device__ void run(long long vb, long long nvb) const {
-        __shared__ double sm[256];
+        __shared__ double sm[8];
         double m = 0.0;
         for (long long e = vb * blockDim.x + threadIdx.x; e < n; e += nvb * blockDim.x) {
             const double2 z = x[e];
-            const double a = sqrt(z.x * z.x + z.y * z.y);
+            const double a = z.x * z.x + z.y * z.y;
             m = (a > m || a != a) ? a : m;     // NaN propagates
         }
-        sm[threadIdx.x] = m;
+        m = warp_max(sqrt(m));
+        if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
         __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if (threadIdx.x < s) {
-                const double o2 = sm[threadIdx.x + s];
-                if (o2 > sm[threadIdx.x] || o2 != o2) sm[threadIdx.x] = o2;
-            }
-            __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) { const double o2 = sm[w]; m = (o2 > m || o2 != o2) ? o2 : m; }
+            part[vb] = m;
         }
-        if (threadIdx.x == 0) part[vb] = sm[0];
+    }
+    __device__ static double warp_max(double m) {
+        for (int off = 16; off > 0; off >>= 1) {
+            const double o2 = __shfl_xor_sync(0xffffffffu, m, off);
+            m = (o2 > m || o2 != o2) ? o2 : m;
+        }
+        return m;
     }
 };
 __global__ void maxabs_partial(const MaxabsOp op) { op.run(blockIdx.x, gridDim.x); }
 
-// *out = max of n partials, in a fixed order (one thread of one block).
+// *out = max of n partials (one warp).
 struct FinalMaxOp {
     const double* part; int n; double* out;
     __device__ void run(long long vb, long long) const {
-        if (threadIdx.x == 0 && vb == 0) {
-            double m = 0.0;
-            for (int i = 0; i < n; ++i) { const double x = part[i]; if (x > m || x != x) m = x; }
-            *out = m;
-        }
+        if (threadIdx.x >= 32 || vb != 0) return;
+        double m = 0.0;
+        for (int i = threadIdx.x; i < n; i += 32) { const double x = part[i]; m = (x > m || x != x) ? x : m; }
+        m = MaxabsOp::warp_max(m);
+        if (threadIdx.x == 0) *out = m;
     }
 };
 
@@ -237,61 +244,100 @@ __global__ void update_kernel(const UpdateOp op) { op.run(blockIdx.x, gridDim.x)
 
 // Energy partial sums: sum f_ia t_i^a + 1/4 sum <ij||ab> t_ij^ab
 //                    + 1/2 sum_{ki,kj} <i ki j kj||a ki b kj> t_i^a t_j^b.
+// A unit is 2048 elements of one momentum block (8 per thread, loaded together); the
+// element index is decoded only in the blocks with ka = ki, which have the t1 term.  The
+// sum of <ij||ab> t_ij^ab is four FMAs per element, so the FP64 pipe (2 per clock and SM)
+// bounds it: at 2x2x2/o8/v32 0.21 ms, and 0.16 ms to read the 1.07 GB; ccsd_energy takes
+// 0.34 ms (0.68 ms with a pass that scaled t2, formed the product and decoded every element,
+// and one thread adding the blocks' sums).
+constexpr int kEnergyUnit = 2048;
 template <typename TS>
-__global__ void energy_partial(const double2* __restrict__ t1, const double2* __restrict__ t2,
-                               const double2* __restrict__ fov, const TS* __restrict__ oovv,
-                               int N, int o, int v, double2* __restrict__ part)
+__global__ void __launch_bounds__(256) energy_partial(
+    const double2* __restrict__ t1, const double2* __restrict__ t2, const double2* __restrict__ fov,
+    const TS* __restrict__ oovv, int N, int o, int v, double2* __restrict__ part)
 {
-    __shared__ double sr[256], si[256];
+    __shared__ double2 sm[8];
     const long long n1 = (long long)N * o * v;
     const long long blk = (long long)o * o * v * v;
-    const long long n2 = (long long)N * N * N * blk;
-    double er = 0.0, ei = 0.0;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n1 + n2;
-         e += (long long)gridDim.x * blockDim.x) {
-        if (e < n1) {
-            const double2 p = cmul(fov[e], t1[e]);
-            er += p.x; ei += p.y;
-        } else {
-            const long long f = e - n1;
-            const double2 g = ldz(oovv + f);
-            double2 amp = t2[f];
-            amp.x *= 0.25; amp.y *= 0.25;
-            const long long kk = f / blk;
-            const int ka = (int)(kk % N), kj = (int)((kk / N) % N), ki = (int)(kk / ((long long)N * N));
-            if (ka == ki) {
-                int r = (int)(f % blk);
-                const int b = r % v; r /= v;
-                const int a = r % v; r /= v;
-                const int j = r % o; const int i = r / o;
-                const double2 q = cmul(t1[((long long)ki * o + i) * v + a], t1[((long long)kj * o + j) * v + b]);
-                amp.x += 0.5 * q.x; amp.y += 0.5 * q.y;
+    const long long nseg = (blk + kEnergyUnit - 1) / kEnergyUnit;
+    double d0[2] = {}, d1[2] = {}, d2[2] = {}, d3[2] = {};   // sum <ij||ab> (t_ij^ab + [t1 term])
+    double sr = 0.0, si = 0.0;              // the f_ia t_i^a term
+    for (long long u = blockIdx.x; u < nseg * N * N * N; u += gridDim.x) {
+        const long long kk = u / nseg;
+        const long long e0 = (u - kk * nseg) * kEnergyUnit, base = kk * blk;
+        const int ka = (int)(kk % N), kj = (int)((kk / N) % N), ki = (int)(kk / ((long long)N * N));
+        double2 g[kEnergyUnit / 256], t[kEnergyUnit / 256];
+#pragma unroll
+        for (int q = 0; q < kEnergyUnit / 256; ++q) {
+            const long long e = e0 + q * 256 + threadIdx.x;
+            g[q] = t[q] = make_double2(0.0, 0.0);
+            if (e < blk) { g[q] = ldz(oovv + base + e); t[q] = t2[base + e]; }
+        }
+        if (ka == ki) {
+            // t + 2 t_i^a t_j^b in place of t
+#pragma unroll
+            for (int q = 0; q < kEnergyUnit / 256; ++q) {
+                const long long e = e0 + q * 256 + threadIdx.x;
+                if (e >= blk) break;
+                int a, bb, i, j;
+                if (blk < (1LL << 31)) {
+                    unsigned r = (unsigned)e;
+                    bb = (int)(r % (unsigned)v); r /= (unsigned)v;
+                    a = (int)(r % (unsigned)v); r /= (unsigned)v;
+                    j = (int)(r % (unsigned)o); i = (int)(r / (unsigned)o);
+                } else {
+                    long long r = e;
+                    bb = (int)(r % v); r /= v;
+                    a = (int)(r % v); r /= v;
+                    j = (int)(r % o); i = (int)(r / o);
+                }
+                double2 x = t1[((long long)ki * o + i) * v + a];
+                const double2 y = t1[((long long)kj * o + j) * v + bb];
+                x.x += x.x; x.y += x.y;
+                t[q].x = fma(x.x, y.x, t[q].x); t[q].x = fma(-x.y, y.y, t[q].x);
+                t[q].y = fma(x.x, y.y, t[q].y); t[q].y = fma(x.y, y.x, t[q].y);
             }
-            const double2 p = cmul(g, amp);
-            er += p.x; ei += p.y;
+        }
+#pragma unroll
+        for (int q = 0; q < kEnergyUnit / 256; ++q) {
+            const int h = q & 1;
+            d0[h] = fma(g[q].x, t[q].x, d0[h]); d1[h] = fma(g[q].y, t[q].y, d1[h]);
+            d2[h] = fma(g[q].x, t[q].y, d2[h]); d3[h] = fma(g[q].y, t[q].x, d3[h]);
         }
     }
-    sr[threadIdx.x] = er; si[threadIdx.x] = ei;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) { sr[threadIdx.x] += sr[threadIdx.x + s]; si[threadIdx.x] += si[threadIdx.x + s]; }
-        __syncthreads();
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n1; e += (long long)gridDim.x * blockDim.x) {
+        const double2 p = cmul(fov[e], t1[e]);
+        sr += p.x; si += p.y;
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = make_double2(sr[0], si[0]);
+    double er = fma(0.25, (d0[0] - d1[0]) + (d0[1] - d1[1]), sr);
+    double ei = fma(0.25, (d2[0] + d3[0]) + (d2[1] + d3[1]), si);
+    for (int off = 16; off > 0; off >>= 1) {
+        er += __shfl_down_sync(0xffffffffu, er, off);
+        ei += __shfl_down_sync(0xffffffffu, ei, off);
+    }
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = make_double2(er, ei);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) { er += sm[w].x; ei += sm[w].y; }
+        part[blockIdx.x] = make_double2(er, ei);
+    }
 }
 
-// Fixed-order final reductions (one block).
+// Fixed-order final reductions (one warp).
 __global__ void final_max(const double* __restrict__ part, int n, double* __restrict__ out)
 {
     FinalMaxOp{part, n, out}.run(blockIdx.x, gridDim.x);
 }
 __global__ void final_csum(const double2* __restrict__ part, int n, double2* __restrict__ out)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double r = 0.0, i2 = 0.0;
-        for (int i = 0; i < n; ++i) { r += part[i].x; i2 += part[i].y; }
-        *out = make_double2(r, i2);
+    if (threadIdx.x >= 32 || blockIdx.x != 0) return;
+    double r = 0.0, i2 = 0.0;
+    for (int i = threadIdx.x; i < n; i += 32) { r += part[i].x; i2 += part[i].y; }
+    for (int off = 16; off > 0; off >>= 1) {
+        r += __shfl_down_sync(0xffffffffu, r, off);
+        i2 += __shfl_down_sync(0xffffffffu, i2, off);
     }
+    if (threadIdx.x == 0) *out = make_double2(r, i2);
 }
 
 // ---------------------------------------------------------------------------
@@ -485,6 +531,7 @@ struct DiisState {
     double gram[DIIS_MAX][DIIS_MAX];
     double coef[DIIS_MAX];
     int depth, next, count, m;
+    int arrived;              // blocks of the packing pass that are done (zero between updates)
     int singular;             // a solve met a zero pivot (that iteration took the plain update)
 };
 
@@ -522,110 +569,89 @@ struct DiisRdenOp {
     }
 };
 
-// pack into slot ds->next, skipped for converged members: x = t + R / D, e = R / D on
-// the canonical elements (R and t read at their full-array positions)
+// One pass of an update, skipped for converged members: x = t + R / D and e = R / D on the
+// canonical elements into slot ds->next (R and t read at their full-array positions), the
+// weighted Re <e | e_j> with every filled slot j while e is in registers, and in the block
+// that finishes last the Gram row, the Pulay solve and the ring advance.  part[j * nred + r]
+// is block r's partial sum for slot j (nred blocks of 256 threads).
 struct DiisPackOp {
     const double2* amp; const double2* res; DiisState* ds;
     const int* cblk; long long nc; const double* rden; int N, o, v;
-    const int* skip;
-    __device__ void run(long long vb, long long nvb) const {
-        if (skip && *skip) return;
-        const int slot = ds->next;
-        double2* x_out = ds->hx[slot];
-        double2* e_out = ds->he[slot];
-        const long long n1 = (long long)N * o * v;
-        const long long blk = (long long)o * o * v * v;
-        const long long total = n1 + nc * blk;
-        for (long long e = vb * blockDim.x + threadIdx.x; e < total; e += nvb * blockDim.x) {
-            long long q = e;
-            if (e >= n1) {
-                const long long pe = e - n1;
-                q = n1 + (long long)cblk[pe / blk] * blk + pe % blk;
-            }
-            const double rd = rden[e];
-            const double2 rq = res[q];
-            const double2 step = make_double2(rq.x * rd, rq.y * rd);
-            const double2 t = amp[q];
-            x_out[e] = make_double2(t.x + step.x, t.y + step.y);
-            e_out[e] = step;
-        }
-    }
-};
-
-// Partial sums of w-weighted Re <e_next | e_j> for every slot j of the history
-// (j >= the filled slots: zero).  Block r of nred takes the elements r * 256 + t
-// (stride nred * 256) and forms all the slots' sums in one pass, so e_next is read
-// once; part[j * nred + r] receives slot j's sum, each reduced over the block in the
-// same fixed tree.
-struct DiisDotOp {
-    const DiisState* ds; long long n1, blk, nc; const double* cw;
-    double* part; int nred;
+    const double* cw; double* part; int nred;
     const int* skip;
     __device__ void run(long long vb, long long) const {
         if (skip && *skip) return;
-        __shared__ double sm[256];
-        const int r = (int)vb;
+        __shared__ double sm[8][DIIS_MAX];
+        __shared__ double gm[DIIS_MAX];
+        __shared__ int s_last;
+        const int r = (int)vb, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        const int slot = ds->next;
         const int m = min(ds->count + 1, ds->depth);
-        const double2* x = ds->he[ds->next];
+        double2* x_out = ds->hx[slot];
+        double2* e_out = ds->he[slot];
         const double2* y[DIIS_MAX];
-#pragma unroll
-        for (int j = 0; j < DIIS_MAX; ++j) y[j] = ds->he[j];
         double s[DIIS_MAX];
 #pragma unroll
-        for (int j = 0; j < DIIS_MAX; ++j) s[j] = 0.0;
-        const long long n = n1 + nc * blk;
-        for (long long e = (long long)r * blockDim.x + threadIdx.x; e < n; e += (long long)nred * blockDim.x) {
-            const double2 a = x[e];
-            const double w = e < n1 ? 1.0 : cw[(e - n1) / blk];
+        for (int j = 0; j < DIIS_MAX; ++j) { y[j] = ds->he[j]; s[j] = 0.0; }
+        const long long n1 = (long long)N * o * v;
+        const long long blk = (long long)o * o * v * v;
+        const long long total = n1 + nc * blk;
+        for (long long e = (long long)r * blockDim.x + threadIdx.x; e < total; e += (long long)nred * blockDim.x) {
+            long long q = e;
+            double w = 1.0;
+            if (e >= n1) {
+                const long long pe = e - n1, p = pe / blk;
+                q = n1 + (long long)cblk[p] * blk + (pe - p * blk);
+                w = cw[p];
+            }
+            const double rd = rden[e];
+            const double2 rq = res[q];
+            const double2 t = amp[q];
+            const double2 step = make_double2(rq.x * rd, rq.y * rd);
+            x_out[e] = make_double2(t.x + step.x, t.y + step.y);
+            e_out[e] = step;
+            const double wx = w * step.x, wy = w * step.y;
 #pragma unroll
             for (int j = 0; j < DIIS_MAX; ++j) {
                 if (j < m) {
-                    const double2 b = y[j][e];
-                    s[j] += w * (a.x * b.x + a.y * b.y);
+                    const double2 b = j == slot ? step : y[j][e];
+                    s[j] = fma(wx, b.x, s[j]);
+                    s[j] = fma(wy, b.y, s[j]);
                 }
             }
         }
 #pragma unroll
         for (int j = 0; j < DIIS_MAX; ++j) {
-            if (j >= ds->depth) break;
-            sm[threadIdx.x] = s[j];
-            __syncthreads();
-            for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-                if (threadIdx.x < st) sm[threadIdx.x] += sm[threadIdx.x + st];
-                __syncthreads();
-            }
-            if (threadIdx.x == 0) part[j * nred + r] = sm[0];
-            __syncthreads();
-        }
-    }
-};
-
-// One thread: the Gram row of the new slot (partials summed in a fixed order), the
-// Pulay solve over the filled slots, and the ring advance.
-struct DiisSolveOp {
-    DiisState* ds; const double* part; int nred;
-    const int* skip;
-    __device__ void run(long long vb, long long) const {
-        if ((skip && *skip) || vb != 0 || threadIdx.x >= 32) return;
-        const int lane = threadIdx.x;
-        const int slot = ds->next;
-        const int m = min(ds->count + 1, ds->depth);
-        // the partials of each slot: lane l sums r = l, l + 32, ... in order, then a fixed
-        // shuffle tree over the lanes
-        double g[DIIS_MAX];
-#pragma unroll
-        for (int j = 0; j < DIIS_MAX; ++j) {
-            double d = 0.0;
             if (j < m)
-                for (int r = lane; r < nred; r += 32) d += part[j * nred + r];
+                for (int off = 16; off > 0; off >>= 1) s[j] += __shfl_down_sync(0xffffffffu, s[j], off);
+            if (lane == 0) sm[warp][j] = s[j];
+        }
+        __syncthreads();
+        if (threadIdx.x < m) {
+            double d = 0.0;
+            for (int w = 0; w < 8; ++w) d += sm[w][threadIdx.x];
+            __stcg(part + (long long)threadIdx.x * nred + r, d);
+            __threadfence();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) s_last = atomicAdd(&ds->arrived, 1) == nred - 1 ? 1 : 0;
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        // warp j: the partials of slot j, lane l summing l, l + 32, ... in order
+        if (warp < m) {
+            double d = 0.0;
+            for (int q = lane; q < nred; q += 32) d += __ldcg(part + (long long)warp * nred + q);
             for (int off = 16; off > 0; off >>= 1) d += __shfl_down_sync(0xffffffffu, d, off);
-            g[j] = d;
+            if (lane == 0) gm[warp] = d;
         }
-        if (lane != 0) return;
+        __syncthreads();
+        if (threadIdx.x != 0) return;
         for (int j = 0; j < m; ++j) {
-            ds->gram[slot][j] = g[j];
-            ds->gram[j][slot] = g[j];
+            ds->gram[slot][j] = gm[j];
+            ds->gram[j][slot] = gm[j];
         }
+        ds->arrived = 0;
         ds->count = m;
         ds->next = (slot + 1) % ds->depth;
         ds->m = m;
