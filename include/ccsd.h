@@ -140,7 +140,7 @@ int ccsd_plan_check(const ccsd_config* cfg, long long* n_launches, size_t* table
 /* The launch plan of this config, built on the host as ccsd_plan_check does: for
  * each of its *n_steps steps (at most max_steps are written; arrays may be NULL)
  * the step kind (0 FP64/FP32 GEMM, 1 copy, 2 permutation, 3 tau, 4 antisymmetrize,
- * 5 tensor-core operand embedding, 6 tensor-core GEMM, 7 zero, 9 complex64 copy,
+ * 5 tensor-core operand embedding, 6 tensor-core GEMM, 9 complex64 copy,
  * 10 W' formation, 11 fused Fock terms, 12 transposed F'vv, 13 fused double-float
  * Fock terms, 14 their double-float copies), the iterations it
  * runs in (mode 0 all; 1 without tensor cores; 2 split-TF32 tensor-core steps of

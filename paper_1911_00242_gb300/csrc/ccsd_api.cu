@@ -89,7 +89,7 @@ struct PermPlan {
 };
 
 struct Step {           // one element of the launch sequence
-    int kind;           // 0 gemm, 1 copy, 2 perm, 3 tau, 4 antisym, 5 embed, 6 tensor-core gemm, 7 zero,
+    int kind;           // 0 gemm, 1 copy, 2 perm, 3 tau, 4 antisym, 5 embed, 6 tensor-core gemm,
                         // 9 complex64 refresh of a buffer, 10 W' formation into the ladder's B operand,
                         // 11 fused Fock/t1 terms of R2 (mixed form), 12 transposed complex64 F'vv
     int idx;
@@ -371,6 +371,14 @@ int finalize_gemm(ccsd_ctx* h, Alloc& al, GemmSpec s, size_t& work_need) {
         GemmArgs& g0 = p.args;
         g0.affA = affine(s.rowA, g0.rAs) && affine(s.colA, g0.cAs) ? 1 : 0;
         g0.affB = affine(s.rowB, g0.rBs) && affine(s.colB, g0.cBs) ? 1 : 0;
+        // consecutive threads read along the index with more unit steps (K on a tie)
+        auto steps = [](const std::vector<int>& t) {
+            size_t n = 0;
+            for (size_t i = 1; i < t.size(); ++i) n += t[i] - t[i - 1] == 1 ? 1 : 0;
+            return t.size() < 2 ? 0.0 : (double)n / (double)(t.size() - 1);
+        };
+        g0.kfA = steps(s.colA) > 0.0 && steps(s.colA) >= steps(s.rowA) ? 1 : 0;
+        g0.kfB = steps(s.rowB) > 0.0 && steps(s.rowB) >= steps(s.colB) ? 1 : 0;
         g0.a0 = g0.affA ? (long long)s.rowA[0] + s.colA[0] : 0;
         g0.b0 = g0.affB ? (long long)s.rowB[0] + s.colB[0] : 0;
     }
@@ -571,7 +579,7 @@ int add_tc(ccsd_ctx* h, Alloc& al, const TcBuf& A, const TcBuf& B, int c, int M,
     // output row m of batch b starts at offC[b * M + m], or (rowC given) at offC[b] + rowC[m]
     const bool oz = h->cur_oz;
     if (A.kpad != B.kpad || A.kpad % (oz ? OZ_BK : TC_BK)) return CCSD_ERR_INVALID;
-    if (!oz && (alpha_im != 0.0 || overwrite || !rowC.empty())) return CCSD_ERR_INVALID;
+    if (!oz && (alpha_im != 0.0 || (overwrite && !offC2.empty()) || !rowC.empty())) return CCSD_ERR_INVALID;
     if (oz && ((long long)h->oz_slices * A.rows > INT_MAX || (long long)h->oz_slices * B.rows > INT_MAX)) {
         refuse("a tensor-core operand exceeds 2^31 rows (32-bit row indices)");
         return CCSD_ERR_INVALID;
@@ -614,6 +622,7 @@ int add_tc(ccsd_ctx* h, Alloc& al, const TcBuf& A, const TcBuf& B, int c, int M,
     a.M = M; a.Nr = Nr; a.nchunk = nchunk; a.kstages = A.kpad / TC_BK; a.nterms = nterms;
     a.tiles_m = (M + TC_BM - 1) / TC_BM; a.tiles_n = (Nr + TC_BN - 1) / TC_BN;
     a.alpha_re = alpha; a.alpha_im = 0.0;
+    a.overwrite = overwrite ? 1 : 0;
     t.blocks = a.tiles_m * a.tiles_n * nbatch;
     if (oz) {
         t.oz = true;
@@ -658,12 +667,6 @@ int add_tc(ccsd_ctx* h, Alloc& al, const TcBuf& A, const TcBuf& B, int c, int M,
     st.mode = tc_mode(h);
     h->seq.push_back(st);
     return 0;
-}
-
-void add_zero(ccsd_ctx* h, int buf) {
-    Step st{7, buf, h->cur_name, 0.0, 16.0 * (double)h->bufsize[buf]};
-    st.mode = tc_mode(h);
-    h->seq.push_back(st);
 }
 
 dim3 ew_grid(long long n);
@@ -1701,7 +1704,6 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
     }
     for (TcSet& T : sets) {
         h->cur_oz = T.oz;
-        add_zero(h, B_ZR);
         // B_ring[D][kn][kj]: rows (j,b), columns (n,f) of W~[kj, kn, kb], kb = kj + D
         std::vector<long long> so;
         for (int D = 0; D < N; ++D) for (int kn = 0; kn < N; ++kn) for (int kj = 0; kj < N; ++kj)
@@ -1722,7 +1724,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
         }
         for (int kj = 0; kj < N; ++kj) for (int j = 0; j < o; ++j) for (int b = 0; b < v; ++b)
             cc.push_back((int)((long long)kj * N * S2 + j * vv + b));
-        if ((rc = add_tc(h, al, T.ra, T.rb, B_ZR, (int)(N * ov), (int)(2 * N * ov), N, N, ra, rb, oc, cc, 1.0, 3)))
+        if ((rc = add_tc(h, al, T.ra, T.rb, B_ZR, (int)(N * ov), (int)(2 * N * ov), N, N, ra, rb, oc, cc, 1.0, 3, {}, {}, {}, 0.0, true)))
             return rc;
     }
     h->cur_name = "ring_t1t1";
@@ -2068,9 +2070,6 @@ void launch_step(ccsd_ctx* h, size_t si) {
                 break;
             case 5: launch_embed(h, h->embeds[s.idx]); break;
             case 6: launch_tc(h, h->tcs[s.idx]); break;
-            case 7:
-                cudaMemsetAsync(h->buf[s.idx], 0, (size_t)h->bufsize[s.idx] * 16, h->st);
-                break;
             case 10: {
                 if (h->wlists[s.idx].oz) {
                     ensure_smem_attr(SMEM_OZ_WPRIME);
@@ -2187,7 +2186,6 @@ StepAccess step_access(const ccsd_ctx* h, const Step& st) {
             break;
         }
         case 6: { const TcPlan& t = h->tcs[st.idx]; a.rd.push_back(t.opA); a.rd.push_back(t.opB); wr(t.c); break; }
-        case 7: wr(st.idx); break;
         case 9: case 12: add(a.rd, st.idx, 0); a.wr.push_back(h->shadow[st.idx]); break;
         case 10: {
             const WListPlan& w = h->wlists[st.idx];
@@ -2629,7 +2627,7 @@ int group_build(Group& G, int fp32, const std::vector<int>& cfgs, double* d_norm
                 ++gi;
                 break;
             }
-            case 1: case 2: case 3: case 4: case 7: case 9: case 11: case 12: {
+            case 1: case 2: case 3: case 4: case 9: case 11: case 12: {
                 // elementwise steps
                 std::vector<long long> blocks;
                 auto build = [&](auto make, auto count) {
@@ -2652,9 +2650,6 @@ int group_build(Group& G, int fp32, const std::vector<int>& cfgs, double* d_norm
                 else if (s0.kind == 4)
                     rc = build([&](ccsd_ctx* h) { return AntisymOp{h->buf[B_R2], h->buf[B_ZR], h->kb_of, h->N, h->o, h->v}; },
                                [&](ccsd_ctx* h) { return h->n2; });
-                else if (s0.kind == 7)
-                    rc = build([&](ccsd_ctx* h) { return ZeroOp{h->buf[h->seq[si].idx], h->bufsize[h->seq[si].idx]}; },
-                               [&](ccsd_ctx* h) { return h->bufsize[h->seq[si].idx]; });
                 else if (s0.kind == 9)
                     rc = build([&](ccsd_ctx* h) {
                                    const int bi = h->seq[si].idx;

@@ -10,6 +10,7 @@
 
 #include "dfloat.cuh"
 #include "diis.h"
+#include "tf32_split.cuh"
 
 namespace ccsdk {
 
@@ -58,8 +59,8 @@ struct TauOp {
             const double2 tt = make_double2(t.x + 0.5 * x.x, t.y + 0.5 * x.y);
             taut[e] = tt;
             if (t2_32) {
-                t2_32[e] = make_float2((float)t.x, (float)t.y);
-                taut_32[e] = make_float2((float)tt.x, (float)tt.y);
+                t2_32[e] = make_float2(f32_rn(t.x), f32_rn(t.y));
+                taut_32[e] = make_float2(f32_rn(tt.x), f32_rn(tt.y));
             }
         }
     }

@@ -32,12 +32,4 @@ __global__ void __launch_bounds__(256) grouped_op_kernel(const Op* __restrict__ 
 template <class Op>
 __global__ void __launch_bounds__(256) op_kernel(const Op op) { op.run(blockIdx.x, gridDim.x); }
 
-// Zeroes n complex elements (the batched counterpart of a memset step).
-struct ZeroOp {
-    double2* p; long long n;
-    __device__ void run(long long vb, long long nvb) const {
-        for (long long e = vb * blockDim.x + threadIdx.x; e < n; e += nvb * blockDim.x) p[e] = make_double2(0.0, 0.0);
-    }
-};
-
 }  // namespace ccsdk

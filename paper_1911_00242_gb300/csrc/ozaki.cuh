@@ -75,7 +75,10 @@ constexpr int OZ_BAR_BYTES = 512;                          // mbarriers, TMEM ad
 constexpr int OZ_REF_BYTES = OZ_ACC_WARPS * 96 * 4;       // per accumulator warp: RB, 1 / RB, chunk column factors
 constexpr int OZ_SMEM_BYTES = OZ_RING_BYTES + 1024 + OZ_BAR_BYTES + OZ_REF_BYTES;
 static_assert((4 + OZ_A_SLOTS + 2 * OZ_MAX_SLICES + 1) * 8 + 8 <= OZ_BAR_BYTES, "barrier area");
-static_assert(2 * OZ_COLS * (OZ_ACC_WARPS * 32) * 4 <= OZ_RING_BYTES, "epilogue park area");
+constexpr int OZ_PARK = OZ_COLS + 2;                       // floats per parked row
+constexpr int OZ_EPI_ROWS = 4;                             // rows of C in flight per lane in the epilogue
+static_assert(2 * OZ_PARK * (OZ_ACC_WARPS * 32) * 4 <= OZ_RING_BYTES, "epilogue park area");
+static_assert(OZ_COLS == 16, "the epilogue's lanes take 8 complex columns of 4 rows");
 
 struct OzArgs {
     const int* rowA;          // [nbatch * nchunk] row of A' (within a slice plane) where chunk c of batch b starts
@@ -436,33 +439,73 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
             }
         }
         if (ok && !*abort_flag) {
-            if (row < g.M) {
-                const long long rb0 = g.rowC ? g.offC[b] + g.rowC[row] : g.offC[b * g.M + row];
-                const long long rb2 = !g.offC2 ? 0 : g.rowC ? g.offC2[b] + g.rowC[row] : g.offC2[b * g.M + row];
+            // Every MMA has completed, so the operand ring is free: park (hi, lo) there and let a
+            // warp's lanes take 8 neighbouring complex columns of 4 rows at a time (128-byte
+            // segments of C, OZ_EPI_ROWS rows in flight; one thread per row touched 16 bytes of
+            // 32 rows at once).  hi and lo widen to FP64 by integer operations, scaled by the
+            // exponents of RA, RB and alpha: two FP64 adds per component where conversions,
+            // products and adds were eight.
+            float* park = (float*)smem + (warp - 2) * (2 * 32 * OZ_PARK);   // hi, then lo: [32 rows][16 + pad]
+            float* rowref = (float*)(smem + OZ_RING_BYTES + OZ_BAR_BYTES) + (warp - 2) * 96 + 32;
 #pragma unroll
-                for (int qq = 0; qq < OZ_COLS / 2; ++qq) {
-                    const int nr = n0 + cg * OZ_COLS + 2 * qq;
-                    if (nr >= g.Nr) continue;
-                    const double xr = ((double)hi[2 * qq] + (double)lo[2 * qq]) * ((double)RA * (double)colref[2 * qq]);
-                    const double xi = ((double)hi[2 * qq + 1] + (double)lo[2 * qq + 1]) *
-                                      ((double)RA * (double)colref[2 * qq + 1]);
-                    if (g.work) {       // partial of this split; oz_split_reduce applies alpha
-                        g.work[(((long long)split * g.nbatch + b) * g.M + row) * (g.Nr / 2) + (nr >> 1)] =
-                            make_double2(xr, xi);
-                        continue;
-                    }
-                    const double yr = g.alpha_re * xr - g.alpha_im * xi;
-                    const double yi = g.alpha_re * xi + g.alpha_im * xr;
-                    double2* pc = g.C + rb0 + g.colC[nr >> 1];
-                    double2 uu = g.overwrite ? make_double2(0.0, 0.0) : *pc;
-                    uu.x += yr; uu.y += yi;
-                    *pc = uu;
-                    if (g.offC2) {
-                        double2* p2 = g.C + rb2 + g.colC2[nr >> 1];
-                        double2 z = g.overwrite ? make_double2(0.0, 0.0) : *p2;
-                        z.x -= yr; z.y -= yi;
-                        *p2 = z;
-                    }
+            for (int i = 0; i < OZ_COLS; ++i) {
+                park[lane * OZ_PARK + i] = hi[i];
+                park[(32 + lane) * OZ_PARK + i] = lo[i];
+            }
+            rowref[lane] = RA;                        // the chunk factors are no longer read
+            __syncwarp();
+            int ea = 0;
+            const bool apow = g.alpha_im == 0.0 && pow2_exponent(fabs(g.alpha_re), ea);
+            const bool neg = g.alpha_re < 0.0;
+            const int qq = lane & 7;                  // complex column of this lane
+            const int nr = n0 + cg * OZ_COLS + 2 * qq;
+            const bool cok = nr < g.Nr;
+            const long long co = cok ? g.colC[nr >> 1] : 0, co2 = cok && g.offC2 ? g.colC2[nr >> 1] : 0;
+            const float RB = colref[2 * qq];          // rows 2n and 2n + 1 of B' hold the same elements
+            const int eb = (__float_as_int(RB) >> 23) - 127;
+            const int rows = min(32, g.M - (m0 + qr * 32));
+            const bool fold = apow && !g.work;        // alpha by its exponent
+            auto value = [&](int r) {
+                const float ra = rowref[r];
+                const float2 h = *(const float2*)(park + r * OZ_PARK + 2 * qq);
+                const float2 l = *(const float2*)(park + (32 + r) * OZ_PARK + 2 * qq);
+                // RA = 0 or RB = 0 (an all-zero row): (hi, lo) are zero
+                int e = ra > 0.f && RB > 0.f ? (__float_as_int(ra) >> 23) - 127 + eb : 0;
+                if (fold) e += ea;
+                const bool ng = fold && neg;
+                const double2 x = make_double2(f64_scaled(h.x, e, ng) + f64_scaled(l.x, e, ng),
+                                               f64_scaled(h.y, e, ng) + f64_scaled(l.y, e, ng));
+                if (fold || g.work) return x;
+                return make_double2(g.alpha_re * x.x - g.alpha_im * x.y, g.alpha_re * x.y + g.alpha_im * x.x);
+            };
+            const int mw = m0 + qr * 32;
+            auto at = [&](const long long* off, int r, long long c) {
+                return (g.rowC ? off[b] + g.rowC[mw + r] : off[b * g.M + mw + r]) + c;
+            };
+#pragma unroll 1
+            for (int r0 = lane >> 3; cok && r0 < rows; r0 += 4 * OZ_EPI_ROWS) {
+                if (g.work) {                         // partial of this split; oz_split_reduce applies alpha
+#pragma unroll
+                    for (int r = r0; r < rows && r < r0 + 4 * OZ_EPI_ROWS; r += 4)
+                        g.work[(((long long)split * g.nbatch + b) * g.M + mw + r) * (g.Nr / 2) + (nr >> 1)] = value(r);
+                    continue;
+                }
+                double2 o[OZ_EPI_ROWS], o2[OZ_EPI_ROWS];
+#pragma unroll
+                for (int j = 0; j < OZ_EPI_ROWS; ++j) {
+                    const int r = r0 + 4 * j;
+                    o[j] = o2[j] = make_double2(0.0, 0.0);
+                    if (r >= rows || g.overwrite) continue;
+                    o[j] = g.C[at(g.offC, r, co)];
+                    if (g.offC2) o2[j] = g.C[at(g.offC2, r, co2)];
+                }
+#pragma unroll
+                for (int j = 0; j < OZ_EPI_ROWS; ++j) {
+                    const int r = r0 + 4 * j;
+                    if (r >= rows) break;
+                    const double2 y = value(r);
+                    g.C[at(g.offC, r, co)] = make_double2(o[j].x + y.x, o[j].y + y.y);
+                    if (g.offC2) g.C[at(g.offC2, r, co2)] = make_double2(o2[j].x - y.x, o2[j].y - y.y);
                 }
             }
         } else if (lane == 0) {

@@ -68,6 +68,9 @@ constexpr int TC_TMEM_COLS = 2 * TC_BN;
 constexpr int TC_PROMOTE_STAGES = 3;
 constexpr int TC_ACC_WARPS = 8;                          // two per TMEM lane quarter, 128 columns each
 constexpr int TC_THREADS = 64 + 32 * TC_ACC_WARPS;       // producer warp, MMA warp, accumulator warps
+constexpr int TC_PARK = TC_BN / 2 + 2;                    // floats per parked row (8-byte aligned, odd pairs)
+constexpr int TC_EPI_ROWS = 16;                           // rows of C in flight per warp in the epilogue
+static_assert(TC_ACC_WARPS * 32 * TC_PARK * 4 <= TC_STAGES * TC_STAGE_BYTES, "the parked sums fit the stage ring");
 constexpr long long TC_SPIN_LIMIT = 1LL << 24;           // polls before a wait gives up (> 0.1 s)
 constexpr long long TC_DRAIN_LIMIT = 1LL << 20;          // polls per in-flight copy at teardown
 
@@ -88,6 +91,7 @@ struct TcArgs {
     const int* nchunk_b;      // per-batch chunk count (<= nchunk) or null
     const long long* offC2;   // antisymmetric mirror: c is also subtracted at offC2[b*M+m] + colC2[n]
     const int* colC2;
+    int overwrite;            // 1: C = alpha c instead of C += (no mirror)
     long long spin_limit;     // polls before a wait gives up (TC_SPIN_LIMIT)
     int skip_stage;           // failure-detection self-test: this stage is never loaded (-1: none)
 };
@@ -331,6 +335,14 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA_big, const 
         bool ok = true;
         for (int seg = 0; seg < nseg; ++seg) {
             const int buf = seg & 1;
+            if (seg == nseg - 3 && !g.overwrite && m0 + q * 32 + lane < g.M) {
+                // the lines of C this warp will add to, one row per lane, into L2
+                const long long m = b * g.M + m0 + q * 32 + lane;
+                for (int c = n0 / 2 + half * (TC_BN / 4), e = min(c + TC_BN / 4, g.Nr / 2); c < e; c += 8) {
+                    asm volatile("prefetch.global.L2 [%0];" :: "l"(g.C + g.offC[m] + g.colC[c]));
+                    if (g.offC2) asm volatile("prefetch.global.L2 [%0];" :: "l"(g.C + g.offC2[m] + g.colC2[c]));
+                }
+            }
             bool got = mbar_wait(smem_u32(&acc_full[buf]), (uint32_t)(seg >> 1) & 1u, abort_flag, g.spin_limit);
             got = __shfl_sync(0xffffffffu, got ? 1 : 0, 0) != 0;   // one decision per warp
             if (!got) { ok = false; break; }
@@ -355,33 +367,70 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA_big, const 
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&acc_empty[buf])) : "memory");
         }
         if (ok && !*abort_flag) {
-            // every MMA has completed (last acc_full), so the stage ring is free: park the
-            // sums there to run the epilogue as a plain loop
-            float* park = (float*)smem;                         // [TC_BN / 2][TC_ACC_WARPS * 32]
-            const int t = (warp - 2) * 32 + lane;
+            // Every MMA has completed (last acc_full), so the stage ring is free: park the sums
+            // there, row by row, and let the 32 lanes of a warp take neighbouring columns of
+            // one row: C is then read and written 512 bytes at a time, TC_EPI_ROWS rows in
+            // flight (one thread per row, one element at a time, cost two L2 latencies per
+            // element: 40 of the 55 us of a small launch).  The sums widen to FP64 by integer
+            // operations and alpha (+-1, +-1/2 in every plan) by its exponent, so the FP64 pipe
+            // (2 operations per clock and SM) does two adds per element where conversions,
+            // products and adds were ten: 21 of the 85 us of a full 128 x 256 tile.
+            float* park = (float*)smem + (warp - 2) * (32 * TC_PARK);   // [32 rows][128 + pad]
 #pragma unroll
-            for (int i = 0; i < TC_BN / 2; ++i) park[i * (TC_ACC_WARPS * 32) + t] = acc[i];
-            const int row = m0 + q * 32 + lane;
-            if (row < g.M) {
-                const long long rbase = g.offC[b * g.M + row];
-                const long long rbase2 = g.offC2 ? g.offC2[b * g.M + row] : 0;
+            for (int i = 0; i < TC_BN / 2; ++i) park[lane * TC_PARK + i] = acc[i];
+            __syncwarp();
+            int ea = 0;
+            const bool apow = g.alpha_im == 0.0 && pow2_exponent(fabs(g.alpha_re), ea);
+            const bool neg = g.alpha_re < 0.0;
+            const int nc = g.Nr / 2;                            // complex columns
+            const int n0c = n0 / 2 + half * (TC_BN / 4);
+            const int rows = min(32, g.M - (m0 + q * 32));
+            auto value = [&](int r, int c) {                    // alpha times the parked sum
+                const float2 x = *(const float2*)(park + r * TC_PARK + 2 * c);
+                if (apow) return make_double2(f64_scaled(x.x, ea, neg), f64_scaled(x.y, ea, neg));
+                const double xr = (double)x.x, xi = (double)x.y;
+                return make_double2(g.alpha_re * xr - g.alpha_im * xi, g.alpha_re * xi + g.alpha_im * xr);
+            };
+            const long long* offC = g.offC + b * g.M + m0 + q * 32;
+            const long long* offC2 = g.offC2 ? g.offC2 + b * g.M + m0 + q * 32 : nullptr;
 #pragma unroll 1
-                for (int qq = 0; qq < TC_BN / 4; ++qq) {
-                    const int nr = n0 + half * (TC_BN / 2) + 2 * qq;   // real column of the pair (re, im)
-                    if (nr >= g.Nr) break;
-                    const double xr = (double)park[(2 * qq) * (TC_ACC_WARPS * 32) + t];
-                    const double xi = (double)park[(2 * qq + 1) * (TC_ACC_WARPS * 32) + t];
-                    double2* p = g.C + rbase + g.colC[nr >> 1];
-                    const double yr = g.alpha_re * xr - g.alpha_im * xi;
-                    const double yi = g.alpha_re * xi + g.alpha_im * xr;
-                    double2 o = *p;
-                    o.x += yr; o.y += yi;
-                    *p = o;
-                    if (g.offC2) {
-                        double2* p2 = g.C + rbase2 + g.colC2[nr >> 1];
-                        double2 u = *p2;
-                        u.x -= yr; u.y -= yi;
-                        *p2 = u;
+            for (int cc = 0; cc < TC_BN / 4; cc += 32) {
+                const int col = n0c + cc + lane;
+                if (col >= nc) break;
+                double2* const C1 = g.C + g.colC[col];
+                if (g.overwrite) {
+#pragma unroll 4
+                    for (int r = 0; r < rows; ++r) C1[offC[r]] = value(r, cc + lane);
+                    continue;
+                }
+                if (!offC2) {
+#pragma unroll 1
+                    for (int r0 = 0; r0 < rows; r0 += TC_EPI_ROWS) {
+                        double2 o[TC_EPI_ROWS];
+#pragma unroll
+                        for (int j = 0; j < TC_EPI_ROWS; ++j) if (r0 + j < rows) o[j] = C1[offC[r0 + j]];
+#pragma unroll
+                        for (int j = 0; j < TC_EPI_ROWS; ++j) {
+                            if (r0 + j >= rows) break;
+                            const double2 y = value(r0 + j, cc + lane);
+                            C1[offC[r0 + j]] = make_double2(o[j].x + y.x, o[j].y + y.y);
+                        }
+                    }
+                    continue;
+                }
+                double2* const C2 = g.C + g.colC2[col];
+#pragma unroll 1
+                for (int r0 = 0; r0 < rows; r0 += TC_EPI_ROWS / 2) {
+                    double2 o[TC_EPI_ROWS / 2], o2[TC_EPI_ROWS / 2];
+#pragma unroll
+                    for (int j = 0; j < TC_EPI_ROWS / 2; ++j)
+                        if (r0 + j < rows) { o[j] = C1[offC[r0 + j]]; o2[j] = C2[offC2[r0 + j]]; }
+#pragma unroll
+                    for (int j = 0; j < TC_EPI_ROWS / 2; ++j) {
+                        if (r0 + j >= rows) break;
+                        const double2 y = value(r0 + j, cc + lane);
+                        C1[offC[r0 + j]] = make_double2(o[j].x + y.x, o[j].y + y.y);
+                        C2[offC2[r0 + j]] = make_double2(o2[j].x - y.x, o2[j].y - y.y);
                     }
                 }
             }

@@ -74,6 +74,32 @@ __host__ __device__ __forceinline__ void split_tf32(double x, float& big, float&
     small = tf32_round((float)(x - (double)big));
 }
 
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ double f64_of_bits(uint64_t u) { return __longlong_as_double((long long)u); }
+#else
+inline double f64_of_bits(uint64_t u) { double x; memcpy(&x, &u, sizeof x); return x; }
+#endif
+
+// x 2^e (negated if neg) as a double, exactly, from the bit pattern with integer operations
+// (a conversion and a scaling would be two operations on GB300's FP64 pipe).  |e| <= 800;
+// zeros, subnormals, infinities and NaN take the FP64 path.
+__host__ __device__ __forceinline__ double f64_scaled(float x, int e = 0, bool neg = false) {
+    const uint32_t u = tf32_bits_of(x) ^ (neg ? 0x80000000u : 0u);
+    const uint32_t ex = (u >> 23) & 0xffu;
+    if (ex - 1u < 254u) {
+        const uint32_t hi = (u & 0x80000000u) | ((ex + (uint32_t)(896 + e)) << 20) | ((u & 0x7fffffu) >> 3);
+        return f64_of_bits(((uint64_t)hi << 32) | (uint64_t)(u << 29));
+    }
+    return (double)tf32_float_of(u) * f64_of_bits((uint64_t)(1023 + e) << 52);
+}
+
+// The exponent of a power of two p > 0 with |exponent| <= 200; false for any other value.
+__host__ __device__ __forceinline__ bool pow2_exponent(double p, int& e) {
+    const uint64_t u = tf32_bits64_of(p);
+    e = (int)(u >> 52) - 1023;
+    return (u & 0xFFFFFFFFFFFFFull) == 0 && e >= -200 && e <= 200;
+}
+
 // A double rounded to float, by integer operations where f32_round_with_residual covers x.
 __host__ __device__ __forceinline__ float f32_rn(double x) {
     float f, r;

@@ -52,9 +52,9 @@ struct GemmArgs {
     int tiles_m, tiles_n;
     // Affine operand tables (set on the host when every entry fits): element (m, k) of A
     // at offA + a0 + m * rAs + k * cAs, element (k, n) of B at offB + b0 + k * rBs + n * cBs.
-    // Gathers then skip the table loads, and an operand whose K index is contiguous is
-    // staged K-fastest (consecutive threads read consecutive elements).
+    // Gathers then skip the table loads.
     int affA, affB;
+    int kfA, kfB;          // stage this operand K-fastest: its K index is the more contiguous one
     long long a0, b0;
     int rAs, cAs, rBs, cBs;
 };
@@ -70,6 +70,11 @@ template <> struct Cplx<df> { using V = df2; };
 // and SM.  The results are those of the plain conversions, bit for bit.
 template <typename T> __device__ __forceinline__ T from_f64(double x) { return T(x); }
 template <> __device__ __forceinline__ float from_f64<float>(double x) { return f32_rn(x); }
+
+// A partial sum as a double; floats widen by integer operations.
+__device__ __forceinline__ double to_f64(double x) { return x; }
+__device__ __forceinline__ double to_f64(float x) { return f64_scaled(x); }
+__device__ __forceinline__ double to_f64(df x) { return f64_scaled(x.h) + f64_scaled(x.l); }
 
 
 // Shared-memory staging of one K step: the complex tiles, and for the FP64 and
@@ -166,7 +171,7 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
     const T sa = g.conjA ? T(-1) : T(1);
     const T sb = g.conjB ? T(-1) : T(1);
     const bool a32 = g.A32 != nullptr, b32 = g.B32 != nullptr;
-    const bool kfA = g.affA && g.cAs == 1, kfB = g.affB && g.rBs == 1;
+    const bool kfA = g.kfA != 0, kfB = g.kfB != 0;
     // this split's share of the flattened (chunk, K) sum
     const int nch = g.nchunk_b ? g.nchunk_b[b] : g.nchunk;
     const int upc = (g.K + ZG_KU - 1) / ZG_KU;
@@ -372,7 +377,7 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
                     const int m = m0 + ty * TM + i, n = n0 + tx * TN + j;
                     if (m < g.M && n < g.N)
                         __stcg(W + split * plane + (long long)m * g.N + n,
-                               make_double2((double)cr[i][j], (double)ci[i][j]));
+                               make_double2(to_f64(cr[i][j]), to_f64(ci[i][j])));
                 }
         }
         // the last CTA of the tile adds the partials (the counter returns to zero for the
@@ -410,7 +415,7 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
 #pragma unroll
             for (int j = 0; j < TN; ++j) {
                 const int m = m0 + ty * TM + i, n = n0 + tx * TN + j;
-                if (m < g.M && n < g.N) put(m, n, (double)cr[i][j], (double)ci[i][j]);
+                if (m < g.M && n < g.N) put(m, n, to_f64(cr[i][j]), to_f64(ci[i][j]));
             }
     }
 }
