@@ -16,7 +16,7 @@
 // instance: a 16 x 16 tile already reads its operands in a tenth of the time its DFMAs
 // take, so tiles and K splits are chosen for even load and little padding
 // (zgemm_shapes.h), and warps outside the result issue none.  Large contractions run at
-// 0.94 of the measured DFMA rate (2x2x2/o8/v32 ring: 349 ms; 362 ms on one resident
+// 0.95 of the measured DFMA rate (2x2x2/o8/v32 ring: 343 ms; 362 ms on one resident
 // 64 x 64 CTA per SM without prefetch).  Contractions with few outputs were bound by one
 // CTA walking the whole K: 3 k points, o = 5, v = 13, one iteration 6.3 -> 1.5 ms; the
 // 2x2x1/o8/v32 double-float F~_oo 2.41 -> 0.18 ms and its R1 terms 4.1 -> 0.7 ms.
@@ -93,15 +93,17 @@ struct ZgemmSmem {
 // A staged operand element travels in registers from its load to the next stage store
 // (the loads of a K step are in flight while the previous one is multiplied).  A
 // complex64 element keeps its 64 bits in .x untouched.
+// conj: 0, or 0x80000000 to negate the imaginary part (a flipped sign bit; a product with -1
+// would be an FP64-pipe operation per element).
 template <typename T>
-__device__ __forceinline__ typename Cplx<T>::V zg_operand(double2 raw, bool c64, T sign) {
+__device__ __forceinline__ typename Cplx<T>::V zg_operand(double2 raw, bool c64, int conj) {
     typename Cplx<T>::V v;
     if (c64) {
         v.x = T(__int_as_float(__double2loint(raw.x)));
-        v.y = T(__int_as_float(__double2hiint(raw.x))) * sign;
+        v.y = T(__int_as_float(__double2hiint(raw.x) ^ conj));
     } else {
         v.x = from_f64<T>(raw.x);
-        v.y = from_f64<T>(raw.y) * sign;
+        v.y = from_f64<T>(__hiloint2double(__double2hiint(raw.y) ^ conj, __double2loint(raw.y)));
     }
     return v;
 }
@@ -168,8 +170,7 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
             if (k3M) cs[i][k3M ? j : 0] = T(0);
         }
 
-    const T sa = g.conjA ? T(-1) : T(1);
-    const T sb = g.conjB ? T(-1) : T(1);
+    const int sa = g.conjA ? (int)0x80000000 : 0, sb = g.conjB ? (int)0x80000000 : 0;
     const bool a32 = g.A32 != nullptr, b32 = g.B32 != nullptr;
     const bool kfA = g.kfA != 0, kfB = g.kfB != 0;
     // this split's share of the flattened (chunk, K) sum
@@ -222,6 +223,7 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
         int kend = c == cl ? kl : g.K;
         fetch(kend);
         for (bool more = true; more;) {
+            const int kst = kend - k0;                // terms of the stage being stored
             __syncthreads();                          // the previous stage has been multiplied
 #pragma unroll
             for (int i = 0; i < EA; ++i) {
@@ -230,7 +232,8 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
                     const int mm = kfA ? e / BK : e % BM, kk = kfA ? e % BK : e / BM;
                     const V v = zg_operand<T>(ra[i], a32, sa);
                     As[kk][mm] = v;
-                    if constexpr (k3M) sm.As[kk][mm] = v.x + v.y;
+                    // (rows outside M x K: no sum, so a warp staging only those issues none)
+                    if constexpr (k3M) sm.As[kk][mm] = pa[i] >= 0 && kk < kst ? v.x + v.y : T(0);
                 }
             }
 #pragma unroll
@@ -240,11 +243,10 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
                     const int nn = kfB ? e / BK : e % BN, kk = kfB ? e % BK : e / BN;
                     const V v = zg_operand<T>(rb[i], b32, sb);
                     Bs[kk][nn] = v;
-                    if constexpr (k3M) sm.Bs[kk][nn] = v.x + v.y;
+                    if constexpr (k3M) sm.Bs[kk][nn] = pb[i] >= 0 && kk < kst ? v.x + v.y : T(0);
                 }
             }
             __syncthreads();
-            const int krem = kend - k0;               // terms of this stage
             k0 += BK;
             if (k0 >= kend) {
                 if (c == cl) more = false;
@@ -261,7 +263,7 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
 #pragma unroll
             for (int kq = 0; kq < KG; ++kq) {
                 const int kk = kq * KS + kgrp;
-                if (kk >= krem) break;
+                if (kk >= kst) break;
                 V a[TM], bb[TN];
 #pragma unroll
                 for (int i = 0; i < TM; ++i) a[i] = As[kk][ty * TM + i];
@@ -332,7 +334,8 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
             }
         }
     }
-    if constexpr (k3M) {
+    const bool writes = active && kgrp == 0;
+    if (k3M && writes) {
 #pragma unroll
         for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -342,7 +345,6 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
                 ci[i][j] = cs[i][k3M ? j : 0] - t1 - t2;
             }
     }
-    const bool writes = active && kgrp == 0;
     double2* const Cb = g.C + g.offC[b];
     double2* const C2 = g.offC2 ? g.C + g.offC2[b] : nullptr;
     // a real alpha takes one FP64 operation per component: the plan's factors are +-1 and
