@@ -181,11 +181,15 @@ struct ccsd_ctx {
     bool cur_oz = false;             // plan building: the operand set being added is the Ozaki one
     int oz_slices = 7;               // slices per operand row (CCSD_OZAKI)
     long long oz_work_elems = 0;     // split partials of the Ozaki GEMMs (complex elements)
-    df2* ovvv_df = nullptr;          // Ozaki form, complex128 ovvv: its double-float copy
-    df2* ooov_df = nullptr;          // the same for complex128 ooov (fused Fock terms)
-    df2* t2_df = nullptr;            // Ozaki iterations: double-float copies for the fused Fock
-    df2* t1_df = nullptr;            // terms (t2_df aliases the idle B operand pool in the
-    df2* fvvpT_df = nullptr;         // pooled layout)
+    // Ozaki form: double-float copies of complex128 operands.  Integrals (constant): ovvv and
+    // ooov, and outside the pooled layout oovv and ovvo; there the tau pass also copies t2 and
+    // tau~.  A double-float GEMM that converts a complex128 operand itself spends eight
+    // FP64-pipe operations per element, more than its products when N is 8: with the copies
+    // the 2x2x2/o8/v32 t1 terms of the ring take 5.0 ms instead of 6.7, R1 3.3 instead of 6.0.
+    df2* dfc[NBUF] = {};
+    df2* t2_df = nullptr;            // t2 for the fused Fock terms: dfc[B_T2], or the idle B operand
+    df2* t1_df = nullptr;            // pool in the pooled layout; and their small operands
+    df2* fvvpT_df = nullptr;
     df2* foop_df = nullptr;
     double2* oz_work = nullptr;
     long long wab_cap_bytes = 12LL << 30;   // bound of the ladder's W' slab buffer
@@ -391,7 +395,11 @@ int finalize_gemm(ccsd_ctx* h, Alloc& al, GemmSpec s, size_t& work_need) {
     for (int w = 0; w < ZG_ARITH; ++w) {
         if (w == ZG_FP32 && h->cfg.precision != CCSD_MIXED) { p.var[w] = p.var[ZG_FP64]; continue; }
         if (w == ZG_DF && !h->has_oz) { p.var[w] = p.var[ZG_FP64]; continue; }
-        auto wide = [&](int b) { return w == ZG_FP32 ? h->shadow[b] == nullptr : !h->in32[b]; };
+        auto wide = [&](int b) {
+            if (w == ZG_FP32) return h->shadow[b] == nullptr;
+            const bool copied = b == B_OOOV || b == B_OVVV || b == B_OOVV || b == B_OVVO || b == B_T2 || b == B_TAUT;
+            return !h->in32[b] && !(w == ZG_DF && copied);
+        };
         const ZgChoice ch = zg_choose(w, s.M, s.N, s.K, s.nchunk, s.nbatch, (wide(s.a) ? 1 : 0) + (wide(s.b) ? 1 : 0),
                                       kSMs);
         const ZgShape& sh = kZgShapes[ch.shape];
@@ -827,6 +835,14 @@ int oz_convert_gemms(ccsd_ctx* h, Alloc& al, std::map<int, GemmSpec>& specs, boo
     return 0;
 }
 
+// The double-float copy of a constant complex128 input.
+int add_df_copy(ccsd_ctx* h, Alloc& al, int b) {
+    h->dfc[b] = (df2*)al.get((size_t)h->bufsize[b] * sizeof(df2));
+    if (al.err) return al.err;
+    if (!al.dry) to_df2_kernel<<<ew_grid(h->bufsize[b]), 256, 0, h->st>>>(h->dfc[b], h->buf[b], h->bufsize[b]);
+    return 0;
+}
+
 // Build the full residual plan.
 int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
     const KGrid& kg = h->kg;
@@ -889,11 +905,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
         if (!al.dry && cudaMemsetAsync(h->tc_err, 0, sizeof(int), h->st) != cudaSuccess) return CCSD_ERR_CUDA;
         if (h->has_oz && !h->in32[B_OVVV]) {
             // the Ozaki W' kernel's t1 terms run in double-float: convert the constant ovvv once
-            h->ovvv_df = (df2*)al.get((size_t)h->bufsize[B_OVVV] * sizeof(df2));
-            if (al.err) return al.err;
-            if (!al.dry)
-                to_df2_kernel<<<ew_grid(h->bufsize[B_OVVV]), 256, 0, h->st>>>(h->ovvv_df, h->buf[B_OVVV],
-                                                                             h->bufsize[B_OVVV]);
+            if ((rc = add_df_copy(h, al, B_OVVV))) return rc;
         }
         long long total_bytes = 0;
         for (TcSet& T : sets) {
@@ -1818,14 +1830,15 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
         // (fock_terms_df_kernel) over double-float copies; the GEMMs stay for FP64 iterations
         for (size_t i = fock_first; i < h->seq.size(); ++i)
             if (h->seq[i].kind == 0) h->seq[i].mode = 1;
-        if (!h->in32[B_OOOV]) {
-            h->ooov_df = (df2*)al.get((size_t)h->bufsize[B_OOOV] * sizeof(df2));
-            if (al.err) return al.err;
-            if (!al.dry)
-                to_df2_kernel<<<ew_grid(h->bufsize[B_OOOV]), 256, 0, h->st>>>(h->ooov_df, h->buf[B_OOOV],
-                                                                             h->bufsize[B_OOOV]);
-        }
-        if (pooled && pool_b_bytes >= (long long)sizeof(df2) * h->n2) {
+        if (!h->in32[B_OOOV] && (rc = add_df_copy(h, al, B_OOOV))) return rc;
+        if (!pooled) {
+            for (int b : {B_OOVV, B_OVVO}) if (!h->in32[b] && (rc = add_df_copy(h, al, b))) return rc;
+            for (int b : {B_T2, B_TAUT}) {
+                h->dfc[b] = (df2*)al.get((size_t)h->n2 * sizeof(df2));
+                if (al.err) return al.err;
+            }
+            h->t2_df = h->dfc[B_T2];              // written by the tau pass
+        } else if (pooled && pool_b_bytes >= (long long)sizeof(df2) * h->n2) {
             h->t2_df = (df2*)pool_b;          // idle between the last tensor-core GEMM and the next residual
         } else {
             h->t2_df = (df2*)al.get((size_t)h->n2 * sizeof(df2));
@@ -1834,7 +1847,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
         h->fvvpT_df = (df2*)al.get((size_t)h->bufsize[B_FVVP] * sizeof(df2));
         h->foop_df = (df2*)al.get((size_t)h->bufsize[B_FOOP] * sizeof(df2));
         if (al.err) return al.err;
-        Step s1{14, 0, h->cur_name, 0.0, 32.0 * (double)(h->n2 + h->n1)};
+        Step s1{14, 0, h->cur_name, 0.0, 32.0 * (double)((h->dfc[B_T2] ? 0 : h->n2) + h->n1)};
         Step s2{13, 0, h->cur_name, 8.0 * 2.0 * (o + v) * (double)h->n2, 16.0 * 4.0 * h->n2};
         s1.mode = s2.mode = 5;
         h->seq.push_back(s1); h->seq.push_back(s2);
@@ -1880,6 +1893,10 @@ GemmArgs gemm_args(const ccsd_ctx* h, const GemmPlan& p, int arith) {
     g.A = h->buf[p.a]; g.B = h->buf[p.b]; g.C = h->buf[p.c]; g.work = h->work; g.cnt = h->cnt;
     g.A32 = (fp32 || h->in32[p.a]) ? h->shadow[p.a] : nullptr;
     g.B32 = (fp32 || h->in32[p.b]) ? h->shadow[p.b] : nullptr;
+    if (arith == ZG_DF) {
+        if (h->dfc[p.a] && !g.A32) { g.A = (const double2*)h->dfc[p.a]; g.dfA = 1; }
+        if (h->dfc[p.b] && !g.B32) { g.B = (const double2*)h->dfc[p.b]; g.dfB = 1; }
+    }
     g.tiles_m = v.tiles_m; g.tiles_n = v.tiles_n; g.nsplit = v.nsplit;
     if (v.nsplit > 1) { g.work += v.work_off; g.cnt += v.cnt_off; }
     return g;
@@ -1911,7 +1928,8 @@ PermOp perm_op(const ccsd_ctx* h, const PermPlan& pp) {
 TauOp tau_op(const ccsd_ctx* h) {
     const bool c64 = h->fp32 && h->cfg.precision == CCSD_MIXED;
     return TauOp{h->buf[B_T1], h->buf[B_T2], h->buf[B_TAU], h->buf[B_TAUT], h->kb_of, h->N, h->o, h->v,
-                 c64 ? h->shadow[B_T2] : nullptr, c64 ? h->shadow[B_TAUT] : nullptr};
+                 c64 ? h->shadow[B_T2] : nullptr, c64 ? h->shadow[B_TAUT] : nullptr,
+                 h->oz_on ? h->dfc[B_T2] : nullptr, h->oz_on ? h->dfc[B_TAUT] : nullptr};
 }
 
 FockTermsOp fock_terms_op(const ccsd_ctx* h) {
@@ -2077,7 +2095,7 @@ void launch_step(ccsd_ctx* h, size_t si) {
                     if (h->in32[B_VVVV]) { z.vvvv32 = h->shadow[B_VVVV]; z.vvvv = nullptr; }
                     else { z.vvvv = h->buf[B_VVVV]; z.vvvv32 = nullptr; }
                     if (h->in32[B_OVVV]) { z.ovvv32 = h->shadow[B_OVVV]; z.ovvv_df = nullptr; }
-                    else { z.ovvv_df = h->ovvv_df; z.ovvv32 = nullptr; }
+                    else { z.ovvv_df = h->dfc[B_OVVV]; z.ovvv32 = nullptr; }
                     z.t1 = h->buf[B_T1];
                     oz_wprime_kernel<<<row_grid((long long)z.nblk * z.nab), 256, (size_t)(z.nef + 2 * z.o) * 16,
                                        h->st>>>(z);
@@ -2102,13 +2120,13 @@ void launch_step(ccsd_ctx* h, size_t si) {
             case 13:  // Ozaki iterations: fused double-float Fock terms into ZR
                 fock_terms_df_kernel<<<ew_grid(h->n2), 256, 0, h->st>>>(FockTermsDfOp{
                     h->buf[B_ZR], h->t2_df, h->t1_df, h->fvvpT_df, h->foop_df,
-                    h->ooov_df, h->in32[B_OOOV] ? h->shadow[B_OOOV] : nullptr,
-                    h->ovvv_df, h->in32[B_OVVV] ? h->shadow[B_OVVV] : nullptr, h->kb_of, N, o, v});
+                    h->dfc[B_OOOV], h->in32[B_OOOV] ? h->shadow[B_OOOV] : nullptr,
+                    h->dfc[B_OVVV], h->in32[B_OVVV] ? h->shadow[B_OVVV] : nullptr, h->kb_of, N, o, v});
                 ++h->launches;
                 break;
             case 14:  // their double-float copies
-                to_df_kernel<<<ew_grid(h->n2 + h->n1), 256, 0, h->st>>>(ToDfOp{
-                    h->t2_df, h->buf[B_T2], h->n2, h->t1_df, h->buf[B_T1], h->n1,
+                to_df_kernel<<<ew_grid((h->dfc[B_T2] ? 0 : h->n2) + h->n1), 256, 0, h->st>>>(ToDfOp{
+                    h->t2_df, h->buf[B_T2], h->dfc[B_T2] ? 0 : h->n2, h->t1_df, h->buf[B_T1], h->n1,
                     h->fvvpT_df, h->buf[B_FVVP], h->foop_df, h->buf[B_FOOP], N, o, v});
                 ++h->launches;
                 break;
@@ -2168,7 +2186,11 @@ StepAccess step_access(const ccsd_ctx* h, const Step& st) {
         if (!halves || part != 2) v.push_back(p);
         if (halves && part != 1) v.push_back(p + 1);
     };
-    auto rd = [&](int id) { add(a.rd, id, 0); if (h->shadow[id]) a.rd.push_back(h->shadow[id]); };
+    auto rd = [&](int id) {
+        add(a.rd, id, 0);
+        if (h->shadow[id]) a.rd.push_back(h->shadow[id]);
+        if (h->dfc[id]) a.rd.push_back(h->dfc[id]);
+    };
     auto wr = [&](int id, int part = 0) { add(a.wr, id, part); };
     switch (st.kind) {
         case 0: { const GemmPlan& p = h->gemms[st.idx]; rd(p.a); rd(p.b); wr(p.c, p.part); break; }
@@ -2177,6 +2199,7 @@ StepAccess step_access(const ccsd_ctx* h, const Step& st) {
         case 3:
             add(a.rd, B_T1, 0); add(a.rd, B_T2, 0); wr(B_TAU); wr(B_TAUT);
             if (h->shadow[B_T2]) { a.wr.push_back(h->shadow[B_T2]); a.wr.push_back(h->shadow[B_TAUT]); }
+            if (h->dfc[B_T2]) { a.wr.push_back(h->dfc[B_T2]); a.wr.push_back(h->dfc[B_TAUT]); }
             break;
         case 4: rd(B_ZR); wr(B_R2); break;
         case 5: {
@@ -2201,8 +2224,9 @@ StepAccess step_access(const ccsd_ctx* h, const Step& st) {
             break;
         case 14:
             rd(B_T2); rd(B_T1); rd(B_FVVP); rd(B_FOOP);
-            for (const void* p : {(const void*)h->t2_df, (const void*)h->t1_df, (const void*)h->fvvpT_df,
-                                  (const void*)h->foop_df}) a.wr.push_back(p);
+            for (const void* p : {(const void*)h->t1_df, (const void*)h->fvvpT_df, (const void*)h->foop_df})
+                a.wr.push_back(p);
+            if (!h->dfc[B_T2]) a.wr.push_back(h->t2_df);
             break;
     }
     return a;

@@ -33,34 +33,61 @@ struct TauOp {
     double2* tau; double2* taut;
     const int* kb_of; int N, o, v;
     float2* t2_32; float2* taut_32;
-    // vb, nvb: this block's index and the block count of its (virtual) grid
+    df2* t2_df; df2* taut_df;      // Ozaki iterations: double-float copies of t2 and tau~ (or null)
+    // vb, nvb: this block's index and the block count of its (virtual) grid.  A unit is 1024
+    // elements of one momentum block; the element index is decoded only in blocks with a t1
+    // term (ki = ka or ki = kb), the others stream.
     __device__ void run(long long vb, long long nvb) const {
         const long long blk = (long long)o * o * v * v;
-        const long long total = (long long)N * N * N * blk;
-        for (long long e = vb * blockDim.x + threadIdx.x; e < total; e += nvb * blockDim.x) {
-            const long long kk = e / blk;
-            int r = (int)(e % blk);
-            const int b = r % v; r /= v;
-            const int a = r % v; r /= v;
-            const int j = r % o; const int i = r / o;
+        const long long nseg = (blk + 1023) / 1024;
+        for (long long u = vb; u < nseg * N * N * N; u += nvb) {
+            const long long kk = u / nseg, base = kk * blk;
+            const long long e0 = (u - kk * nseg) * 1024;
             const int ka = (int)(kk % N), kj = (int)((kk / N) % N), ki = (int)(kk / ((long long)N * N));
             const int kb = kb_of[kk];
-            double2 x = make_double2(0.0, 0.0);
-            if (ki == ka) {
-                const double2 p = cmul(t1[((long long)ki * o + i) * v + a], t1[((long long)kj * o + j) * v + b]);
-                x.x += p.x; x.y += p.y;
+            double2 t[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const long long e = e0 + q * 256 + threadIdx.x;
+                t[q] = e < blk ? t2[base + e] : make_double2(0.0, 0.0);
             }
-            if (ki == kb) {
-                const double2 p = cmul(t1[((long long)ki * o + i) * v + b], t1[((long long)kj * o + j) * v + a]);
-                x.x -= p.x; x.y -= p.y;
-            }
-            const double2 t = t2[e];
-            tau[e] = make_double2(t.x + x.x, t.y + x.y);
-            const double2 tt = make_double2(t.x + 0.5 * x.x, t.y + 0.5 * x.y);
-            taut[e] = tt;
-            if (t2_32) {
-                t2_32[e] = make_float2(f32_rn(t.x), f32_rn(t.y));
-                taut_32[e] = make_float2(f32_rn(tt.x), f32_rn(tt.y));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const long long e = e0 + q * 256 + threadIdx.x;
+                if (e >= blk) break;
+                double2 tf = t[q], tt = t[q];
+                if (ki == ka || ki == kb) {
+                    int b, a, j, i;
+                    if (blk < (1LL << 31)) {
+                        unsigned r = (unsigned)e;
+                        b = (int)(r % (unsigned)v); r /= (unsigned)v;
+                        a = (int)(r % (unsigned)v); r /= (unsigned)v;
+                        j = (int)(r % (unsigned)o); i = (int)(r / (unsigned)o);
+                    } else {
+                        long long r = e;
+                        b = (int)(r % v); r /= v;
+                        a = (int)(r % v); r /= v;
+                        j = (int)(r % o); i = (int)(r / o);
+                    }
+                    double2 x = make_double2(0.0, 0.0);
+                    if (ki == ka) {
+                        const double2 p = cmul(t1[((long long)ki * o + i) * v + a], t1[((long long)kj * o + j) * v + b]);
+                        x.x += p.x; x.y += p.y;
+                    }
+                    if (ki == kb) {
+                        const double2 p = cmul(t1[((long long)ki * o + i) * v + b], t1[((long long)kj * o + j) * v + a]);
+                        x.x -= p.x; x.y -= p.y;
+                    }
+                    tf = make_double2(tf.x + x.x, tf.y + x.y);
+                    tt = make_double2(tt.x + 0.5 * x.x, tt.y + 0.5 * x.y);
+                }
+                tau[base + e] = tf;
+                taut[base + e] = tt;
+                if (t2_32) {
+                    t2_32[base + e] = make_float2(f32_rn(t[q].x), f32_rn(t[q].y));
+                    taut_32[base + e] = make_float2(f32_rn(tt.x), f32_rn(tt.y));
+                }
+                if (t2_df) { t2_df[base + e] = df2_of(t[q]); taut_df[base + e] = df2_of(tt); }
             }
         }
     }
@@ -498,7 +525,7 @@ struct ToDfOp {
         const long long nv = (long long)N * v * v, no = (long long)N * o * o;
         const long long total = n2 + n1 + nv + no;
         for (long long e = vb * blockDim.x + threadIdx.x; e < total; e += nvb * blockDim.x) {
-            if (e < n2) { t2_df[e] = ld_df2(t2 + e); continue; }
+            if (e < n2) { t2_df[e] = df2_of(t2[e]); continue; }
             long long f = e - n2;
             if (f < n1) { t1_df[f] = ld_df2(t1 + f); continue; }
             f -= n1;

@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "tf32_split.cuh"
+
 namespace ccsdk {
 
 // The rounded FP32 operations the error-free transformations are written with.  On
@@ -82,13 +84,23 @@ __device__ __forceinline__ df2 ld_df2(const double2* p) { const double2 z = *p; 
 __device__ __forceinline__ df2 ld_df2(const float2* p) { const float2 z = *p; return df2{df(z.x), df(z.y)}; }
 __device__ __forceinline__ df2 ld_df2(const df2* p) { return *p; }
 
+// A double as a double-float pair from its bit pattern (f32_round_with_residual: the float
+// nearest x and the float of the exact remainder, as df(x) forms them), so that copies of
+// whole arrays stay off the FP64 pipe (four operations per component otherwise).
+__device__ __forceinline__ df df_of_bits(double x) {
+    float f, r;
+    if (f32_zero(x, f)) return df(f, 0.f);
+    return f32_round_with_residual(x, f, r) ? df(f, r) : df(x);
+}
+__device__ __forceinline__ df2 df2_of(double2 z) { return df2{df_of_bits(z.x), df_of_bits(z.y)}; }
+
 // dst = src as double-float pairs (the split costs FP64 operations, so constant inputs
 // are converted once)
 static __global__ void to_df2_kernel(df2* __restrict__ dst, const double2* __restrict__ src, long long n)
 {
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
          e += (long long)gridDim.x * blockDim.x)
-        dst[e] = ld_df2(src + e);
+        dst[e] = df2_of(src[e]);
 }
 
 }  // namespace ccsdk

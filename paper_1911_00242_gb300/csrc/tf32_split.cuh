@@ -62,8 +62,10 @@ __host__ __device__ __forceinline__ void split_tf32f(float x, float& big, float&
 // of x, small from the remainder x - big = (f - big) + (x - f), whose first term is
 // exact in FP32 and whose second is the float residual (FP32 operations only; outside
 // the range of f32_round_with_residual, FP64 arithmetic).
+__host__ __device__ __forceinline__ bool f32_zero(double x, float& f);
 __host__ __device__ __forceinline__ void split_tf32(double x, float& big, float& small) {
     float f, r;
+    if (f32_zero(x, f)) { big = f; small = 0.f; return; }
     if (f32_round_with_residual(x, f, r)) {
         big = tf32_round(f);
         small = tf32_round((f - big) + r);
@@ -100,9 +102,18 @@ __host__ __device__ __forceinline__ bool pow2_exponent(double p, int& e) {
     return (u & 0xFFFFFFFFFFFFFull) == 0 && e >= -200 && e <= 200;
 }
 
+// +-0 as a float; false for any other x.  Blocks that time reversal makes real have only
+// zeros for imaginary parts, so zero does not take the FP64 path.
+__host__ __device__ __forceinline__ bool f32_zero(double x, float& f) {
+    const uint64_t u = tf32_bits64_of(x);
+    f = tf32_float_of((uint32_t)(u >> 32));
+    return (u << 1) == 0;
+}
+
 // A double rounded to float, by integer operations where f32_round_with_residual covers x.
 __host__ __device__ __forceinline__ float f32_rn(double x) {
     float f, r;
+    if (f32_zero(x, f)) return f;
     return f32_round_with_residual(x, f, r) ? f : (float)x;
 }
 

@@ -33,6 +33,7 @@
 #include "tf32_split.cuh"
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <type_traits>
 
 namespace ccsdk {
 
@@ -54,6 +55,7 @@ struct GemmArgs {
     // at offA + a0 + m * rAs + k * cAs, element (k, n) of B at offB + b0 + k * rBs + n * cBs.
     // Gathers then skip the table loads.
     int affA, affB;
+    int dfA, dfB;          // A / B holds double-float pairs (copies for the df instance)
     int kfA, kfB;          // stage this operand K-fastest: its K index is the more contiguous one
     long long a0, b0;
     int rAs, cAs, rBs, cBs;
@@ -93,11 +95,19 @@ struct ZgemmSmem {
 // A staged operand element travels in registers from its load to the next stage store
 // (the loads of a K step are in flight while the previous one is multiplied).  A
 // complex64 element keeps its 64 bits in .x untouched.
+// (df instance: split, the element is a stored double-float pair, read by its bits.)
 // conj: 0, or 0x80000000 to negate the imaginary part (a flipped sign bit; a product with -1
 // would be an FP64-pipe operation per element).
 template <typename T>
-__device__ __forceinline__ typename Cplx<T>::V zg_operand(double2 raw, bool c64, int conj) {
+__device__ __forceinline__ typename Cplx<T>::V zg_operand(double2 raw, bool c64, bool split, int conj) {
     typename Cplx<T>::V v;
+    if constexpr (sizeof(v) == sizeof(df2) && sizeof(T) == sizeof(df) && !std::is_same<T, double>::value) {
+        if (split) {
+            v.x = df(__int_as_float(__double2loint(raw.x)), __int_as_float(__double2hiint(raw.x)));
+            v.y = df(__int_as_float(__double2loint(raw.y) ^ conj), __int_as_float(__double2hiint(raw.y) ^ conj));
+            return v;
+        }
+    }
     if (c64) {
         v.x = T(__int_as_float(__double2loint(raw.x)));
         v.y = T(__int_as_float(__double2hiint(raw.x) ^ conj));
@@ -230,7 +240,7 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
                 const int e = tid + i * NT;
                 if (BM * BK % NT == 0 || e < BM * BK) {
                     const int mm = kfA ? e / BK : e % BM, kk = kfA ? e % BK : e / BM;
-                    const V v = zg_operand<T>(ra[i], a32, sa);
+                    const V v = zg_operand<T>(ra[i], a32, g.dfA != 0, sa);
                     As[kk][mm] = v;
                     // (rows outside M x K: no sum, so a warp staging only those issues none)
                     if constexpr (k3M) sm.As[kk][mm] = pa[i] >= 0 && kk < kst ? v.x + v.y : T(0);
@@ -241,7 +251,7 @@ __device__ __forceinline__ void zgemm_tile(const GemmArgs& g, int tile, long lon
                 const int e = tid + i * NT;
                 if (BN * BK % NT == 0 || e < BN * BK) {
                     const int nn = kfB ? e / BK : e % BN, kk = kfB ? e % BK : e / BN;
-                    const V v = zg_operand<T>(rb[i], b32, sb);
+                    const V v = zg_operand<T>(rb[i], b32, g.dfB != 0, sb);
                     Bs[kk][nn] = v;
                     if constexpr (k3M) sm.Bs[kk][nn] = pb[i] >= 0 && kk < kst ? v.x + v.y : T(0);
                 }
