@@ -112,23 +112,17 @@ __host__ __device__ constexpr uint32_t oz_idesc_bf16(int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(OZ_BM >> 4) << 24);
 }
 
-__device__ __forceinline__ void oz_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n\t.reg .pred p;\n\t"
-                 "setp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 :: "r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
-}
-
-// The four K = 16 steps (32 bytes each) of one 64-wide K slice into one accumulator:
-// the first accumulates iff acc != 0, the others always.
+// The four K = 16 steps (32 bytes each) of one 64-wide K slice into one accumulator, by one
+// elected lane of a converged warp: the first accumulates iff acc != 0, the others always.
 __device__ __forceinline__ void oz_mma4(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n\t.reg .pred p, t;\n\t"
+    asm volatile("{\n\t.reg .pred p, e;\n\t"
+                 "elect.sync _|e, 0xffffffff;\n\t"
                  "setp.ne.b32 p, %4, 0;\n\t"
-                 "setp.eq.b32 t, %4, %4;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %5, %6, %3, t;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %7, %8, %3, t;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %9, %10, %3, t;\n\t}"
+                 "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+                 "setp.eq.b32 p, %4, %4;\n\t"
+                 "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %5, %6, %3, p;\n\t"
+                 "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %7, %8, %3, p;\n\t"
+                 "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %9, %10, %3, p;\n\t}"
                  :: "r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc), "l"(adesc + 2), "l"(bdesc + 2),
                     "l"(adesc + 4), "l"(bdesc + 4), "l"(adesc + 6), "l"(bdesc + 6) : "memory");
 }
@@ -176,7 +170,7 @@ __device__ __forceinline__ int oz_issue_slice(int S_rt, uint32_t tmem, uint64_t 
         if (SC == 0 && p >= S) break;
         const int h = ja & 1;
         if (h == 0) {
-            if (!mbar_wait(fA0 + 8 * ps, pph, abort_flag, spin_limit)) return 2;
+            if (!mbar_wait_warp(fA0 + 8 * ps, pph, abort_flag, spin_limit)) return 2;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
         const uint64_t da = da0 + (uint64_t)((2 * ps + h) * (OZ_A_BYTES >> 4));
@@ -188,7 +182,7 @@ __device__ __forceinline__ int oz_issue_slice(int S_rt, uint32_t tmem, uint64_t 
             if (fresh && w > 0) {
                 // diagonals q0 .. q0+n-1 of the previous window have been promoted
                 for (int d = q0; d < q0 + n; ++d)
-                    if (!mbar_wait(accE0 + 8 * d, (uint32_t)((w - 1) & 1), abort_flag, spin_limit)) return 4;
+                    if (!mbar_wait_warp(accE0 + 8 * d, (uint32_t)((w - 1) & 1), abort_flag, spin_limit)) return 4;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             }
             const uint64_t db = dbs + (uint64_t)(q0 * (OZ_B_BYTES >> 4));
@@ -197,11 +191,11 @@ __device__ __forceinline__ int oz_issue_slice(int S_rt, uint32_t tmem, uint64_t 
             oz_mma4(dst, da, db, idesc, fresh ? 0u : 1u);
         }
         if (h == 1 || ja + 1 == totalA) {
-            tc_commit(eA0 + 8 * ps);
+            tc_commit_warp(eA0 + 8 * ps);
             if (++ps == nP) { ps = 0; pph ^= 1u; }
         }
         ++ja;
-        if (wlast) tc_commit(accF0 + 8 * p);
+        if (wlast) tc_commit_warp(accF0 + 8 * p);
     }
     return 0;
 }
@@ -227,7 +221,7 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     volatile uint32_t* tmem_slot = (volatile uint32_t*)(drain + 1);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int ntile = g.tiles_m * g.tiles_n;
     const int tile = blockIdx.x % ntile;
     const long long b = (blockIdx.x / ntile) % g.nbatch;
@@ -260,7 +254,7 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     }
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     const int nch = g.nchunk_b ? g.nchunk_b[b] : g.nchunk;
     const int W = oz_kwin(S), nw = oz_nwin(g.kstages, S);
@@ -335,45 +329,45 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer: per K slice, the B slot, then oz_issue_slice (the
-            // slice count 7, the default, compiled as a constant).  The descriptors are the
-            // slot-0 ones plus the slot offset (their start-address field is the shared
-            // address / 16, below 2^14); slots and phases advance incrementally.
-            const uint64_t da0 = smem_desc_sw128(smem_u32(stA)), db0 = smem_desc_sw128(smem_u32(stB));
-            const uint32_t fA0 = smem_u32(&fullA[0]), eA0 = smem_u32(&emptyA[0]);
-            const uint32_t accF0 = smem_u32(&acc_full[0]), accE0 = smem_u32(&acc_empty[0]);
-            int ja = 0, ps = 0, bs = 0, w = 0;
-            uint32_t pph = 0, bph = 0;
-            int fail = 0;
-            for (int u = u0; u < u1 && !fail; ++u, ++w) {
-                const int k0 = (u % nw) * W, k1 = min(k0 + W, g.kstages);
-                for (int kst = k0; kst < k1; ++kst) {
-                    if (!mbar_wait(smem_u32(&fullB[bs]), bph, abort_flag, g.spin_limit)) {
-                        fail = 2;
-                        break;
-                    }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint64_t dbs = db0 + (uint64_t)((bs * bslot) >> 4);
-                    const bool wfirst = kst == k0, wlast = kst + 1 == k1;
-                    fail = S == 7 ? oz_issue_slice<7>(S, tmem, da0, dbs, fA0, eA0, accF0, accE0, nP, totalA, ja, ps,
-                                                      pph, wfirst, wlast, w, abort_flag, g.spin_limit)
-                                  : oz_issue_slice<0>(S, tmem, da0, dbs, fA0, eA0, accF0, accE0, nP, totalA, ja, ps,
-                                                      pph, wfirst, wlast, w, abort_flag, g.spin_limit);
-                    if (fail) break;
-                    tc_commit(smem_u32(&emptyB[bs]));
-                    bs ^= 1;
-                    if (bs == 0) bph ^= 1u;
+        // ---------------- MMA issuer, the whole warp in uniform code (one elected lane issues):
+        // per K slice, the B slot, then oz_issue_slice (the slice count 7, the default,
+        // compiled as a constant).  The descriptors are the slot-0 ones plus the slot offset
+        // (their start-address field is the shared address / 16, below 2^14); slots and phases
+        // advance incrementally.
+        const uint64_t da0 = smem_desc_sw128(smem_u32(stA)), db0 = smem_desc_sw128(smem_u32(stB));
+        const uint32_t fA0 = smem_u32(&fullA[0]), eA0 = smem_u32(&emptyA[0]);
+        const uint32_t accF0 = smem_u32(&acc_full[0]), accE0 = smem_u32(&acc_empty[0]);
+        int ja = 0, ps = 0, bs = 0, w = 0;
+        uint32_t pph = 0, bph = 0;
+        int fail = 0;
+        for (int u = u0; u < u1 && !fail; ++u, ++w) {
+            const int k0 = (u % nw) * W, k1 = min(k0 + W, g.kstages);
+            for (int kst = k0; kst < k1; ++kst) {
+                if (!mbar_wait_warp(smem_u32(&fullB[bs]), bph, abort_flag, g.spin_limit)) {
+                    fail = 2;
+                    break;
                 }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint64_t dbs = db0 + (uint64_t)((bs * bslot) >> 4);
+                const bool wfirst = kst == k0, wlast = kst + 1 == k1;
+                fail = S == 7 ? oz_issue_slice<7>(S, tmem, da0, dbs, fA0, eA0, accF0, accE0, nP, totalA, ja, ps,
+                                                  pph, wfirst, wlast, w, abort_flag, g.spin_limit)
+                              : oz_issue_slice<0>(S, tmem, da0, dbs, fA0, eA0, accF0, accE0, nP, totalA, ja, ps,
+                                                  pph, wfirst, wlast, w, abort_flag, g.spin_limit);
+                if (fail) break;
+                tc_commit_warp(smem_u32(&emptyB[bs]));
+                bs ^= 1;
+                if (bs == 0) bph ^= 1u;
             }
-            if (fail) {
-                atomicCAS(g.err, 0, fail);
-                *abort_flag = 1;
-            }
-            if (*abort_flag) {
-                tc_commit(smem_u32(drain));
-                mbar_wait(smem_u32(drain), 0u, nullptr, TC_DRAIN_LIMIT);
-            }
+        }
+        if (fail && lane == 0) {
+            atomicCAS(g.err, 0, fail);
+            *abort_flag = 1;
+        }
+        __syncwarp();
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) {
+            tc_commit_warp(smem_u32(drain));
+            mbar_wait(smem_u32(drain), 0u, nullptr, TC_DRAIN_LIMIT);
         }
     } else {
         // ---------------- accumulator warps: exact window sums -> (hi, lo) in registers,

@@ -123,6 +123,30 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return false;
 }
 
+// The same by a whole warp: every lane polls and the votes make the outcome uniform.  The
+// MMA issuers run warp-uniform code (with one elected lane inside each tcgen05 statement), so
+// that descriptors, slots and phases stay in uniform registers: a single lane's loop had to
+// move every operand of every MMA there, which cost more than the MMA itself (2x2x2/o8/v32
+// ring: Ozaki 13.0 -> 10.7 ms, split TF32 2.16 -> 1.93 ms; the same MMAs on resident operands
+// with constant descriptors take 3702 of the ideal 3584 clocks per Ozaki K slice, the single
+// lane's loop took 6880).
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                               long long limit) {
+    for (long long i = 0; i < limit; ++i) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.b32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (__all_sync(0xffffffffu, ok != 0)) return true;
+        if ((i & 1023) == 1023 && __any_sync(0xffffffffu, *abort_flag != 0)) return false;
+    }
+    return false;
+}
+
+// The index of this warp, in a form the compiler knows to be uniform.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
                  " [%0], [%1, {%2, %3}], [%4];"
@@ -157,15 +181,20 @@ __host__ __device__ constexpr uint32_t tc_idesc_tf32() {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TC_BN >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
 }
 
+// One MMA by an elected lane of a converged warp.
 __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n\t.reg .pred p;\n\t"
+    asm volatile("{\n\t.reg .pred p, e;\n\t"
+                 "elect.sync _|e, 0xffffffff;\n\t"
                  "setp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+                 "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
                  :: "r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
 }
 
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+// Commit of the MMAs issued so far to an mbarrier, by one elected lane of a converged warp.
+__device__ __forceinline__ void tc_commit_warp(uint32_t bar) {
+    asm volatile("{\n\t.reg .pred e;\n\t"
+                 "elect.sync _|e, 0xffffffff;\n\t"
+                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
                  :: "r"(bar) : "memory");
 }
 
@@ -198,7 +227,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA_big, const 
     volatile uint32_t* tmem_slot = (volatile uint32_t*)(bars + 2 * TC_STAGES + 5);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int ntile = g.tiles_m * g.tiles_n;
     const int tile = (int)(bid % ntile);
     const long long b = bid / ntile;
@@ -226,7 +255,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA_big, const 
     }
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     // one stage = one K slice of both parts of A and B; all terms of the slice run on it
     const bool split3 = g.nterms == 3;
@@ -274,56 +303,54 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA_big, const 
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer.  Stage descriptors: the stage-0 one plus the stage
-            // and part offsets (the start-address field is the shared address / 16, below 2^14).
-            const uint32_t idesc = tc_idesc_tf32();
-            const uint64_t d0 = smem_desc_sw64(smem_u32(smem));
-            const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[TC_STAGES]);
-            for (int s = 0; s < total; ++s) {
-                const int seg = s / TC_PROMOTE_STAGES;
-                const int buf = seg & 1;
-                const bool seg_first = (s % TC_PROMOTE_STAGES) == 0;
-                if (seg_first && seg >= 2) {
-                    // the accumulator warps must have drained this buffer's previous segment
-                    if (!mbar_wait(smem_u32(&acc_empty[buf]), (uint32_t)((seg - 2) >> 1) & 1u, abort_flag, g.spin_limit)) {
-                        atomicCAS(g.err, 0, 4);
-                        *abort_flag = 1;
-                        break;
-                    }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                }
-                const int st = s & (TC_STAGES - 1);
-                const uint32_t ph = (uint32_t)(s / TC_STAGES) & 1u;
-                if (!mbar_wait(full0 + 8 * st, ph, abort_flag, g.spin_limit)) {
-                    atomicCAS(g.err, 0, 2);
-                    *abort_flag = 1;
+        // ---------------- MMA issuer: the whole warp in uniform code, one elected lane issues.
+        // Stage descriptors: the stage-0 one plus the stage and part offsets (the start-address
+        // field is the shared address / 16, below 2^14).
+        const uint32_t idesc = tc_idesc_tf32();
+        const uint64_t d0 = smem_desc_sw64(smem_u32(smem));
+        const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[TC_STAGES]);
+        for (int s = 0; s < total; ++s) {
+            const int seg = s / TC_PROMOTE_STAGES;
+            const int buf = seg & 1;
+            const bool seg_first = (s % TC_PROMOTE_STAGES) == 0;
+            if (seg_first && seg >= 2) {
+                // the accumulator warps must have drained this buffer's previous segment
+                if (!mbar_wait_warp(smem_u32(&acc_empty[buf]), (uint32_t)((seg - 2) >> 1) & 1u, abort_flag, g.spin_limit)) {
+                    if (lane == 0) { atomicCAS(g.err, 0, 4); *abort_flag = 1; }
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint64_t dab = d0 + (uint64_t)(st * (TC_STAGE_BYTES >> 4));   // A big
-                const uint64_t das = dab + (uint64_t)(TC_A_BYTES >> 4);              // A small
-                const uint64_t dbb = dab + (uint64_t)((2 * TC_A_BYTES) >> 4);        // B big
-                const uint64_t dbs = dbb + (uint64_t)(TC_B_BYTES >> 4);              // B small
-                const uint32_t dst = tmem + (uint32_t)(buf * TC_BN);
+            }
+            const int st = s & (TC_STAGES - 1);
+            const uint32_t ph = (uint32_t)(s / TC_STAGES) & 1u;
+            if (!mbar_wait_warp(full0 + 8 * st, ph, abort_flag, g.spin_limit)) {
+                if (lane == 0) { atomicCAS(g.err, 0, 2); *abort_flag = 1; }
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint64_t dab = d0 + (uint64_t)(st * (TC_STAGE_BYTES >> 4));   // A big
+            const uint64_t das = dab + (uint64_t)(TC_A_BYTES >> 4);              // A small
+            const uint64_t dbb = dab + (uint64_t)((2 * TC_A_BYTES) >> 4);        // B big
+            const uint64_t dbs = dbb + (uint64_t)(TC_B_BYTES >> 4);              // B small
+            const uint32_t dst = tmem + (uint32_t)(buf * TC_BN);
 #pragma unroll
-                for (int kk = 0; kk < 2; ++kk) {                                     // K = 8 tf32 (32 bytes) each
-                    const uint64_t o = (uint64_t)(2 * kk);
-                    tc_mma(dst, dab + o, dbb + o, idesc, (seg_first && kk == 0) ? 0u : 1u);
-                    if (split3) {
-                        tc_mma(dst, dab + o, dbs + o, idesc, 1u);
-                        tc_mma(dst, das + o, dbb + o, idesc, 1u);
-                    }
+            for (int kk = 0; kk < 2; ++kk) {                                     // K = 8 tf32 (32 bytes) each
+                const uint64_t o = (uint64_t)(2 * kk);
+                tc_mma(dst, dab + o, dbb + o, idesc, (seg_first && kk == 0) ? 0u : 1u);
+                if (split3) {
+                    tc_mma(dst, dab + o, dbs + o, idesc, 1u);
+                    tc_mma(dst, das + o, dbb + o, idesc, 1u);
                 }
-                tc_commit(empty0 + 8 * st);                      // stage free once these MMAs have read it
-                if ((s % TC_PROMOTE_STAGES) == TC_PROMOTE_STAGES - 1 || s == total - 1)
-                    tc_commit(smem_u32(&acc_full[buf]));        // segment complete
             }
-            if (*abort_flag) {
-                // MMAs already issued must finish before the TMEM is released (bounded)
-                tc_commit(smem_u32(drain));
-                mbar_wait(smem_u32(drain), 0u, nullptr, TC_DRAIN_LIMIT);
-            }
+            tc_commit_warp(empty0 + 8 * st);                      // stage free once these MMAs have read it
+            if ((s % TC_PROMOTE_STAGES) == TC_PROMOTE_STAGES - 1 || s == total - 1)
+                tc_commit_warp(smem_u32(&acc_full[buf]));        // segment complete
+        }
+        __syncwarp();
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) {
+            // MMAs already issued must finish before the TMEM is released (bounded)
+            tc_commit_warp(smem_u32(drain));
+            mbar_wait(smem_u32(drain), 0u, nullptr, TC_DRAIN_LIMIT);
         }
     } else {
         // ---------------- accumulator warps: promote every segment, then the epilogue
