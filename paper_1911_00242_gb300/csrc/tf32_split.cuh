@@ -84,7 +84,7 @@ inline double f64_of_bits(uint64_t u) { double x; memcpy(&x, &u, sizeof x); retu
 
 // x 2^e (negated if neg) as a double, exactly, from the bit pattern with integer operations
 // (a conversion and a scaling would be two operations on GB300's FP64 pipe).  |e| <= 800;
-// zeros, subnormals, infinities and NaN take the FP64 path.
+// subnormals, infinities and NaN take the FP64 path.
 __host__ __device__ __forceinline__ double f64_scaled(float x, int e = 0, bool neg = false) {
     const uint32_t u = tf32_bits_of(x) ^ (neg ? 0x80000000u : 0u);
     const uint32_t ex = (u >> 23) & 0xffu;
@@ -92,6 +92,7 @@ __host__ __device__ __forceinline__ double f64_scaled(float x, int e = 0, bool n
         const uint32_t hi = (u & 0x80000000u) | ((ex + (uint32_t)(896 + e)) << 20) | ((u & 0x7fffffu) >> 3);
         return f64_of_bits(((uint64_t)hi << 32) | (uint64_t)(u << 29));
     }
+    if ((u << 1) == 0) return f64_of_bits((uint64_t)u << 32);       // +-0
     return (double)tf32_float_of(u) * f64_of_bits((uint64_t)(1023 + e) << 52);
 }
 
