@@ -869,6 +869,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
         int KQ, kpl, kplp, kpr, kpo;
         long long epb;                       // bytes per operand element
         TcBuf la, lap, lb, ra, rb, b1, ha, hb, h2a, h2b;
+        TcBuf xb[2][2], wa[2], wb[2][2];     // packed hole-hole operands, by class (see pack_hh)
         long long lb_floats;                 // ladder B capacity (elements per part / slice plane)
         long long lb_sc_rows;                // and its row scales (Ozaki): the (e < f) rows are shorter
         long long lad_max, lad_cap, pa, pb;  // sizes in elements per part / plane
@@ -883,7 +884,31 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
     float* pool_asc = nullptr;
     float* pool_bsc = nullptr;    // Ozaki pools: row scales
     long long pool_b_bytes = 0;
-    const long long nlt_vv = (long long)v * (v - 1) / 2;
+    const long long nlt_vv = (long long)v * (v - 1) / 2, nlt_oo = (long long)o * (o - 1) / 2;
+    // Hole-hole contractions on the tensor cores, packed by antisymmetry like the ladder: a
+    // class of outputs and one of summed pairs, each (p < q) with all orbital pairs or (p = q)
+    // with the ordered ones, a quarter of the products and of the tau operand.  The classes
+    // are up to four launches instead of one, so small problems (below kPackHhFlops) and the
+    // pooled layout keep the full sums.  At 2x2x2/o8/v32 the two steps take 3.8 ms instead of
+    // 8.2 (Ozaki) and 1.6 instead of 2.1 (mixed).
+    constexpr double kPackHhFlops = 4e9;
+    bool pack_hh = tcp && 8.0 * N * N * N * (double)N * oo * oo * vv >= kPackHhFlops;   // and not pooled (below)
+    struct PairClass { std::vector<std::pair<int, int>> pq; std::vector<std::vector<int>> in; };
+    // pairs (p <= q) of class `diag` with the first members k of the summed pairs of class `diag_in`
+    auto pair_class = [&](int diag, int diag_in) {
+        PairClass r;
+        for (int p = 0; p < N; ++p) for (int q = p; q < N; ++q) {
+            if ((p == q) != (diag == 1)) continue;
+            const int S = kg.k4(p, q, 0);
+            std::vector<int> ks;
+            for (int k = 0; k < N; ++k) { const int k2 = kg.k4(S, 0, k); if (diag_in ? k == k2 : k < k2) ks.push_back(k); }
+            if (ks.empty()) continue;
+            r.pq.push_back({p, q});
+            r.in.push_back(ks);
+        }
+        return r;
+    };
+    auto class_blocks = [](const PairClass& c) { long long n = 0; for (const auto& x : c.in) n += (long long)x.size(); return n; };
     if (tcp) {
         const long long N3l = (long long)N * N * N;
         h->tc_err = (int*)al.get(sizeof(int));
@@ -945,6 +970,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
             total_bytes += total * T.epb;
         }
         pooled = h->cfg.lean || total_bytes > (24LL << 30) * (long long)sets.size();
+        if (pooled) pack_hh = false;
         if (!pooled) {
             for (TcSet& T : sets) {
                 h->cur_oz = T.oz;
@@ -954,9 +980,24 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
                     (rc = tc_alloc(h, al, T.lb, T.lb_floats / T.kpl + 1, T.kpl, T.lb_floats / std::max(T.kplp, T.KQ) + 1)) ||
                     (rc = tc_alloc(h, al, T.ra, N3l * ov, T.kpr)) || (rc = tc_alloc(h, al, T.rb, N3l * 2 * ov, T.kpr)) ||
                     (rc = tc_alloc(h, al, T.b1, N3l * 2 * ov, T.kpr)) ||
-                    (rc = tc_alloc(h, al, T.ha, N3l * oo, T.kpl)) || (rc = tc_alloc(h, al, T.hb, N3l * 2 * oo, T.kpl)) ||
-                    (rc = tc_alloc(h, al, T.h2a, N3l * oo, T.kpo)) || (rc = tc_alloc(h, al, T.h2b, N3l * 2 * vv, T.kpo)))
+                    (!pack_hh && ((rc = tc_alloc(h, al, T.ha, N3l * oo, T.kpl)) || (rc = tc_alloc(h, al, T.hb, N3l * 2 * oo, T.kpl)) ||
+                                  (rc = tc_alloc(h, al, T.h2a, N3l * oo, T.kpo)) || (rc = tc_alloc(h, al, T.h2b, N3l * 2 * vv, T.kpo)))))
                     return rc;
+                if (pack_hh) {
+                    const int kplt = (int)((2 * nlt_oo + T.KQ - 1) / T.KQ * T.KQ);
+                    for (int d = 0; d < 2; ++d) for (int e = 0; e < 2; ++e) {
+                        const long long blocks = class_blocks(pair_class(d, e));
+                        const long long nmn = d ? nlt_oo : oo, nab = d ? nlt_vv : vv;
+                        if (blocks * nmn * (e ? nlt_vv : vv) && (rc = tc_alloc(h, al, T.xb[d][e], blocks * 2 * nmn, e ? T.kplp : T.kpl)))
+                            return rc;
+                        if (blocks * nab * (e ? nlt_oo : oo) && (rc = tc_alloc(h, al, T.wb[d][e], blocks * 2 * nab, e ? kplt : T.kpo)))
+                            return rc;
+                    }
+                    for (int e = 0; e < 2; ++e) {
+                        if (e && !nlt_oo) continue;
+                        if ((rc = tc_alloc(h, al, T.wa[e], N3l * oo, e ? kplt : T.kpo))) return rc;
+                    }
+                }
                 T.lb_floats = T.lb.rows * T.kpl;
                 T.lb_sc_rows = T.lb.sc_rows;
             }
@@ -1279,7 +1320,57 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
             if (tcp) h->seq.back().mode = 1;
         }
     }
-    for (TcSet& T : sets) {
+    // tau rows [S][ke][ki](ij) of the ladder's (and the packed X's) A operand
+    std::vector<long long> so_lad;
+    for (int S = 0; S < N; ++S) for (int ke = 0; ke < N; ++ke) for (int ki = 0; ki < N; ++ki)
+        so_lad.push_back(blk(S2, ki, kg.k4(S, 0, ki), ke));
+    if (pack_hh) for (TcSet& T : sets) {
+        h->cur_oz = T.oz;
+        // X packed: batches (km <= kn), rows (ki, ij) of tau (the ladder's operand), columns
+        // the (m n) list of <mn||ef> (constant), K = (ke, ef list); mirror Whh(nm) = -Whh(mn)
+        for (int e = 0; e < 2; ++e) {
+            const std::vector<int>& efl = e ? vv_lt : vv_full;
+            if (efl.empty()) continue;
+            const TcBuf& A = e ? T.lap : T.la;
+            if ((rc = add_embed(h, al, B_TAU, A, 0, (int)oo, (int)efl.size(), so_lad, tab({{(int)oo, vv}}), efl, false)))
+                return rc;
+            for (int d = 0; d < 2; ++d) {
+                const std::vector<int>& mnl = d ? oo_lt : oo_full;
+                const PairClass c = pair_class(d, e);
+                if (mnl.empty() || c.pq.empty()) continue;
+                std::vector<long long> so, oc, oc2;
+                std::vector<int> ra, rb, cnt, cc, cc2, srow;
+                size_t nch = 0;
+                for (const auto& x : c.in) nch = std::max(nch, x.size());
+                int used = 0;
+                for (size_t q = 0; q < c.pq.size(); ++q) {
+                    const int km = c.pq[q].first, kn = c.pq[q].second, S = kg.k4(km, kn, 0);
+                    for (int ke : c.in[q]) so.push_back(blk(S2, km, kn, ke));
+                    for (size_t z = 0; z < nch; ++z) {
+                        const int zz = (int)std::min(z, c.in[q].size() - 1);
+                        ra.push_back((int)((((long long)S * N + c.in[q][(size_t)zz]) * N) * oo));
+                        rb.push_back((int)((used + zz) * 2 * (long long)mnl.size()));
+                    }
+                    used += (int)c.in[q].size();
+                    cnt.push_back((int)c.in[q].size());
+                    for (int ki = 0; ki < N; ++ki) for (int ij = 0; ij < (int)oo; ++ij) {
+                        oc.push_back(blk(Soooo, km, kn, ki) + ij);
+                        oc2.push_back(blk(Soooo, kn, km, ki) + ij);
+                    }
+                }
+                for (int x : mnl) {
+                    srow.push_back(x * (int)vv);
+                    cc.push_back(x * (int)oo);
+                    cc2.push_back(swap_pair(x, o) * (int)oo);
+                }
+                if ((rc = add_embed(h, al, B_OOVV, T.xb[d][e], 1, (int)mnl.size(), (int)efl.size(), so, srow, efl, true)) ||
+                    (rc = add_tc(h, al, A, T.xb[d][e], B_WHH, (int)(N * oo), (int)(2 * mnl.size()), (int)c.pq.size(),
+                                 (int)nch, ra, rb, oc, cc, 1.0, 3, cnt, oc2, cc2)))
+                    return rc;
+            }
+        }
+    }
+    if (!pack_hh) for (TcSet& T : sets) {
         h->cur_oz = T.oz;
         // X on tensor cores, one batch per momentum sum S = km + kn = ki + kj:
         // rows (km, mn) of <mn||ef> (constant operand), columns (ki, ij) of tau, K = (ke, ef)
@@ -1342,7 +1433,61 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
             if (tcp) h->seq.back().mode = 1;
         }
     }
-    for (TcSet& T : sets) {
+    if (pack_hh) for (TcSet& T : sets) {
+        h->cur_oz = T.oz;
+        // R2 += tau_mn^ab Whh_mnij packed: batches (ka <= kb), rows (ki, ij) of Whh^T, columns
+        // the (a b) list of tau, K = (km, mn list); mirror R2(ba) = -R2(ab)
+        for (int e = 0; e < 2; ++e) {
+            const std::vector<int>& mnl = e ? oo_lt : oo_full;
+            if (mnl.empty()) continue;
+            // Whh^T of the summed pairs of this class, [S][km][ki](ij)
+            std::vector<long long> so;
+            std::vector<int> at((size_t)N * N, -1), scol;
+            int nblk = 0;
+            for (int S = 0; S < N; ++S) for (int km = 0; km < N; ++km) {
+                const int kn = kg.k4(S, 0, km);
+                if (!(e ? km == kn : km < kn)) continue;
+                at[(size_t)S * N + km] = nblk;
+                for (int ki = 0; ki < N; ++ki, ++nblk) so.push_back(blk(Soooo, km, kn, ki));
+            }
+            if (so.empty()) continue;
+            for (int x : mnl) scol.push_back(x * (int)oo);
+            if ((rc = add_embed(h, al, B_WHH, T.wa[e], 0, (int)oo, (int)mnl.size(), so, tab({{(int)oo, 1}}), scol, false)))
+                return rc;
+            for (int d = 0; d < 2; ++d) {
+                const std::vector<int>& abl = d ? vv_lt : vv_full;
+                const PairClass c = pair_class(d, e);
+                if (abl.empty() || c.pq.empty()) continue;
+                std::vector<long long> sb, oc, oc2;
+                std::vector<int> ra, rb, cnt, cc2, mcol;
+                size_t nch = 0;
+                for (const auto& x : c.in) nch = std::max(nch, x.size());
+                int used = 0;
+                for (size_t q = 0; q < c.pq.size(); ++q) {
+                    const int ka = c.pq[q].first, kb = c.pq[q].second, S = kg.k4(ka, kb, 0);
+                    for (int km : c.in[q]) sb.push_back(blk(S2, km, kg.k4(S, 0, km), ka));
+                    for (size_t z = 0; z < nch; ++z) {
+                        const int zz = (int)std::min(z, c.in[q].size() - 1);
+                        ra.push_back(at[(size_t)S * N + c.in[q][(size_t)zz]] * (int)oo);
+                        rb.push_back((int)((used + zz) * 2 * (long long)abl.size()));
+                    }
+                    used += (int)c.in[q].size();
+                    cnt.push_back((int)c.in[q].size());
+                    for (int ki = 0; ki < N; ++ki) for (int ij = 0; ij < (int)oo; ++ij) {
+                        oc.push_back(blk(S2, ki, kg.k4(S, 0, ki), ka) + ij * vv);
+                        oc2.push_back(blk(S2, ki, kg.k4(S, 0, ki), kb) + ij * vv);
+                    }
+                }
+                for (int x : abl) cc2.push_back(swap_pair(x, v));
+                for (int x : mnl) mcol.push_back(x * (int)vv);
+                if ((rc = add_embed(h, al, B_TAU, T.wb[d][e], 1, (int)abl.size(), (int)mnl.size(), sb, abl, mcol, false)) ||
+                    (rc = add_tc(h, al, T.wa[e], T.wb[d][e], B_R2, (int)(N * oo), (int)(2 * abl.size()), (int)c.pq.size(),
+                                 (int)nch, ra, rb, oc, abl, 1.0, 3, cnt, oc2, cc2)))
+                    return rc;
+            }
+        }
+    }
+    if (!pack_hh) for (TcSet& T : sets) {
         h->cur_oz = T.oz;
         // R2 += 1/2 tau_mn^ab Whh_mnij on tensor cores, one batch per S = ki + kj:
         // rows (ki, ij) of Whh^T, columns (ka, ab) of tau, K = (km, mn)
@@ -1482,9 +1627,6 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
         // A' = tau rows [S = ki + kj][ke][ki](ij), columns the (e f) list; B' = W' formed
         // straight into its embedding for the blocks of one chunk at a time (the buffer
         // holds T.lb_floats per part), each chunk followed by its GEMM.
-        std::vector<long long> so_lad;
-        for (int S = 0; S < N; ++S) for (int ke = 0; ke < N; ++ke) for (int ki = 0; ki < N; ++ki)
-            so_lad.push_back(blk(S2, ki, kg.k4(S, 0, ki), ke));
         std::vector<int> full_vv = tab({{(int)vv, 1}}), lt_vv;
         for (int x = 0; x < v; ++x) for (int y = x + 1; y < v; ++y) lt_vv.push_back(x * v + y);
         const int M = (int)(N * oo);
@@ -1492,7 +1634,8 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
             const std::vector<int>& efl = diag_ef ? lt_vv : full_vv;
             if (efl.empty()) continue;
             const TcBuf& A = diag_ef ? T.lap : T.la;
-            if ((rc = add_embed(h, al, B_TAU, A, 0, (int)oo, (int)efl.size(), so_lad, tab({{(int)oo, vv}}), efl, false)))
+            if (!pack_hh &&                  // (the packed X has embedded it)
+                (rc = add_embed(h, al, B_TAU, A, 0, (int)oo, (int)efl.size(), so_lad, tab({{(int)oo, vv}}), efl, false)))
                 return rc;
             for (int diag_ab = 0; diag_ab < 2; ++diag_ab) {
                 const std::vector<int>& abl = diag_ab ? lt_vv : full_vv;
