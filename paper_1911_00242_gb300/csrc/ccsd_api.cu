@@ -1969,13 +1969,10 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
         h->seq.push_back(s1); h->seq.push_back(s2); h->seq.push_back(s3);
     }
     if (h->has_oz) {
-        // Ozaki iterations: below kFockGemms amplitudes (and in the pooled layout) the four
-        // GEMMs above become one fused double-float pass (fock_terms_df_kernel) over
-        // double-float copies and stay for FP64 iterations; above, the GEMMs on the copies,
-        // one of them moved to the tensor cores, are faster: fused against GEMMs 8.5 / 6.9 ms
-        // at 2x2x2/o8/v32 (34 M amplitudes), 0.83 / 0.85 at 2x2x1/o8/v30 (3.7 M), 0.18 / 0.25
-        // at 2x2x1/o6/v20 (0.9 M), 31 / 65 us at 3x1x1/o5/v13.
-        constexpr long long kFockGemms = 1LL << 22;
+        // Ozaki iterations: the four GEMMs above become one fused double-float pass
+        // (fock_terms_df_kernel) over double-float copies; the GEMMs stay for FP64 iterations
+        for (size_t i = fock_first; i < h->seq.size(); ++i)
+            if (h->seq[i].kind == 0) h->seq[i].mode = 1;
         if (!h->in32[B_OOOV] && (rc = add_df_copy(h, al, B_OOOV))) return rc;
         if (!pooled) {
             for (int b : {B_OOVV, B_OVVO}) if (!h->in32[b] && (rc = add_df_copy(h, al, b))) return rc;
@@ -1984,23 +1981,19 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
                 if (al.err) return al.err;
             }
             h->t2_df = h->dfc[B_T2];              // written by the tau pass
-        } else if (pool_b_bytes >= (long long)sizeof(df2) * h->n2) {
+        } else if (pooled && pool_b_bytes >= (long long)sizeof(df2) * h->n2) {
             h->t2_df = (df2*)pool_b;          // idle between the last tensor-core GEMM and the next residual
         } else {
             h->t2_df = (df2*)al.get((size_t)h->n2 * sizeof(df2));
         }
-        if (pooled || h->n2 < kFockGemms) {
-            for (size_t i = fock_first; i < h->seq.size(); ++i)
-                if (h->seq[i].kind == 0) h->seq[i].mode = 1;
-            h->t1_df = (df2*)al.get((size_t)h->n1 * sizeof(df2));
-            h->fvvpT_df = (df2*)al.get((size_t)h->bufsize[B_FVVP] * sizeof(df2));
-            h->foop_df = (df2*)al.get((size_t)h->bufsize[B_FOOP] * sizeof(df2));
-            if (al.err) return al.err;
-            Step s1{14, 0, h->cur_name, 0.0, 32.0 * (double)((h->dfc[B_T2] ? 0 : h->n2) + h->n1)};
-            Step s2{13, 0, h->cur_name, 8.0 * 2.0 * (o + v) * (double)h->n2, 16.0 * 4.0 * h->n2};
-            s1.mode = s2.mode = 5;
-            h->seq.push_back(s1); h->seq.push_back(s2);
-        }
+        h->t1_df = (df2*)al.get((size_t)h->n1 * sizeof(df2));
+        h->fvvpT_df = (df2*)al.get((size_t)h->bufsize[B_FVVP] * sizeof(df2));
+        h->foop_df = (df2*)al.get((size_t)h->bufsize[B_FOOP] * sizeof(df2));
+        if (al.err) return al.err;
+        Step s1{14, 0, h->cur_name, 0.0, 32.0 * (double)((h->dfc[B_T2] ? 0 : h->n2) + h->n1)};
+        Step s2{13, 0, h->cur_name, 8.0 * 2.0 * (o + v) * (double)h->n2, 16.0 * 4.0 * h->n2};
+        s1.mode = s2.mode = 5;
+        h->seq.push_back(s1); h->seq.push_back(s2);
     }
     h->seq.push_back({4, 0, "antisym_R2", 0.0, 16.0 * 3.0 * h->n2});
     h->cur_oz = true;
