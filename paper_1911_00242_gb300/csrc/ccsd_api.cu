@@ -2148,7 +2148,7 @@ void ensure_smem_attr(int which) {
             cudaFuncSetAttribute(tc_gemm_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES);
             break;
         default:
-            cudaFuncSetAttribute(oz_wprime_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+            cudaFuncSetAttribute(oz_wprime_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
             break;
     }
 }
@@ -2240,7 +2240,7 @@ void launch_step(ccsd_ctx* h, size_t si) {
                     if (h->in32[B_OVVV]) { z.ovvv32 = h->shadow[B_OVVV]; z.ovvv_df = nullptr; }
                     else { z.ovvv_df = h->dfc[B_OVVV]; z.ovvv32 = nullptr; }
                     z.t1 = h->buf[B_T1];
-                    oz_wprime_kernel<<<row_grid((long long)z.nblk * z.nab), 256, (size_t)(z.nef + 2 * z.o) * 16,
+                    oz_wprime_kernel<<<row_grid((long long)z.nblk * z.nab), 256, (size_t)(z.nef + 4 * z.o) * 16,
                                        h->st>>>(z);
                     ++h->launches;
                     break;
@@ -2261,10 +2261,13 @@ void launch_step(ccsd_ctx* h, size_t si) {
                 break;
             }
             case 13:  // Ozaki iterations: fused double-float Fock terms into ZR
-                fock_terms_df_kernel<<<ew_grid(h->n2), 256, 0, h->st>>>(FockTermsDfOp{
+            {
+                const FockTermsDfOp op{
                     h->buf[B_ZR], h->t2_df, h->t1_df, h->fvvpT_df, h->foop_df,
                     h->dfc[B_OOOV], h->in32[B_OOOV] ? h->shadow[B_OOOV] : nullptr,
-                    h->dfc[B_OVVV], h->in32[B_OVVV] ? h->shadow[B_OVVV] : nullptr, h->kb_of, N, o, v});
+                    h->dfc[B_OVVV], h->in32[B_OVVV] ? h->shadow[B_OVVV] : nullptr, h->kb_of, N, o, v};
+                fock_terms_df_kernel<<<ew_grid(op.units()), 256, 0, h->st>>>(op);
+            }
                 ++h->launches;
                 break;
             case 14:  // their double-float copies

@@ -456,63 +456,87 @@ __global__ void fock_terms_kernel(const FockTermsOp op) { op.run(blockIdx.x, gri
 // widen exactly):
 //   Zr += 1/2 sum_f t_ij^af F'^{bf}(kb) - 1/2 sum_r t_r^a(ka) <ij||rb>^*
 //       - 1/2 sum_n t_in^ab F'_nj(kj)   - 1/2 sum_c t_i^c(ki) <jc||ab>^*
-// One thread per Zr element; the four short sums accumulate in double-float and
-// Zr receives their FP64 sum.
-__device__ __forceinline__ void cfma_df(const df2& a, const df2& b, df2& c) {
-    c.x = fma(a.x, b.x, c.x); c.x = fma(-a.y, b.y, c.x);
-    c.y = fma(a.x, b.y, c.y); c.y = fma(a.y, b.x, c.y);
-}
-__device__ __forceinline__ void cfma_conjb_df(const df2& a, const df2& b, df2& c) {
-    c.x = fma(a.x, b.x, c.x); c.x = fma(a.y, b.y, c.x);
-    c.y = fma(-a.x, b.y, c.y); c.y = fma(a.y, b.x, c.y);
-}
+// One thread per pair (i, i + 1) of Zr elements, which share the vectors along b of F' and
+// ovvv (one element a thread read them twice as often from L2); the four short sums accumulate
+// in double-float, packed, and Zr receives their FP64 sum.  Bound by the FP32 pipe (4.8 ms of
+// packed arithmetic at 2x2x2/o8/v32): 7.1 ms against 8.5 ms with one element a thread and
+// scalar operations; loops not unrolled, since spills cost 0.6 ms.
 struct FockTermsDfOp {
     double2* Zr; const df2* t2; const df2* t1; const df2* fvvpT; const df2* foop;
     const df2* ooov; const float2* ooov32;       // double-float copy, or complex64 input
     const df2* ovvv; const float2* ovvv32;
     const int* kb_of; int N, o, v;
+    __host__ __device__ long long units() const {
+        return (long long)N * N * N * ((o + 1) / 2) * o * v * v;
+    }
     __device__ void run(long long vb, long long nvb) const {
-        const long long blk = (long long)o * o * v * v;
-        const long long total = (long long)N * N * N * blk;
+        const int oh = (o + 1) / 2;
+        const long long blk = (long long)o * o * v * v, ublk = (long long)oh * o * v * v;
+        const long long total = (long long)N * N * N * ublk;
         const long long vv = (long long)v * v, ov3 = (long long)o * v * vv, o3v = (long long)o * o * o * v;
         for (long long e = vb * blockDim.x + threadIdx.x; e < total; e += nvb * blockDim.x) {
-            const long long kk = e / blk;
-            int r = (int)(e % blk);
+            const long long kk = e / ublk;
+            int r = (int)(e % ublk);
             const int b = r % v; r /= v;
             const int a = r % v; r /= v;
-            const int j = r % o; const int i = r / o;
+            const int j = r % o;
+            const int i0 = 2 * (r / o), i1 = i0 + 1 < o ? i0 + 1 : i0;                // an odd last i is summed twice, written once
             const int ka = (int)(kk % N), kj = (int)((kk / N) % N), ki = (int)(kk / ((long long)N * N));
             const int kb = kb_of[kk];
             const df2* tb = t2 + kk * blk;
-            df2 p{df(0.f, 0.f), df(0.f, 0.f)}, q{df(0.f, 0.f), df(0.f, 0.f)};
-            const df2* trow = tb + (((long long)i * o + j) * v + a) * v;              // t_ij^{a f}
-            const df2* fcol = fvvpT + (long long)kb * v * v + b;                      // F'^{b f}(kb) at f v
-            for (int f = 0; f < v; ++f) cfma_df(trow[f], fcol[(long long)f * v], p);
-            const long long oo_off = kk * o3v + ((long long)i * o + j) * o * v + b;   // <ij||r b>
-            const df2* ta = t1 + (long long)ka * o * v + a;                           // t_r^a(ka)
-            for (int rr = 0; rr < o; ++rr) {
-                const df2 w = ooov32 ? ld_df2(ooov32 + oo_off + (long long)rr * v) : ooov[oo_off + (long long)rr * v];
-                cfma_conjb_df(ta[rr * v], w, q);
+            const int is[2] = {i0, i1};
+            dfp p[2], q[2], h[2];                                                     // F'vv, t1 and F'oo terms
+            const df2* trow[2]; const df2* ti[2]; const df2* tn[2];
+            long long oo_off[2];
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                const int i = is[g];
+                p[g] = q[g] = h[g] = dfp{0, 0};
+                trow[g] = tb + (((long long)i * o + j) * v + a) * v;                  // t_ij^{a f}
+                ti[g] = t1 + ((long long)ki * o + i) * v;                             // t_i^c(ki)
+                tn[g] = tb + ((long long)i * o * v + a) * v + b;                      // t_in^{ab}, n stride v^2
+                oo_off[g] = kk * o3v + ((long long)i * o + j) * o * v + b;            // <ij||r b>
             }
-            const df2* tn = tb + ((long long)i * o * v + a) * v + b;                  // t_in^{ab}, n stride v^2
-            const df2* fo = foop + (long long)kj * o * o + j;                         // F'_{n j}(kj)
-            for (int n = 0; n < o; ++n) cfma_df(tn[(long long)n * vv], fo[n * o], q);
+            const df2* fcol = fvvpT + (long long)kb * v * v + b;                      // F'^{b f}(kb) at f v
             const long long kjia = ((long long)kj * N + ki) * N + ka;
             const long long vb_off = kjia * ov3 + (long long)j * v * vv + (long long)a * v + b;   // <j c||a b>
-            const df2* ti = t1 + ((long long)ki * o + i) * v;                         // t_i^c(ki)
-            for (int c = 0; c < v; ++c) {
-                const df2 w = ovvv32 ? ld_df2(ovvv32 + vb_off + (long long)c * vv) : ovvv[vb_off + (long long)c * vv];
-                cfma_conjb_df(ti[c], w, q);
+#pragma unroll 1
+            for (int f = 0; f < v; ++f) {
+                const df2 w = ovvv32 ? ld_df2(ovvv32 + vb_off + (long long)f * vv) : ovvv[vb_off + (long long)f * vv];
+                const df2 u = fcol[(long long)f * v];
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    p[g] = cfma(trow[g][f], u, p[g]);
+                    q[g] = cfma_conj(ti[g][f], w, q[g]);
+                }
             }
-            const df2 d{p.x - q.x, p.y - q.y};
-            double2 z = Zr[e];
-            z.x += 0.5 * (double)d.x;
-            z.y += 0.5 * (double)d.y;
-            Zr[e] = z;
+            const df2* ta = t1 + (long long)ka * o * v + a;                           // t_r^a(ka)
+            const df2* fo = foop + (long long)kj * o * o + j;                         // F'_{n j}(kj)
+#pragma unroll 1
+            for (int n = 0; n < o; ++n) {
+                const df2 u = fo[n * o], s = ta[n * v];
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    const df2 w = ooov32 ? ld_df2(ooov32 + oo_off[g] + (long long)n * v) : ooov[oo_off[g] + (long long)n * v];
+                    h[g] = cfma(u, tn[g][(long long)n * vv], h[g]);
+                    q[g] = cfma_conj(s, w, q[g]);
+                }
+            }
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                if (g == 1 && i1 == i0) break;
+                const df2 x = dfp_split(p[g]), y = dfp_split(q[g]), w = dfp_split(h[g]);
+                const df2 d{x.x - (y.x + w.x), x.y - (y.y + w.y)};
+                double2* zp = Zr + kk * blk + (((long long)is[g] * o + j) * v + a) * v + b;
+                double2 z = *zp;
+                z.x += 0.5 * (double)d.x;
+                z.y += 0.5 * (double)d.y;
+                *zp = z;
+            }
         }
     }
 };
-__global__ void fock_terms_df_kernel(const FockTermsDfOp op) { op.run(blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(256, 2) fock_terms_df_kernel(const FockTermsDfOp op) { op.run(blockIdx.x, gridDim.x); }
 
 // Double-float copies for fock_terms_df_kernel: t2 (n2 elements) into t2_df; t1 into
 // t1_df, F'vv transposed per k into fvvpT_df, F'oo into foop_df.  Each element is split

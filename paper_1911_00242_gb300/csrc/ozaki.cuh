@@ -559,9 +559,8 @@ __global__ void oz_split_reduce(const OzArgs g)
 
 // ---------------------------------------------------------------- operand prep
 
-__device__ __forceinline__ uint32_t pack_bf16x2(uint16_t lo, uint16_t hi) {
-    return (uint32_t)lo | ((uint32_t)hi << 16);
-}
+// Upper halves of two FP32 patterns (BF16-exact values) as lo, hi.
+__device__ __forceinline__ uint32_t pack_bf16x2(uint32_t lo, uint32_t hi) { return __byte_perm(lo, hi, 0x7632); }
 
 __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long x) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -625,21 +624,18 @@ __device__ __forceinline__ void oz_embed_row(const OzEmbedArgs& e, const T* src,
     uint32_t* out0 = (uint32_t*)(e.sl + row0 * e.Kpad);
     const int kh = e.Kpad / 2;
     for (int k = tid; k < kh; k += nthr) {
-        uint16_t sr[OZ_MAX_SLICES], si[OZ_MAX_SLICES];
-        if (k < e.Kc) {
-            const double2 z = ldz(src + base + e.scol[k]);
-            oz_split(z.x, fx, e.slices, sr);
-            oz_split(e.conj ? -z.y : z.y, fx, e.slices, si);
-        } else {
-            for (int p = 0; p < e.slices; ++p) { sr[p] = 0; si[p] = 0; }
-        }
-        for (int p = 0; p < e.slices; ++p) {
+        const double2 z = k < e.Kc ? ldz(src + base + e.scol[k]) : make_double2(0.0, 0.0);
+        const OzDigits dr = oz_digits(z.x, fx, e.slices), di = oz_digits(e.conj ? -z.y : z.y, fx, e.slices);
+#pragma unroll
+        for (int p = 0; p < OZ_MAX_SLICES; ++p) {
+            if (p >= e.slices) break;
             uint32_t* o = out0 + (p * plane) / 2;
+            const uint32_t re = oz_digit(dr, p), im = oz_digit(di, p);
             if (e.mode == 0) {
-                o[k] = pack_bf16x2(sr[p], si[p]);
+                o[k] = pack_bf16x2(re, im);
             } else {
-                o[k] = pack_bf16x2(sr[p], si[p] ^ 0x8000u);      // (Re, -Im)
-                o[kh + k] = pack_bf16x2(si[p], sr[p]);           // (Im, Re)
+                o[k] = pack_bf16x2(re, im ^ 0x80000000u);        // (Re, -Im)
+                o[kh + k] = pack_bf16x2(im, re);                 // (Im, Re)
             }
         }
     }
@@ -681,10 +677,13 @@ struct OzWprimeArgs {
 };
 
 // The t1 terms are summed in double-float (FP32 pipe) from a double-float copy of
-// ovvv (or its complex64 values) and t1 values staged in shared memory.
+// ovvv (or its complex64 values) and t1 values staged in shared memory.  Bound by issue (72 %
+// of the slots): the t1 products are two thirds of the instructions, the slices most of the
+// rest.  2x2x2/o8/v32: 7.5 ms with scalar double-float and digit-by-digit slices, 6.6 ms with
+// the slices as bit fields and the widening off the FP64 pipe, 6.4 ms with packed products.
 template <typename TV, typename TO>
 __device__ void oz_wprime_row(const OzWprimeArgs& w, const TV* vvvv, const TO* ovvv, long long row,
-                              double2* vals, unsigned long long* red, df2* t1s) {
+                              double2* vals, unsigned long long* red, dfp* t1s) {
     const int N = w.N, o = w.o, v = w.v;
     const long long vv = (long long)v * v, v4 = vv * vv, ov3 = (long long)o * v * vv;
     const long long bi = row / w.nab;
@@ -697,35 +696,37 @@ __device__ void oz_wprime_row(const OzWprimeArgs& w, const TV* vvvv, const TO* o
     const TV* g0 = vvvv + blk_ab * v4 + (long long)ab * vv;
     const TO* pa = ovvv + blk_ba * ov3 + (long long)a * vv;         // + r v vv: ovvv[kb,ka,ke](r,a,.)
     const TO* pb = ovvv + blk_ab * ov3 + (long long)b * vv;         // ovvv[ka,kb,ke](r,b,.)
-    // t1s[r] = t_r^b(kb), t1s[o + r] = -t_r^a(ka)
+    // t1s[2 r, 2 r + 1] = (x, x), (-y, y) of t_r^b(kb), from 2 o on of -t_r^a(ka)
     __syncthreads();                              // t1s of the previous row is no longer read
     for (int r = threadIdx.x; r < 2 * o; r += blockDim.x) {
         if (r < o) {
-            t1s[r] = ld_df2(w.t1 + (long long)kb * o * v + (long long)r * v + b);
+            const df2 z = ld_df2(w.t1 + (long long)kb * o * v + (long long)r * v + b);
+            t1s[2 * r] = dfp_of(z.x, z.x);
+            t1s[2 * r + 1] = dfp_of(-z.y, z.y);
         } else {
             const df2 z = ld_df2(w.t1 + (long long)ka * o * v + (long long)(r - o) * v + a);
-            t1s[r] = df2{-z.x, -z.y};
+            t1s[2 * r] = dfp_of(-z.x, -z.x);
+            t1s[2 * r + 1] = dfp_of(z.y, -z.y);
         }
     }
     __syncthreads();
     unsigned long long m = 0;
     for (int ei = threadIdx.x; ei < w.nef; ei += blockDim.x) {
         const int ef = w.efl[ei];
-        df2 s{df(0), df(0)};
+        dfp acc{0, 0};
         for (int r = 0; r < o; ++r) {
             // + t_r^b(kb) ovvv[kb,ka,ke](r,a,e,f) - t_r^a(ka) ovvv[ka,kb,ke](r,b,e,f)
             const df2 p = ld_df2(pa + (long long)r * v * vv + ef);
-            const df2 tb = t1s[r];
-            s.x = fma(tb.x, p.x, s.x); s.x = fma(-tb.y, p.y, s.x);
-            s.y = fma(tb.x, p.y, s.y); s.y = fma(tb.y, p.x, s.y);
+            acc = fma(t1s[2 * r], dfp_of(p.x, p.y), acc);
+            acc = fma(t1s[2 * r + 1], dfp_of(p.y, p.x), acc);
             const df2 q = ld_df2(pb + (long long)r * v * vv + ef);
-            const df2 ta = t1s[o + r];
-            s.x = fma(ta.x, q.x, s.x); s.x = fma(-ta.y, q.y, s.x);
-            s.y = fma(ta.x, q.y, s.y); s.y = fma(ta.y, q.x, s.y);
+            acc = fma(t1s[2 * (o + r)], dfp_of(q.x, q.y), acc);
+            acc = fma(t1s[2 * (o + r) + 1], dfp_of(q.y, q.x), acc);
         }
+        const df2 s = dfp_split(acc);
         double2 g = ldz(g0 + ef);
-        g.x += (double)s.x;
-        g.y += (double)s.y;
+        g.x += f64_scaled(s.x.h) + f64_scaled(s.x.l);      // the widening stays off the FP64 pipe
+        g.y += f64_scaled(s.y.h) + f64_scaled(s.y.l);
         vals[ei] = g;
         const unsigned long long a = abs_bits(g.x), c = abs_bits(g.y);
         m = a > m ? a : m;
@@ -740,29 +741,26 @@ __device__ void oz_wprime_row(const OzWprimeArgs& w, const TV* vvvv, const TO* o
     uint32_t* out0 = (uint32_t*)(w.sl + row0 * w.Kpad);
     const int kh = w.Kpad / 2;
     for (int k = threadIdx.x; k < kh; k += blockDim.x) {
-        uint16_t sr[OZ_MAX_SLICES], si[OZ_MAX_SLICES];
-        if (k < w.nef) {
-            const double2 z = vals[k];
-            oz_split(z.x, fx, w.slices, sr);
-            oz_split(z.y, fx, w.slices, si);
-        } else {
-            for (int p = 0; p < w.slices; ++p) { sr[p] = 0; si[p] = 0; }
-        }
-        for (int p = 0; p < w.slices; ++p) {
+        const double2 z = k < w.nef ? vals[k] : make_double2(0.0, 0.0);
+        const OzDigits dr = oz_digits(z.x, fx, w.slices), di = oz_digits(z.y, fx, w.slices);
+#pragma unroll
+        for (int p = 0; p < OZ_MAX_SLICES; ++p) {
+            if (p >= w.slices) break;
             uint32_t* out = out0 + (p * plane) / 2;
-            out[k] = pack_bf16x2(sr[p], si[p] ^ 0x8000u);
-            out[kh + k] = pack_bf16x2(si[p], sr[p]);
+            const uint32_t re = oz_digit(dr, p), im = oz_digit(di, p);
+            out[k] = pack_bf16x2(re, im ^ 0x80000000u);
+            out[kh + k] = pack_bf16x2(im, re);
         }
     }
     __syncthreads();                                  // vals[] is rewritten by the next row
 }
 
 // One CTA per output row pair; dynamic shared memory holds the row's nef values.
-__global__ void oz_wprime_kernel(const OzWprimeArgs w)
+__global__ void __launch_bounds__(256, 4) oz_wprime_kernel(const OzWprimeArgs w)
 {
-    extern __shared__ double2 vals[];             // [nef] values, then [2 o] t1 values (df2)
+    extern __shared__ double2 vals[];             // [nef] values, then [2 o][2] t1 values (dfp)
     __shared__ unsigned long long red[32];
-    df2* t1s = (df2*)(vals + w.nef);
+    dfp* t1s = (dfp*)(vals + w.nef);
     const long long rows = (long long)w.nblk * w.nab;
     for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
         if (w.vvvv32) {
