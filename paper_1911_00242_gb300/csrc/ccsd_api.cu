@@ -889,7 +889,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
     // class of outputs and one of summed pairs, each (p < q) with all orbital pairs or (p = q)
     // with the ordered ones, a quarter of the products and of the tau operand.  The classes
     // are up to four launches instead of one, so small problems (below kPackHhFlops) and the
-    // pooled layout keep the full sums.  At 2x2x2/o8/v32 the two steps take 3.8 ms instead of
+    // pooled layout keep the full sums.  At 2x2x2/o8/v32 the two steps take 3.6 ms instead of
     // 8.2 (Ozaki) and 1.6 instead of 2.1 (mixed).
     constexpr double kPackHhFlops = 4e9;
     bool pack_hh = tcp && 8.0 * N * N * N * (double)N * oo * oo * vv >= kPackHhFlops;   // and not pooled (below)
@@ -2541,7 +2541,7 @@ int run_residual(ccsd_ctx* h) {
 // the group:
 //   * contractions: zgemm_grouped_kernel, a persistent CTA set striding a
 //     [member][split][batch][tile] work list, with one tile shape per step (picked by
-//     an autotuner in the batched form); split-K reductions grouped the same way;
+//     an autotuner in the batched form); a tile's last split adds its partials;
 //   * tensor-core contractions: tc_gemm_grouped_kernel, one CTA per tile of every
 //     member, each member's tensor maps and arguments read from global memory;
 //   * elementwise and row-wise steps (tau, copies, permutations, operand embedding,

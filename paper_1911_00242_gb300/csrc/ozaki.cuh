@@ -39,7 +39,7 @@
 // accumulators p + q (TMEM columns 64 d).  Each staged byte thus feeds s / 2 products
 // on average (one in a layout that stages one pair at a time), which keeps the shared
 // memory's bandwidth, shared by the copies and the MMA operand reads, from bounding
-// the tensor pipe.  Warp 0 / lane 0 issues the TMA loads, warp 1 / lane 0 the MMAs;
+// the tensor pipe.  Warp 0 / lane 0 issues the TMA loads, an elected lane of warp 1 the MMAs;
 // warps 2..17 promote each diagonal's window as soon as its last product is in
 // (diagonal p is complete once slice p of A is done in the window's last K slice) and
 // keep (hi, lo) of 16 columns of one TMEM lane quarter in registers.  A launch with

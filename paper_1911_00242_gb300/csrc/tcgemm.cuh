@@ -28,8 +28,8 @@
 // One CTA computes one 128 x 256 tile (cta_group::1, M = 128, N = 256), 10 warps:
 //   warp 0 / lane 0 issues TMA loads into a 4-stage ring (48 KiB per stage: a K
 //   slice of 16 of both parts of A' and B', 64-byte swizzle),
-//   warp 1 / lane 0 issues 6 MMAs (K = 8 each: two K steps of the three products)
-//   per stage into TMEM buffer (segment & 1), warps 2..9 promote segments and run
+//   warp 1 (one elected lane) issues 6 MMAs (K = 8 each: two K steps of the three
+//   products) per stage into TMEM buffer (segment & 1), warps 2..9 promote segments and run
 //   the epilogue.
 // Every mbarrier wait is bounded; on timeout the CTA records an error code,
 // stops issuing, waits (bounded) for its copies and MMAs in flight, frees its
@@ -201,7 +201,7 @@ __device__ __forceinline__ void tc_commit_warp(uint32_t bar) {
 // One 128 x 256 output tile of one batch: C[rows m][cols n] += alpha * sum over the
 // batch's chunks, K stages and split terms of A'(rows) . B'(rows)^T.
 //   warp 0, lane 0: TMA producer into a TC_STAGES ring (full/empty mbarriers)
-//   warp 1, lane 0: MMA issuer; segment g of TC_PROMOTE_STAGES stages accumulates
+//   warp 1: MMA issuer (an elected lane); segment g of TC_PROMOTE_STAGES stages accumulates
 //                   in TMEM buffer g & 1, then commits to acc_full[g & 1]
 //   warps 2..9:     accumulator warps; warp w reads TMEM lanes 32 (w % 4) ..
 //                   (its rows) and columns 128 ((w - 2) / 4) .. + 127 of each
