@@ -38,6 +38,9 @@ constexpr int zg_warp_cols(const ZgShape& s) { return (s.bn / s.tn < 8 ? s.bn / 
 
 constexpr int kZgUnit = 32;            // K terms of one split unit (ZG_KU of the kernel)
 constexpr int kZgMaxSplit = 64;
+// Most partials of one launch (16 bytes each: 1 GiB).  Without the bound 3x3x3/o8/v24 took 4 GB
+// of workspace beside 290 GB in use; at 2x2x2/o8/v32 the chosen splits need half of it.
+constexpr long long kZgMaxPartials = 1LL << 26;
 constexpr long long kZgFp32Chain = 8192;   // longest FP32 partial sum of the mixed form
 
 struct ZgChoice { int shape, nsplit; double seconds; };
@@ -110,6 +113,7 @@ inline ZgChoice zg_choose(int arith, int M, int N, int K, long long nchunk, long
         static const int kSplits[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
         for (int want : kSplits) {
             const long long ns = std::max<long long>(lo, std::min<long long>(want, units));
+            if (ns > lo && ns * nbatch * M * N > kZgMaxPartials) continue;
             const double t = zg_estimate(arith, i, (int)ns, M, N, K, nchunk, nbatch, c128, sms);
             if (t < best.seconds) best = ZgChoice{i, (int)ns, t};
         }
