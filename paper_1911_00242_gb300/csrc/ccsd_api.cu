@@ -2403,12 +2403,15 @@ struct HazardMap {
 struct GraphBuilder {
     cudaGraph_t g = nullptr;
     cudaStream_t cs = nullptr;
+    bool open = false;            // a piece's capture has begun and not ended
     cudaError_t err = cudaSuccess;
     GraphBuilder() {
         err = cudaGraphCreate(&g, 0);
         if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     }
     ~GraphBuilder() {
+        cudaGraph_t same = nullptr;
+        if (open) cudaStreamEndCapture(cs, &same);      // an exception left the piece
         if (g) cudaGraphDestroy(g);
         if (cs) cudaStreamDestroy(cs);
     }
@@ -2421,6 +2424,7 @@ struct GraphBuilder {
         if (err != cudaSuccess) return ends;
         err = cudaStreamBeginCaptureToGraph(cs, g, pre.data(), nullptr, pre.size(), cudaStreamCaptureModeThreadLocal);
         if (err != cudaSuccess) return ends;
+        open = true;
         fn(cs);
         cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
         const cudaGraphNode_t* nodes = nullptr;
@@ -2429,6 +2433,7 @@ struct GraphBuilder {
         if (err == cudaSuccess) ends.assign(nodes, nodes + n);
         cudaGraph_t same = nullptr;
         const cudaError_t e2 = cudaStreamEndCapture(cs, &same);
+        open = false;
         if (err == cudaSuccess) err = e2;
         return ends;
     }
@@ -2459,8 +2464,10 @@ std::vector<int> first_n(int n) {
 // Captures the residual (and, norm set, max|R| and the host copies) into a graph.
 int build_graph(ccsd_ctx* h, bool norm, cudaGraphExec_t* out, long long* launches) {
     GraphBuilder gb;
-    const cudaStream_t own = h->st;
-    const long long before = h->launches;
+    struct Own {                  // the handle's stream and launch count, put back on every way out
+        ccsd_ctx* h; cudaStream_t st; long long launches;
+        ~Own() { h->st = st; h->launches = launches; }
+    } own{h, h->st, h->launches};
     h->st = gb.cs;
     HazardMap hz;
     std::vector<std::vector<cudaGraphNode_t>> ends(h->seq.size());
@@ -2478,9 +2485,7 @@ int build_graph(ccsd_ctx* h, bool norm, cudaGraphExec_t* out, long long* launche
         all.push_back(gb.piece(GraphBuilder::join(ends, pre), [&](cudaStream_t) { launch_norm(h); }));
         gb.piece(GraphBuilder::join(all, first_n((int)all.size())), [&](cudaStream_t) { rc = copy_host_words(h, true); });
     }
-    h->st = own;
-    *launches = h->launches - before;
-    h->launches = before;
+    *launches = h->launches - own.launches;
     const int frc = gb.finish(out);
     return rc ? rc : frc;
 }
@@ -2495,14 +2500,28 @@ bool use_graph(const ccsd_ctx* h) {
     return s == cudaStreamCaptureStatusNone;
 }
 
-int replay_graph(ccsd_ctx* h, int which) {
+// Replays the residual, built on its first use.  A graph that cannot be had (no memory on the
+// host or the device, a refused instantiation) is no error: *ran stays false, and this call and
+// the handle's later ones launch the steps one by one.
+int replay_graph(ccsd_ctx* h, int which, bool* ran) {
     const int w = gemm_arith(h);
     if (!h->graph[which][w]) {
-        const int rc = build_graph(h, which == 0, &h->graph[which][w], &h->graph_launches[which][w]);
-        if (rc) return rc;
+        int rc;
+        try {
+            rc = build_graph(h, which == 0, &h->graph[which][w], &h->graph_launches[which][w]);
+        } catch (const std::bad_alloc&) {
+            rc = CCSD_ERR_OOM;
+        }
+        if (rc) {
+            cudaGetLastError();
+            g_errbuf[0] = 0;
+            h->graphable = false;
+            return 0;
+        }
     }
     CK(cudaGraphLaunch(h->graph[which][w], h->st));
     h->launches += h->graph_launches[which][w];
+    *ran = true;
     return 0;
 }
 
@@ -3410,9 +3429,9 @@ size_t footprint_bytes(const ccsd_config* c, const bool* on_dev, int int_dtype, 
 // copied into pinned host memory; returns without waiting.
 int iter_begin(ccsd_ctx* h) {
     int rc;
-    if (use_graph(h)) {
-        if ((rc = replay_graph(h, 0))) return rc;
-    } else {
+    bool ran = false;
+    if (use_graph(h) && (rc = replay_graph(h, 0, &ran))) return rc;
+    if (!ran) {
         if ((rc = run_residual_async(h))) return rc;
         launch_norm(h);
         if ((rc = copy_host_words(h, true))) return rc;
@@ -4105,13 +4124,16 @@ int ccsd_residual(ccsd_t h, const void* t1, const void* t2, void* r1, void* r2) 
         op_kernel<PairCopyOp><<<ew_grid(h->n1 + h->n2), 256, 0, h->st>>>(in);
         double2* amp[2] = {h->buf[B_T1], h->buf[B_T2]};
         h->buf[B_T1] = h->stage; h->buf[B_T2] = h->stage + h->n1;
-        int rc = replay_graph(h, 1);
+        bool ran = false;
+        const int rc = replay_graph(h, 1, &ran);
         h->buf[B_T1] = amp[0]; h->buf[B_T2] = amp[1];
         if (rc) return rc;
-        op_kernel<PairCopyOp><<<ew_grid(h->n1 + h->n2), 256, 0, h->st>>>(back);
-        h->launches += 2;
-        CK(cudaGetLastError());
-        return check_tc_err(h);
+        if (ran) {
+            op_kernel<PairCopyOp><<<ew_grid(h->n1 + h->n2), 256, 0, h->st>>>(back);
+            h->launches += 2;
+            CK(cudaGetLastError());
+            return check_tc_err(h);
+        }
     }
     double2* save[4] = {h->buf[B_T1], h->buf[B_T2], h->buf[B_R1], h->buf[B_R2]};
     h->buf[B_T1] = (double2*)t1; h->buf[B_T2] = (double2*)t2;
