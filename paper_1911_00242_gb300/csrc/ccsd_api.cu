@@ -2461,8 +2461,19 @@ std::vector<int> first_n(int n) {
     return v;
 }
 
+// Lets this thread make the calls that a capture under way on another stream would forbid it (and
+// be broken by): building a graph needs some of them, and none touches that capture's streams.
+struct CaptureRelaxed {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CaptureRelaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~CaptureRelaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    CaptureRelaxed(const CaptureRelaxed&) = delete;
+    CaptureRelaxed& operator=(const CaptureRelaxed&) = delete;
+};
+
 // Captures the residual (and, norm set, max|R| and the host copies) into a graph.
 int build_graph(ccsd_ctx* h, bool norm, cudaGraphExec_t* out, long long* launches) {
+    CaptureRelaxed relaxed;
     GraphBuilder gb;
     struct Own {                  // the handle's stream and launch count, put back on every way out
         ccsd_ctx* h; cudaStream_t st; long long launches;
