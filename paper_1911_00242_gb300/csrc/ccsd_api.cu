@@ -129,6 +129,10 @@ struct TcPlan {
 
 }  // namespace
 
+// Who iterates a handle: its caller; a batch (grouped launches from the batch's own graph); the
+// serving loop (grouped launches, and iterations of its own in the Ozaki arithmetic).
+enum class HandleUse { own, batch, served };
+
 struct ccsd_ctx {
     ccsd_config cfg;
     KGrid kg;
@@ -203,7 +207,8 @@ struct ccsd_ctx {
     // Problems of up to kGraphElems replay the residual as a CUDA graph whose edges are the
     // plan's data dependencies.  [0]: on the handle's amplitudes, with max|R| and the error
     // word copied to the host; [1]: on `stage` (ccsd_residual's arguments are copied in and out).
-    bool graphable = false;
+    HandleUse use = HandleUse::own;
+    bool graphable[ZG_ARITH] = {};
     double2* stage = nullptr;        // [t1 | t2]
     cudaGraphExec_t graph[2][ZG_ARITH] = {};
     long long graph_launches[2][ZG_ARITH] = {};
@@ -241,11 +246,17 @@ struct Alloc {
     ccsd_ctx* h;
     int err = 0;
     bool dry = false;     // plan validation only: no device memory, no copies
+    uintptr_t next = 256;                 // dry: every buffer has an address of its own
+    void* place(size_t bytes) {
+        void* p = (void*)next;
+        next += (bytes + 255) / 256 * 256 + 256;
+        return p;
+    }
     void* get(size_t bytes) {
         if (err) return nullptr;
         void* p = nullptr;
         if (bytes == 0) bytes = 16;
-        if (dry) { h->owned_bytes += bytes; return (void*)(uintptr_t)256; }
+        if (dry) { h->owned_bytes += bytes; return place(bytes); }
         cudaError_t e = cudaMalloc(&p, bytes);
         if (e != cudaSuccess) { cudaGetLastError(); err = (e == cudaErrorMemoryAllocation) ? CCSD_ERR_OOM : CCSD_ERR_CUDA; return nullptr; }
         h->owned.push_back(p);
@@ -298,7 +309,10 @@ const int kSMs = 152;
 // 2x2x2/o8/v32 (n2 = 34 M) each step fills the chip (87.9 and 87.8 ms), and ccsd_residual's
 // arguments, copied in and out, cost memory and time.
 const long long kGraphElems = 1LL << 24;
-const size_t kGraphWorkBytes = 1ull << 30;    // most split workspace for a region per step
+const size_t kGraphWorkBytes = 1ull << 30;    // split partials (all steps') above which launches fill the chip
+// What a replay may take beside the step-by-step workspace (the split partials of steps that run
+// side by side, and the staged amplitudes): at most half of the handle's other memory.
+const size_t kGraphShare = 2;
 const int kRedBlocks = kSMs * 4;    // blocks of the reductions (max|R|, inner products, energy)
 
 // Momentum pairs (ka <= kb) whose ladder W' blocks one slab holds: as many as fit in
@@ -2504,7 +2518,7 @@ int build_graph(ccsd_ctx* h, bool norm, cudaGraphExec_t* out, long long* launche
 // True if this call replays the graph: problems up to its size, except while tracing and while the
 // caller captures the handle's stream (the launches then become part of that capture).
 bool use_graph(const ccsd_ctx* h) {
-    if (!h->graphable || h->trace) return false;
+    if (!h->graphable[gemm_arith(h)] || h->trace) return false;
     if (!h->st) return true;
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(h->st, &s) != cudaSuccess) { cudaGetLastError(); return false; }
@@ -2526,7 +2540,7 @@ int replay_graph(ccsd_ctx* h, int which, bool* ran) {
         if (rc) {
             cudaGetLastError();
             g_errbuf[0] = 0;
-            h->graphable = false;
+            for (bool& g : h->graphable) g = false;
             return 0;
         }
     }
@@ -3238,6 +3252,96 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Steps that split their sums and what they need of a workspace.
+struct Region { size_t step, size; long long* off; };
+
+// Places the regions of one workspace, each as low as it fits: two of them may share elements
+// only if the graph orders their steps (before[i][j]: step j ends before step i starts).
+size_t place_regions(const std::vector<Region>& rs, const std::vector<std::vector<bool>>& before) {
+    size_t top = 0;
+    for (size_t i = 0; i < rs.size(); ++i) {
+        size_t off = 0;
+        for (bool moved = true; moved;) {
+            moved = false;
+            for (size_t j = 0; j < i; ++j) {
+                const size_t oj = (size_t)*rs[j].off, ej = oj + rs[j].size;
+                if (before[rs[i].step][rs[j].step] || off >= ej || off + rs[i].size <= oj) continue;
+                off = ej;
+                moved = true;
+            }
+        }
+        *rs[i].off = (long long)off;
+        top = std::max(top, off + rs[i].size);
+    }
+    return top;
+}
+
+// Decides in which arithmetics this handle's residual is replayed as a graph and lays out the
+// split workspaces for it: steps that the graph may run side by side get disjoint partials and
+// counters (one arithmetic is active at a time, so the arithmetics share the space).  Where a
+// replay would take more than its share of memory, and in handles that never replay (batch
+// members; grouped iterations of served solves), every step uses the front of one workspace,
+// one after another.  The regions a graph needs are some 1.0 to 1.3 times the largest step's: a
+// region each, as large as their sum, took 273 MB instead of 133 MB at 2x2x1/o6/v20 (FP64).
+void lay_out_graph(ccsd_ctx* h, size_t& work_need) {
+    if (h->use == HandleUse::batch || h->n2 > kGraphElems) return;
+    const int fp32 = h->fp32, oz_on = h->oz_on;
+    const long long oz_need = h->oz_work_elems;
+    size_t work = work_need, ozw = (size_t)oz_need, cnt = h->cnt_need;
+    size_t partials = 0;                  // of all steps, in the arithmetic that has most
+    bool any = false;
+    for (int w = 0; w < ZG_ARITH; ++w) {
+        if ((w == ZG_FP32 && h->cfg.precision != CCSD_MIXED) || (w == ZG_DF && !h->has_oz)) continue;
+        if (h->use == HandleUse::served && w != ZG_DF) continue;
+        h->fp32 = w == ZG_FP32;
+        h->oz_on = w == ZG_DF;
+        const size_t n = h->seq.size();
+        HazardMap hz;
+        std::vector<std::vector<bool>> before(n, std::vector<bool>(n, false));
+        std::vector<Region> rw, rc, ro;
+        for (size_t i = 0; i < n; ++i) {
+            const Step& st = h->seq[i];
+            if (!step_active(h, st)) continue;
+            for (int p : hz.add((int)i, step_access(h, st))) {
+                before[i][(size_t)p] = true;
+                for (size_t j = 0; j < (size_t)p; ++j) if (before[(size_t)p][j]) before[i][j] = true;
+            }
+            if (st.kind == 0) {
+                GemmPlan& g = h->gemms[st.idx];
+                GemmVar& v = g.var[w];
+                if (v.nsplit < 2) continue;
+                rw.push_back({i, (size_t)v.nsplit * g.args.nbatch * g.args.M * g.args.N, &v.work_off});
+                rc.push_back({i, (size_t)v.blocks, &v.cnt_off});
+            } else if (st.kind == 6 && h->tcs[st.idx].oz && h->tcs[st.idx].z.nsplit > 1) {
+                TcPlan& t = h->tcs[st.idx];
+                ro.push_back({i, (size_t)t.z.nsplit * t.z.nbatch * t.z.M * (t.z.Nr / 2), &t.work_off});
+            }
+        }
+        size_t sum = 0;
+        for (const auto* rs : {&rw, &ro}) for (const Region& r : *rs) sum += r.size * 16;
+        partials = std::max(partials, sum);
+        work = std::max(work, place_regions(rw, before));
+        cnt = std::max(cnt, place_regions(rc, before));
+        ozw = std::max(ozw, place_regions(ro, before));
+        h->graphable[w] = any = true;
+    }
+    h->fp32 = fp32;
+    h->oz_on = oz_on;
+    if (!any) return;
+    const size_t base = h->owned_bytes + (work_need + (size_t)oz_need) * 16;
+    const size_t more = (work - work_need + ozw - (size_t)oz_need) * 16 +
+                        (h->use == HandleUse::own ? (size_t)(h->n1 + h->n2) * 16 : 0);
+    if (partials > kGraphWorkBytes || more > base / kGraphShare) {
+        for (bool& g : h->graphable) g = false;
+        for (GemmPlan& g : h->gemms) for (GemmVar& v : g.var) v.work_off = v.cnt_off = 0;
+        for (TcPlan& t : h->tcs) t.work_off = 0;
+        return;
+    }
+    work_need = work;
+    h->cnt_need = cnt;
+    h->oz_work_elems = (long long)ozw;
+}
+
 // Fills a handle whose cfg, grid and sizes are set: inputs (device ones borrowed, host
 // ones copied), amplitudes, work buffers, DIIS history, Fock diagonals, the residual
 // plan and its tables.  With al.dry nothing is allocated, copied or launched and
@@ -3252,11 +3356,11 @@ int setup_handle(ccsd_ctx* h, Alloc& al, const void* const* ins, const bool* on_
         const size_t bytes = (size_t)sizes[i] * (c64 ? 8 : 16);
         void* d = nullptr;
         if (on_dev[i]) {
-            d = al.dry ? (void*)(uintptr_t)256 : const_cast<void*>(ins[i]);
+            d = al.dry ? al.place(bytes) : const_cast<void*>(ins[i]);
         } else if (i == 8 && vvvv_on_host) {
             // vvvv read in place from host memory (mapped, pinned): no device copy
             if (al.dry) {
-                d = (void*)(uintptr_t)256;
+                d = al.place(bytes);
             } else {
                 void* hp = const_cast<void*>(ins[i]);
                 const int r = host_register(hp, bytes);
@@ -3350,41 +3454,8 @@ int setup_handle(ccsd_ctx* h, Alloc& al, const void* const* ins, const bool* on_
     size_t work_need = 0;
     int rc = build_plan(h, al, work_need);
     if (rc) return rc;
-    if (h->n2 <= kGraphElems) {
-        // the steps of a graph run side by side: they have their own split partials and counters (one
-        // arithmetic is active at a time, so the arithmetics share the space)
-        size_t work = 0, cnt = 0, ozw = 0;
-        auto lay_out = [&](bool assign) {
-            for (int w = 0; w < ZG_ARITH; ++w) {
-                size_t wk = 0, ct = 0;
-                for (GemmPlan& p : h->gemms) {
-                    GemmVar& v = p.var[w];
-                    if (v.nsplit < 2) continue;
-                    if (assign) { v.work_off = (long long)wk; v.cnt_off = (long long)ct; }
-                    wk += (size_t)v.nsplit * p.args.nbatch * p.args.M * p.args.N;
-                    ct += (size_t)v.blocks;
-                }
-                work = std::max(work, wk);
-                cnt = std::max(cnt, ct);
-            }
-            size_t oz = 0;
-            for (TcPlan& t : h->tcs) {
-                if (!t.oz || t.split_cap < 2) continue;
-                if (assign) t.work_off = (long long)oz;
-                oz += (size_t)t.split_cap * t.z.nbatch * t.z.M * (t.z.Nr / 2);
-            }
-            ozw = std::max(ozw, oz);
-        };
-        lay_out(false);
-        if ((work + ozw) * 16 <= kGraphWorkBytes) {
-            lay_out(true);
-            h->graphable = true;
-            work_need = std::max(work_need, work);
-            h->cnt_need = std::max(h->cnt_need, cnt);
-            h->oz_work_elems = std::max(h->oz_work_elems, (long long)ozw);
-        }
-    }
-    if (h->graphable) {
+    lay_out_graph(h, work_need);
+    if (h->graphable[gemm_arith(h)] && h->use == HandleUse::own) {      // (own: all its arithmetics or none)
         h->stage = dalloc(h->n1 + h->n2);
         if (!h->stage) return al.err;
     }
@@ -3422,16 +3493,45 @@ void init_ctx(ccsd_ctx* h, const ccsd_config* cfg) {
 }
 
 // Device bytes ccsd_create takes for this config, from a dry run of its setup; 0 on error.
-size_t footprint_bytes(const ccsd_config* c, const bool* on_dev, int int_dtype, bool vvvv_on_host = false) {
+size_t footprint_bytes(const ccsd_config* c, const bool* on_dev, int int_dtype, bool vvvv_on_host = false,
+                       HandleUse use = HandleUse::own) {
     ccsd_ctx* h = new (std::nothrow) ccsd_ctx();
     if (!h) return 0;
     init_ctx(h, c);
+    h->use = use;
     Alloc al{h};
     al.dry = true;
     const int rc = setup_handle(h, al, nullptr, on_dev, int_dtype, vvvv_on_host);
     const size_t b = rc ? 0 : h->owned_bytes;
     delete h;
     return b;
+}
+
+// ccsd_create, for the use the handle is put to.
+int create_handle(const ccsd_config* cfg, const ccsd_inputs* in, void* stream, HandleUse use, ccsd_t* out) {
+    ApiScope api_scope_;
+    if (!out) return CCSD_ERR_INVALID;
+    *out = nullptr;
+    if (!valid_cfg(cfg) || !in || (in->int_dtype != CCSD_C128 && in->int_dtype != CCSD_C64)) return CCSD_ERR_INVALID;
+    const void* ins[9] = {in->f_oo, in->f_vv, in->f_ov, in->oooo, in->ooov, in->oovv, in->ovvo, in->ovvv, in->vvvv};
+    for (const void* p : ins) if (!p) return CCSD_ERR_INVALID;
+    bool on_dev[9];
+    for (int i = 0; i < 9; ++i) on_dev[i] = is_device_ptr(ins[i]);
+    ccsd_ctx* h = new (std::nothrow) ccsd_ctx();
+    if (!h) return CCSD_ERR_OOM;
+    init_ctx(h, cfg);
+    h->use = use;
+    h->st = (cudaStream_t)stream;
+    Alloc al{h};
+    auto fail = [&](int code) { ccsd_destroy(h); return code; };
+    int rc = setup_handle(h, al, ins, on_dev, in->int_dtype, in->vvvv_on_host != 0);
+    if (rc) return fail(rc);
+    for (int ei : h->const_embeds) launch_embed(h, h->embeds[ei]);
+    if (cudaMallocHost(&h->norm_host, 2 * sizeof(double)) != cudaSuccess) { cudaGetLastError(); h->norm_host = nullptr; return fail(CCSD_ERR_OOM); }
+    if (cudaEventCreateWithFlags(&h->ev_norm, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); h->ev_norm = nullptr; return fail(CCSD_ERR_CUDA); }
+    if (cudaStreamSynchronize(h->st) != cudaSuccess) return fail(CCSD_ERR_CUDA);
+    *out = h;
+    return CCSD_OK;
 }
 
 }  // namespace
@@ -3592,7 +3692,7 @@ size_t request_bytes(const ccsd_config& c, const ccsd_inputs& in) {
     const void* ins[9] = {in.f_oo, in.f_vv, in.f_ov, in.oooo, in.ooov, in.oovv, in.ovvo, in.ovvv, in.vvvv};
     bool on_dev[9];
     for (int i = 0; i < 9; ++i) on_dev[i] = is_device_ptr(ins[i]);
-    return footprint_bytes(&c, on_dev, in.int_dtype, in.vvvv_on_host != 0);
+    return footprint_bytes(&c, on_dev, in.int_dtype, in.vvvv_on_host != 0, HandleUse::served);
 }
 
 // Fields that ccsd_poll reads (state, energy, iterations, max|R|) change only under S->mu.
@@ -3834,7 +3934,7 @@ void server_loop(ccsd_server* S) {
         }
         for (ServerReq* r : admit) {
             r->lane = lane_of(r->cfg);
-            int rc = ccsd_create(&r->cfg, &r->in, S->lanes[r->lane].st, &r->h);
+            int rc = create_handle(&r->cfg, &r->in, S->lanes[r->lane].st, HandleUse::served, &r->h);
             if (rc) { server_finish(S, r, rc); continue; }
             r->polish_left = r->cfg.precision == CCSD_MIXED ? r->cfg.polish_iters : 0;
             if (r->cfg.precision == CCSD_MIXED) r->h->cfg.conv_tol = std::max(r->cfg.mixed_tol, r->cfg.conv_tol);
@@ -4097,28 +4197,7 @@ int ccsd_tc_timeout_selftest(void) {
 }
 
 int ccsd_create(const ccsd_config* cfg, const ccsd_inputs* in, void* stream, ccsd_t* out) {
-    ApiScope api_scope_;
-    if (!out) return CCSD_ERR_INVALID;
-    *out = nullptr;
-    if (!valid_cfg(cfg) || !in || (in->int_dtype != CCSD_C128 && in->int_dtype != CCSD_C64)) return CCSD_ERR_INVALID;
-    const void* ins[9] = {in->f_oo, in->f_vv, in->f_ov, in->oooo, in->ooov, in->oovv, in->ovvo, in->ovvv, in->vvvv};
-    for (const void* p : ins) if (!p) return CCSD_ERR_INVALID;
-    bool on_dev[9];
-    for (int i = 0; i < 9; ++i) on_dev[i] = is_device_ptr(ins[i]);
-    ccsd_ctx* h = new (std::nothrow) ccsd_ctx();
-    if (!h) return CCSD_ERR_OOM;
-    init_ctx(h, cfg);
-    h->st = (cudaStream_t)stream;
-    Alloc al{h};
-    auto fail = [&](int code) { ccsd_destroy(h); return code; };
-    int rc = setup_handle(h, al, ins, on_dev, in->int_dtype, in->vvvv_on_host != 0);
-    if (rc) return fail(rc);
-    for (int ei : h->const_embeds) launch_embed(h, h->embeds[ei]);
-    if (cudaMallocHost(&h->norm_host, 2 * sizeof(double)) != cudaSuccess) { cudaGetLastError(); h->norm_host = nullptr; return fail(CCSD_ERR_OOM); }
-    if (cudaEventCreateWithFlags(&h->ev_norm, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); h->ev_norm = nullptr; return fail(CCSD_ERR_CUDA); }
-    if (cudaStreamSynchronize(h->st) != cudaSuccess) return fail(CCSD_ERR_CUDA);
-    *out = h;
-    return CCSD_OK;
+    return create_handle(cfg, in, stream, HandleUse::own, out);
 }
 
 int ccsd_residual(ccsd_t h, const void* t1, const void* t2, void* r1, void* r2) {
@@ -4127,7 +4206,7 @@ int ccsd_residual(ccsd_t h, const void* t1, const void* t2, void* r1, void* r2) 
     // the kernels read and write these directly: host memory is refused, not faulted on
     if (!is_device_ptr(t1) || !is_device_ptr(t2) || !is_device_ptr(r1) || !is_device_ptr(r2)) return CCSD_ERR_INVALID;
     h->launches = 0;
-    if (use_graph(h)) {
+    if (h->stage && use_graph(h)) {
         // the graph reads the staged amplitudes and writes the handle's residual buffer
         // (scratch between calls): one copy in, one out
         const PairCopyOp in{h->stage, h->stage + h->n1, (const double2*)t1, (const double2*)t2, h->n1, h->n2};
@@ -4332,7 +4411,7 @@ int ccsd_batch_create(int n, const ccsd_config* cfgs, const ccsd_inputs* inputs,
     if (cudaStreamCreateWithFlags(&B->st, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); B->st = nullptr; return fail(CCSD_ERR_CUDA); }
     for (int i = 0; i < n; ++i) {
         ccsd_t h = nullptr;
-        int rc = ccsd_create(&cfgs[i], &inputs[i], B->st, &h);
+        int rc = create_handle(&cfgs[i], &inputs[i], B->st, HandleUse::batch, &h);
         if (rc) return fail(rc);
         B->m.push_back(h);
     }

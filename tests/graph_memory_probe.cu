@@ -1,0 +1,90 @@
+// Host build of the library's plan code (no launches): the split workspaces of a replayed handle.
+#include "../paper_1911_00242_gb300/csrc/ccsd_api.cu"
+
+namespace ccsdk {
+void launch_zgemm(int, int, const GemmArgs&, int, cudaStream_t) {}
+void launch_zgemm_grouped(int, int, const GemmArgs*, const long long*, int, long long, int, cudaStream_t) {}
+}  // namespace ccsdk
+
+namespace {
+
+struct Dry {
+    ccsd_ctx h;
+    int rc;
+    Dry(const ccsd_config* c, int use) {
+        init_ctx(&h, c);
+        h.use = (HandleUse)use;
+        Alloc al{&h};
+        al.dry = true;
+        const bool on_dev[9] = {true, true, true, true, true, true, true, true, true};
+        rc = setup_handle(&h, al, nullptr, on_dev, CCSD_C128, false);
+    }
+};
+
+}  // namespace
+
+extern "C" long long probe_bytes(const ccsd_config* c, int use) {
+    Dry d(c, use);
+    return d.rc ? -1 : (long long)d.h.owned_bytes;
+}
+
+// Bit w: replayed in arithmetic w; bit 8: the handle stages ccsd_residual's arguments.
+extern "C" int probe_replays(const ccsd_config* c, int use) {
+    Dry d(c, use);
+    if (d.rc) return -1;
+    int m = d.h.stage ? 256 : 0;
+    for (int w = 0; w < ZG_ARITH; ++w) m |= d.h.graphable[w] ? 1 << w : 0;
+    return m;
+}
+
+// Pairs of steps whose partials or counters share memory although no path of the graph's edges
+// orders them, in every arithmetic the handle replays; *shared counts the pairs that are ordered.
+extern "C" int probe_conflicts(const ccsd_config* c, int use, int* shared) {
+    Dry d(c, use);
+    *shared = 0;
+    if (d.rc) return -1;
+    ccsd_ctx* h = &d.h;
+    int bad = 0;
+    for (int w = 0; w < ZG_ARITH; ++w) {
+        if (!h->graphable[w]) continue;
+        h->fp32 = w == ZG_FP32;
+        h->oz_on = w == ZG_DF;
+        struct Use { int step, kind; long long off, n; };
+        std::vector<Use> us;
+        std::map<int, std::vector<int>> next;
+        HazardMap hz;
+        for (int i = 0; i < (int)h->seq.size(); ++i) {
+            const Step& st = h->seq[i];
+            if (!step_active(h, st)) continue;
+            for (int p : hz.add(i, step_access(h, st))) next[p].push_back(i);
+            if (st.kind == 0) {
+                const GemmPlan& g = h->gemms[st.idx];
+                const GemmVar& v = g.var[w];
+                if (v.nsplit < 2) continue;
+                us.push_back({i, 0, v.work_off, (long long)v.nsplit * g.args.nbatch * g.args.M * g.args.N});
+                us.push_back({i, 1, v.cnt_off, v.blocks});
+            } else if (st.kind == 6 && h->tcs[st.idx].oz && h->tcs[st.idx].z.nsplit > 1) {
+                const TcPlan& t = h->tcs[st.idx];
+                us.push_back({i, 2, t.work_off, (long long)t.z.nsplit * t.z.nbatch * t.z.M * (t.z.Nr / 2)});
+            }
+        }
+        for (const Use& a : us) {
+            std::set<int> seen{a.step};
+            std::vector<int> todo{a.step};
+            while (!todo.empty()) {
+                const int x = todo.back();
+                todo.pop_back();
+                for (int y : next[x]) if (seen.insert(y).second) todo.push_back(y);
+            }
+            for (const Use& b : us) {
+                if (b.step <= a.step || b.kind != a.kind) continue;
+                if (a.off + a.n <= b.off || b.off + b.n <= a.off) continue;
+                if (seen.count(b.step)) ++*shared; else ++bad;
+            }
+            const long long cap = a.kind == 0 ? (long long)h->work_elems : a.kind == 1 ? (long long)h->cnt_need
+                                                                                        : h->oz_work_elems;
+            if (a.off < 0 || a.off + a.n > cap) ++bad;
+        }
+    }
+    return bad;
+}

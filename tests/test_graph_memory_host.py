@@ -1,0 +1,69 @@
+"""Device memory that the graph replay of small problems costs: handles that replay share split
+workspaces between steps the graph orders, and handles that never replay (batch members, the
+grouped arithmetics of served solves) take no graph workspace and no staging copy."""
+import ctypes
+import random
+
+import pytest
+
+from helpers import build_host_probe
+
+OWN, BATCH, SERVED = 0, 1, 2
+
+
+@pytest.fixture(scope="module")
+def probe():
+    lib = build_host_probe("graph_memory_probe.cu", "graph_memory_probe")
+    lib.probe_bytes.restype = ctypes.c_longlong
+    return lib
+
+
+def config(grid, o, v, precision=0, polish=0, **more):
+    from paper_1911_00242_gb300 import binding
+    return binding.make_config(grid, o, v, precision=precision, polish_precision=polish, diis_depth=6, **more)
+
+
+# (grid, o, v, precision, MB of a handle whose steps use one workspace of two to four splits)
+@pytest.mark.parametrize("grid,o,v,precision,mb", [((2, 2, 1), 6, 20, 0, 311.8), ((2, 2, 1), 8, 32, 0, 1512.6),
+                                                   ((4, 1, 1), 4, 8, 0, 19.9), ((2, 2, 1), 7, 18, 0, 301.8),
+                                                   ((2, 2, 2), 4, 16, 0, 675.1), ((3, 1, 1), 5, 13, 2, 103.8),
+                                                   ((2, 2, 1), 6, 20, 1, 686.2)])
+def test_footprint_of_small_handles(probe, grid, o, v, precision, mb):
+    c = config(grid, o, v, precision)
+    own, batch, served = (probe.probe_bytes(ctypes.byref(c), use) for use in (OWN, BATCH, SERVED))
+    assert own < 1.5e6 * mb
+    assert batch <= served <= own
+    if precision != 2:
+        assert batch == served
+
+
+def test_replays_by_use(probe):
+    """Bits 0..2: FP64, FP32 and double-float (Ozaki) arithmetics; 256: staging copy."""
+    for precision, polish, own, served in ((0, 0, 1 + 256, 0), (1, 0, 3 + 256, 0), (1, 2, 7 + 256, 4), (2, 0, 5 + 256, 4)):
+        c = config((3, 1, 1), 5, 13, precision, polish)
+        assert probe.probe_replays(ctypes.byref(c), OWN) == own
+        assert probe.probe_replays(ctypes.byref(c), BATCH) == 0
+        assert probe.probe_replays(ctypes.byref(c), SERVED) == served
+    big = config((2, 2, 2), 8, 32)
+    assert probe.probe_replays(ctypes.byref(big), OWN) == 0
+
+
+def test_steps_that_share_memory_are_ordered(probe):
+    """Every pair of steps whose split partials or counters overlap is joined by a path of the
+    graph's edges, over forms, layouts and sizes on both sides of the packed hole-hole rule."""
+    rng = random.Random(11)
+    sizes = [((2, 2, 2), 10, 5), ((2, 1, 1), 33, 6), ((1, 1, 1), 49, 10), ((2, 2, 1), 8, 32)]
+    for _ in range(40):
+        sizes.append((rng.choice([(1, 1, 1), (2, 1, 1), (3, 1, 1), (2, 2, 1), (3, 2, 1), (2, 2, 2)]),
+                      rng.randint(1, 9), rng.randint(1, 24)))
+    total = 0
+    for grid, o, v in sizes:
+        for precision, polish in ((0, 0), (1, 0), (1, 2), (2, 0)):
+            for lean in (0, 1):
+                c = config(grid, o, v, precision, polish, lean=lean)
+                for use in (OWN, SERVED):
+                    shared = ctypes.c_int(0)
+                    bad = probe.probe_conflicts(ctypes.byref(c), use, ctypes.byref(shared))
+                    assert bad == 0, (grid, o, v, precision, polish, lean, use)
+                    total += shared.value
+    assert total > 1000
