@@ -323,6 +323,17 @@ long long wab_pairs_per_slab(long long N, long long v, long long cap) {
     return std::max<long long>(1, std::min<long long>(pairs, cap / pair_bytes));
 }
 
+// Operands a contraction of buffers a and b reads as complex128 in one arithmetic (the others
+// as complex64: inputs stored so, the copies of mixed iterations, the double-float copies).
+int wide_operands(const ccsd_ctx* h, int arith, int a, int b) {
+    auto wide = [&](int x) {
+        if (arith == ZG_FP32) return h->shadow[x] == nullptr;
+        const bool copied = x == B_OOOV || x == B_OVVV || x == B_OOVV || x == B_OVVO || x == B_T2 || x == B_TAUT;
+        return !h->in32[x] && !(arith == ZG_DF && copied);
+    };
+    return (wide(a) ? 1 : 0) + (wide(b) ? 1 : 0);
+}
+
 int finalize_gemm(ccsd_ctx* h, Alloc& al, GemmSpec s, size_t& work_need) {
     if (s.nbatch == 0) {
         // an empty contraction (no momentum blocks for this shape): kept as a no-op step
@@ -404,18 +415,11 @@ int finalize_gemm(ccsd_ctx* h, Alloc& al, GemmSpec s, size_t& work_need) {
     g.M = s.M; g.N = s.N; g.K = s.K; g.nbatch = s.nbatch; g.nchunk = s.nchunk;
     g.conjA = s.conjA; g.conjB = s.conjB; g.accumulate = s.acc ? 1 : 0;
     g.alpha_re = s.ar; g.alpha_im = s.ai;
-    // Tile shape and K split for each arithmetic the step may run in (zgemm_shapes.h); the
-    // operands with a complex64 copy in mixed iterations are those to_c64 refreshes
+    // Tile shape and K split for each arithmetic the step may run in (zgemm_shapes.h)
     for (int w = 0; w < ZG_ARITH; ++w) {
         if (w == ZG_FP32 && h->cfg.precision != CCSD_MIXED) { p.var[w] = p.var[ZG_FP64]; continue; }
         if (w == ZG_DF && !h->has_oz) { p.var[w] = p.var[ZG_FP64]; continue; }
-        auto wide = [&](int b) {
-            if (w == ZG_FP32) return h->shadow[b] == nullptr;
-            const bool copied = b == B_OOOV || b == B_OVVV || b == B_OOVV || b == B_OVVO || b == B_T2 || b == B_TAUT;
-            return !h->in32[b] && !(w == ZG_DF && copied);
-        };
-        const ZgChoice ch = zg_choose(w, s.M, s.N, s.K, s.nchunk, s.nbatch, (wide(s.a) ? 1 : 0) + (wide(s.b) ? 1 : 0),
-                                      kSMs);
+        const ZgChoice ch = zg_choose(w, s.M, s.N, s.K, s.nchunk, s.nbatch, wide_operands(h, w, s.a, s.b), kSMs);
         const ZgShape& sh = kZgShapes[ch.shape];
         GemmVar& v = p.var[w];
         v.shape = ch.shape; v.nsplit = ch.nsplit;
@@ -3091,6 +3095,27 @@ int batch_alloc(ccsd_batch* B, size_t bytes, void** p) {
     return 0;
 }
 
+// Tile shapes for one contraction step of members m that share a launch, the fastest first by the
+// summed estimate (each member with its best split of that shape).
+std::vector<int> rank_shapes(const std::vector<ccsd_ctx*>& m, size_t si, int arith) {
+    std::vector<std::pair<double, int>> order;
+    for (int c = 0; c < kZgShapeCount; ++c) {
+        double est = 0.0;
+        for (const ccsd_ctx* h : m) {
+            const GemmPlan& p = h->gemms[h->seq[si].idx];
+            const GemmArgs& a = p.args;
+            if (a.nbatch > 0)
+                est += zg_best_split(arith, c, a.M, a.N, a.K, a.nchunk, a.nbatch, wide_operands(h, arith, p.a, p.b),
+                                     kSMs).seconds;
+        }
+        order.emplace_back(est, c);
+    }
+    std::sort(order.begin(), order.end());
+    std::vector<int> out;
+    for (const auto& x : order) out.push_back(x.second);
+    return out;
+}
+
 // Autotuner: times the kTuneShapes tile shapes that the shape rule's model ranks first
 // for every grouped contraction (its ranking is within a few percent of the measured one,
 // so timing all shapes would only lengthen the first iteration) and keeps the fastest.
@@ -3111,24 +3136,9 @@ int batch_autotune(ccsd_batch* B) {
             const size_t si = G.steps[k];
             int best = bg.cfg;
             float best_ms = 1e30f;
-            std::vector<std::pair<double, int>> order;
-            for (int c = 0; c < kZgShapeCount; ++c) {
-                double est = 0.0;               // the members' tiles share the launch
-                for (const ccsd_ctx* h : G.m) {
-                    const GemmPlan& p = h->gemms[h->seq[si].idx];
-                    if (p.args.nbatch == 0) continue;
-                    const int c128 = (h->in32[p.a] ? 0 : 1) + (h->in32[p.b] ? 0 : 1);
-                    double one = 1e300;
-                    for (int ns : {1, 4, 16, kZgMaxSplit})
-                        one = std::min(one, zg_estimate(B->fp32 ? ZG_FP32 : ZG_FP64, c, ns, p.args.M, p.args.N,
-                                                        p.args.K, p.args.nchunk, p.args.nbatch, c128, kSMs));
-                    est += one;
-                }
-                order.emplace_back(est, c);
-            }
-            std::sort(order.begin(), order.end());
+            const std::vector<int> order = rank_shapes(G.m, si, B->fp32 ? ZG_FP32 : ZG_FP64);
             for (int q = 0; q < kTuneShapes; ++q) {
-                const int c = order[(size_t)q].second;
+                const int c = order[(size_t)q];
                 if ((rc = group_gemm_descriptors(G, bg, si, c, B->st))) break;
                 launch_gemm_group(bg, B->fp32, B->st, n);     // warm
                 cudaEventRecord(e0, B->st);

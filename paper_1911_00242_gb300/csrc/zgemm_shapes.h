@@ -104,19 +104,28 @@ inline long long zg_fp32_splits(int K, long long nchunk) {
     return (units + most - 1) / most;
 }
 
-inline ZgChoice zg_choose(int arith, int M, int N, int K, long long nchunk, long long nbatch, int c128, int sms) {
-    const int upc = (K + kZgUnit - 1) / kZgUnit;
-    const long long units = nchunk * upc;
+// The best K split of one shape: within the units there are, with FP32 sums as short as they must
+// be, and with bounded partials.
+inline ZgChoice zg_best_split(int arith, int shape, int M, int N, int K, long long nchunk, long long nbatch, int c128,
+                              int sms) {
+    const long long units = nchunk * ((K + kZgUnit - 1) / kZgUnit);
     const long long lo = arith == ZG_FP32 ? zg_fp32_splits(K, nchunk) : 1;
-    ZgChoice best{0, (int)lo, 1e300};
+    ZgChoice best{shape, (int)lo, 1e300};
+    static const int kSplits[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
+    for (int want : kSplits) {
+        const long long ns = std::max<long long>(lo, std::min<long long>(want, units));
+        if (ns > lo && ns * nbatch * M * N > kZgMaxPartials) continue;
+        const double t = zg_estimate(arith, shape, (int)ns, M, N, K, nchunk, nbatch, c128, sms);
+        if (t < best.seconds) best = ZgChoice{shape, (int)ns, t};
+    }
+    return best;
+}
+
+inline ZgChoice zg_choose(int arith, int M, int N, int K, long long nchunk, long long nbatch, int c128, int sms) {
+    ZgChoice best{0, 1, 1e300};
     for (int i = 0; i < kZgShapeCount; ++i) {
-        static const int kSplits[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
-        for (int want : kSplits) {
-            const long long ns = std::max<long long>(lo, std::min<long long>(want, units));
-            if (ns > lo && ns * nbatch * M * N > kZgMaxPartials) continue;
-            const double t = zg_estimate(arith, i, (int)ns, M, N, K, nchunk, nbatch, c128, sms);
-            if (t < best.seconds) best = ZgChoice{i, (int)ns, t};
-        }
+        const ZgChoice c = zg_best_split(arith, i, M, N, K, nchunk, nbatch, c128, sms);
+        if (c.seconds < best.seconds) best = c;
     }
     return best;
 }

@@ -1,4 +1,5 @@
-// Host build of the library's plan code (no launches): the split workspaces of a replayed handle.
+// Host build of the library's plan code (no launches): the split workspaces of a replayed handle,
+// the tile shapes of grouped contractions.
 #include "../paper_1911_00242_gb300/csrc/ccsd_api.cu"
 
 namespace ccsdk {
@@ -11,13 +12,13 @@ namespace {
 struct Dry {
     ccsd_ctx h;
     int rc;
-    Dry(const ccsd_config* c, int use) {
+    Dry(const ccsd_config* c, int use, int dtype = CCSD_C128) {
         init_ctx(&h, c);
         h.use = (HandleUse)use;
         Alloc al{&h};
         al.dry = true;
         const bool on_dev[9] = {true, true, true, true, true, true, true, true, true};
-        rc = setup_handle(&h, al, nullptr, on_dev, CCSD_C128, false);
+        rc = setup_handle(&h, al, nullptr, on_dev, dtype, false);
     }
 };
 
@@ -87,4 +88,24 @@ extern "C" int probe_conflicts(const ccsd_config* c, int use, int* shared) {
         }
     }
     return bad;
+}
+
+// Shapes of contraction step number `gemm` (of those active in mixed or FP64 iterations) in rank
+// order, for a group of this one member; the shape its own plan takes in *own.  -1: no such step.
+extern "C" int probe_rank(const ccsd_config* c, int dtype, int fp32, int gemm, int* order, int* own) {
+    Dry d(c, 1, dtype);
+    if (d.rc) return -1;
+    ccsd_ctx* h = &d.h;
+    h->fp32 = fp32;
+    for (size_t si = 0; si < h->seq.size(); ++si) {
+        const Step& st = h->seq[si];
+        if (st.kind != 0 || !step_active(h, st) || gemm-- > 0) continue;
+        const GemmPlan& p = h->gemms[st.idx];
+        if (p.args.nbatch == 0) return 0;
+        const std::vector<int> r = rank_shapes({h}, si, fp32 ? ZG_FP32 : ZG_FP64);
+        for (size_t i = 0; i < r.size(); ++i) order[i] = r[i];
+        *own = p.var[fp32 ? ZG_FP32 : ZG_FP64].shape;
+        return (int)r.size();
+    }
+    return -1;
 }

@@ -67,3 +67,30 @@ def test_steps_that_share_memory_are_ordered(probe):
                     assert bad == 0, (grid, o, v, precision, polish, lean, use)
                     total += shared.value
     assert total > 1000
+
+
+def ranks(probe, c, dtype, fp32):
+    out = []
+    while True:
+        order, own = (ctypes.c_int * 16)(), ctypes.c_int(-1)
+        n = probe.probe_rank(ctypes.byref(c), dtype, fp32, len(out), order, ctypes.byref(own))
+        if n < 0:
+            return out
+        out.append((own.value, list(order[:n])))
+
+
+@pytest.mark.parametrize("grid,o,v", [((1, 1, 1), 6, 16), ((2, 1, 1), 4, 11), ((2, 2, 1), 8, 24), ((3, 1, 1), 5, 13)])
+@pytest.mark.parametrize("fp32", [0, 1])
+def test_autotuner_ranks_what_the_launch_reads(probe, grid, o, v, fp32):
+    """For a group of one member the first candidate is the shape of the member's own plan (same
+    model, same operand types, same splits), and mixed iterations, which read complex64 copies
+    of complex128 integrals, rank as with integrals stored complex64."""
+    c = config(grid, o, v, 1 if fp32 else 0)
+    got = ranks(probe, c, 0, fp32)
+    assert len(got) > 10
+    for own, order in got:
+        if order:
+            assert sorted(order) == sorted(set(order))
+            assert order[0] == own
+    if fp32:
+        assert got == ranks(probe, c, 1, fp32)
