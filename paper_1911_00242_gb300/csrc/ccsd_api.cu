@@ -2602,11 +2602,19 @@ struct BatchGroup {
     GemmArgs* d_args = nullptr;
     long long* d_prefix = nullptr;
     long long total = 0;
-    double2* work = nullptr;          // split partials and tile counters of this step
-    size_t work_cap = 0;
+    double2* work = nullptr;          // split partials and tile counters of this step, owned (the
+    size_t work_cap = 0;              // steps of a replayed iteration run side by side)
     int* cnt = nullptr;
     size_t cnt_cap = 0;
 };
+
+void group_split_free(BatchGroup& bg) {
+    if (bg.work) cudaFree(bg.work);
+    if (bg.cnt) cudaFree(bg.cnt);
+    bg.work = nullptr;
+    bg.cnt = nullptr;
+    bg.work_cap = bg.cnt_cap = 0;
+}
 
 // One grouped launch: enqueues itself on a stream (no host synchronization).
 struct GLaunch {
@@ -2696,6 +2704,7 @@ T* group_upload(Group& G, const std::vector<T>& v, cudaStream_t st, int* rc) {
 }
 
 void group_free(Group& G) {
+    for (BatchGroup& bg : G.gemms) group_split_free(bg);
     for (void* p : G.owned) cudaFree(p);
     if (G.pool) for (void* c : G.chunks) G.pool->free_chunks.push_back(c);
     ChunkPool* pool = G.pool;
@@ -2734,43 +2743,64 @@ long long tiles_for(const GemmArgs& a, int cfg, int* tm, int* tn) {
     return (long long)*tm * *tn * a.nbatch;
 }
 
-// The split partials and tile counters of one grouped contraction, grown to what it needs
-// (a region of its own: the steps of a replayed iteration run side by side).
-int group_split_space(Group& G, BatchGroup& bg, size_t work, size_t tiles, cudaStream_t st) {
-    if (work > bg.work_cap) {
-        void* w = nullptr;
-        if (cudaMalloc(&w, work * 16) != cudaSuccess) { cudaGetLastError(); return CCSD_ERR_OOM; }
-        G.owned.push_back(w);
-        bg.work = (double2*)w;
-        bg.work_cap = work;
+// Room for the split partials and tile counters of one grouped contraction.  A region that is
+// too small is freed once its launches have ended, and a larger one taken.
+int group_split_space(BatchGroup& bg, size_t work, size_t tiles, cudaStream_t st) {
+    if (work <= bg.work_cap && tiles <= bg.cnt_cap) return 0;
+    CK(cudaStreamSynchronize(st));
+    group_split_free(bg);
+    void *w = nullptr, *c = nullptr;
+    if (cudaMalloc(&w, work * 16) != cudaSuccess || cudaMalloc(&c, tiles * sizeof(int)) != cudaSuccess) {
+        cudaGetLastError();
+        if (w) cudaFree(w);
+        return CCSD_ERR_OOM;
     }
-    if (tiles > bg.cnt_cap) {
-        void* w = nullptr;
-        if (cudaMalloc(&w, tiles * sizeof(int)) != cudaSuccess) { cudaGetLastError(); return CCSD_ERR_OOM; }
-        G.owned.push_back(w);
-        CK(cudaMemsetAsync(w, 0, tiles * sizeof(int), st));
-        bg.cnt = (int*)w;
-        bg.cnt_cap = tiles;
-    }
+    bg.work = (double2*)w;
+    bg.cnt = (int*)c;
+    bg.work_cap = work;
+    bg.cnt_cap = tiles;
+    CK(cudaMemsetAsync(c, 0, tiles * sizeof(int), st));
     return 0;
 }
 
-int group_gemm_descriptors(Group& G, BatchGroup& bg, size_t si, int cfg, cudaStream_t st, bool own_split = false) {
+// K splits of each member in a grouped contraction of tile shape cfg, by load balance: the
+// persistent CTAs stride one work list, so no work item (a tile and its share of the sum)
+// should hold more than half the mean load of a CTA.  Contractions with few outputs (a few
+// tiles over a long K, like the F~ and R1 sums) are then spread over many CTAs even when the
+// whole group has plenty of tiles.  FP32 partial sums stay short.  least: only the splits that
+// they need.  (A split item holds at least half of the cap, so beyond those a launch has at most
+// 4 x 8 x 152 split items: 0.32 GB of partials in the largest tiles.)
+std::vector<int> group_splits(const std::vector<ccsd_ctx*>& m, size_t si, int cfg, int arith, bool least = false) {
+    double total_work = 0.0;             // sum over members of tiles x K x chunks
+    for (const ccsd_ctx* h : m) {
+        int tm, tn;
+        const GemmArgs& a = h->gemms[h->seq[si].idx].args;
+        total_work += (double)tiles_for(a, cfg, &tm, &tn) * a.K * a.nchunk;
+    }
+    const double item_cap = std::max(4.0 * kZgUnit, 0.5 * total_work / (double)(kSMs * 8));
+    std::vector<int> ns;
+    for (const ccsd_ctx* h : m) {
+        const GemmArgs& a = h->gemms[h->seq[si].idx].args;
+        const long long units = (long long)a.nchunk * ((a.K + kZgUnit - 1) / kZgUnit);
+        const int l = a.nbatch > 0 && arith == ZG_FP32 ? (int)zg_fp32_splits(a.K, a.nchunk) : 1;
+        const int n = a.nbatch == 0 || least ? l
+                    : std::max(l, (int)std::max<long long>(1, std::min<long long>(std::min<long long>(units, kZgMaxSplit),
+                                                   (long long)std::ceil((double)a.K * a.nchunk / item_cap))));
+        ns.push_back(n);
+    }
+    return ns;
+}
+
+// The launch of one contraction step over the members.  own_split: each with the splits and the
+// workspace of its own plan; otherwise group_splits, or the least splits (see there).
+int group_gemm_descriptors(Group& G, BatchGroup& bg, size_t si, int cfg, cudaStream_t st, bool own_split = false,
+                           bool least = false) {
     const int n = (int)G.m.size();
     const int arith = G.fp32 ? ZG_FP32 : ZG_FP64;
     bg.cfg = cfg;
     bg.args.clear();
-    // Split-K by load balance: the persistent CTAs stride one work list, so no work item
-    // (a tile and its share of the sum) should hold more than half the mean load of a
-    // CTA.  Contractions with few outputs (a few tiles over a long K, like the F~ and R1
-    // sums) are then spread over many CTAs even when the whole group has plenty of tiles.
-    double total_work = 0.0;             // sum over members of tiles x K x chunks
-    for (int i = 0; i < n; ++i) {
-        int tm, tn;
-        const GemmArgs& a0 = G.m[i]->gemms[G.m[i]->seq[si].idx].args;
-        total_work += (double)tiles_for(a0, cfg, &tm, &tn) * a0.K * a0.nchunk;
-    }
-    const double item_cap = std::max(4.0 * kZgUnit, 0.5 * total_work / (double)(kSMs * 8));
+    std::vector<int> splits;
+    if (!own_split) splits = group_splits(G.m, si, cfg, arith, least);
     long long tot = 0;
     std::vector<long long> prefix;
     size_t work = 0, tiles = 0;          // split partials and counters of the members that split
@@ -2779,17 +2809,10 @@ int group_gemm_descriptors(Group& G, BatchGroup& bg, size_t si, int cfg, cudaStr
         ccsd_ctx* h = G.m[i];
         const GemmPlan& p = h->gemms[h->seq[si].idx];
         const GemmVar& v = p.var[arith];
-        int tm, tn, ns = v.nsplit;
+        int tm, tn;
+        const int ns = own_split ? v.nsplit : splits[(size_t)i];
         tiles_for(p.args, cfg, &tm, &tn);
-        if (own_split) {
-            if (cfg != v.shape && v.blocks > 0) { refuse("members of a split-keeping group must share each step's tile shape"); return CCSD_ERR_INVALID; }
-        } else {
-            const long long units = (long long)p.args.nchunk * ((p.args.K + kZgUnit - 1) / kZgUnit);
-            ns = (int)std::max<long long>(1, std::min<long long>(std::min<long long>(units, kZgMaxSplit),
-                                              (long long)std::ceil((double)p.args.K * p.args.nchunk / item_cap)));
-            if (G.fp32) ns = std::max(ns, (int)zg_fp32_splits(p.args.K, p.args.nchunk));   // short FP32 partial sums
-            if (p.args.nbatch == 0) ns = 1;
-        }
+        if (own_split && cfg != v.shape && v.blocks > 0) { refuse("members of a split-keeping group must share each step's tile shape"); return CCSD_ERR_INVALID; }
         GemmArgs a = gemm_args(h, p, arith);
         if (!own_split && ns > 1) {
             work_off.push_back(work);
@@ -2808,8 +2831,8 @@ int group_gemm_descriptors(Group& G, BatchGroup& bg, size_t si, int cfg, cudaStr
     prefix.push_back(tot);
     bg.total = tot;
     if (work) {
-        const int rc = group_split_space(G, bg, work, tiles, st);
-        if (rc) return rc;
+        const int rc = group_split_space(bg, work, tiles, st);
+        if (rc) { bg.total = 0; return rc; }
         for (int i = 0; i < n; ++i) {
             GemmArgs& a = bg.args[(size_t)i];
             if (a.nsplit < 2) continue;
@@ -2876,7 +2899,9 @@ int group_build(Group& G, int fp32, const std::vector<int>& cfgs, double* d_norm
         switch (s0.kind) {
             case 0: {
                 const int cfg = gi < (int)cfgs.size() ? cfgs[gi] : group_shape(G, si, fp32 ? ZG_FP32 : ZG_FP64);
-                if ((rc = group_gemm_descriptors(G, G.gemms[gi], si, cfg, st, own_split))) return rc;
+                rc = group_gemm_descriptors(G, G.gemms[gi], si, cfg, st, own_split);
+                if (rc == CCSD_ERR_OOM && !own_split) rc = group_gemm_descriptors(G, G.gemms[gi], si, cfg, st, false, true);
+                if (rc) return rc;
                 const BatchGroup* bg = &G.gemms[gi];
                 gl.gemm = gi;
                 gl.launches = bg->total > 0 ? 1 : 0;
@@ -3139,7 +3164,9 @@ int batch_autotune(ccsd_batch* B) {
             const std::vector<int> order = rank_shapes(G.m, si, B->fp32 ? ZG_FP32 : ZG_FP64);
             for (int q = 0; q < kTuneShapes; ++q) {
                 const int c = order[(size_t)q];
-                if ((rc = group_gemm_descriptors(G, bg, si, c, B->st))) break;
+                rc = group_gemm_descriptors(G, bg, si, c, B->st);
+                if (rc == CCSD_ERR_OOM) { rc = 0; continue; }     // no room for this candidate's splits
+                if (rc) break;
                 launch_gemm_group(bg, B->fp32, B->st, n);     // warm
                 cudaEventRecord(e0, B->st);
                 launch_gemm_group(bg, B->fp32, B->st, n);
@@ -3152,7 +3179,13 @@ int batch_autotune(ccsd_batch* B) {
                 }
                 if (ms < best_ms) { best_ms = ms; best = c; }
             }
-            if (!rc) rc = group_gemm_descriptors(G, bg, si, best, B->st);
+            if (!rc) {
+                // the chosen shape's own room, and not the largest candidate's
+                CK(cudaStreamSynchronize(B->st));
+                group_split_free(bg);
+                rc = group_gemm_descriptors(G, bg, si, best, B->st);
+                if (rc == CCSD_ERR_OOM) rc = group_gemm_descriptors(G, bg, si, best, B->st, false, true);
+            }
             G.res[k].launches = bg.total > 0 ? 1 : 0;
             ++gi;
         }

@@ -109,3 +109,27 @@ extern "C" int probe_rank(const ccsd_config* c, int dtype, int fp32, int gemm, i
     }
     return -1;
 }
+
+// Elements of split partials in one launch of contraction step `gemm` (as in probe_rank) over n
+// members like this one, in tile shape cfg; *least: what the FP32 sums alone need.  -1: no such step.
+extern "C" long long probe_group_partials(const ccsd_config* c, int n, int fp32, int gemm, int cfg, long long* least) {
+    Dry d(c, 1);
+    if (d.rc) return -1;
+    ccsd_ctx* h = &d.h;
+    h->fp32 = fp32;
+    for (size_t si = 0; si < h->seq.size(); ++si) {
+        const Step& st = h->seq[si];
+        if (st.kind != 0 || !step_active(h, st) || gemm-- > 0) continue;
+        const GemmArgs& a = h->gemms[st.idx].args;
+        const std::vector<ccsd_ctx*> m((size_t)n, h);
+        long long out[2];
+        for (int q = 0; q < 2; ++q) {
+            out[q] = 0;
+            for (int ns : group_splits(m, si, cfg, fp32 ? ZG_FP32 : ZG_FP64, q == 1))
+                if (ns > 1) out[q] += (long long)ns * a.nbatch * a.M * a.N;
+        }
+        *least = out[1];
+        return out[0];
+    }
+    return -1;
+}

@@ -33,6 +33,28 @@ def build_host_probe(source, name):
     return lib
 
 
+def load_with_fakes(source, calls):
+    """The library's objects linked again with tests/<source>, whose __wrap_<call> stands in for
+    each CUDA call in `calls`; loaded as the binding declares it."""
+    from paper_1911_00242_gb300 import binding, build
+    objdir = os.path.join(ROOT, "_build", "lib")
+    objs = [os.path.join(objdir, os.path.splitext(os.path.basename(s))[0] + ".o") for s in build.SOURCES]
+    if not all(os.path.exists(o) for o in objs):
+        build.build()
+    outdir = os.path.join(ROOT, "_build", "probes")
+    os.makedirs(outdir, exist_ok=True)
+    out = os.path.join(outdir, f"lib{os.path.splitext(source)[0]}_{os.getpid()}.so")
+    wrap = [x for c in calls for x in ("-Xlinker", f"--wrap={c}")]
+    subprocess.run([build.nvcc(), *build.ARCH, "-shared", "-Xcompiler", "-fPIC", *wrap, "-o", out,
+                    os.path.join(ROOT, "tests", source), *objs], check=True)
+    save, binding._lib = binding._lib, None
+    try:
+        return binding.load(out)
+    finally:
+        binding._lib = save
+        os.unlink(out)
+
+
 def dense_bloch(spec):
     """Dense Bloch-basis tensor and Fock built from the real-space supercell by an
     explicit unitary transform (independent of the generator's block DFT).

@@ -1,13 +1,11 @@
 """A residual graph that cannot be instantiated is no error: the handle launches its steps one
 by one, with the same bits.  The failing call is a fake (an error code from a wrapped
 cudaGraphInstantiate in a second link of the library's objects); nothing faults on the device."""
-import os
-import subprocess
-
 import numpy as np
 import pytest
 
 import ccsd_synth as cs
+from helpers import load_with_fakes
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -15,22 +13,14 @@ pytestmark = pytest.mark.gpu
 
 @pytest.fixture(scope="module")
 def wrapped(lib):
-    """The library linked again with the fake in place of cudaGraphInstantiate."""
-    from paper_1911_00242_gb300 import binding, build
-    objdir = os.path.join(build.ROOT, "_build", "lib")
-    objs = [os.path.join(objdir, os.path.splitext(os.path.basename(s))[0] + ".o") for s in build.SOURCES]
-    if not all(os.path.exists(o) for o in objs):
-        build.build()
-    path = os.path.join(build.ROOT, "_build", "probes", f"libfallback_{os.getpid()}.so")
-    os.makedirs(os.path.dirname(path), exist_ok=True)
-    subprocess.run([build.nvcc(), *build.ARCH, "-shared", "-Xcompiler", "-fPIC", "-Xlinker", "--wrap=cudaGraphInstantiate",
-                    "-o", path, os.path.join(build.ROOT, "tests", "graph_fallback_wrap.cpp"), *objs], check=True)
-    save, binding._lib = binding._lib, None
+    """The library with a fake in place of cudaGraphInstantiate."""
+    from paper_1911_00242_gb300 import binding
+    save = binding._lib
+    binding._lib = load_with_fakes("graph_fallback_wrap.cpp", ["cudaGraphInstantiate"])
     try:
-        yield binding.load(path)
+        yield binding._lib
     finally:
         binding._lib = save
-        os.unlink(path)
 
 
 @pytest.mark.parametrize("precision", [0, 1, 2])

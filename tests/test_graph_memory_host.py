@@ -14,7 +14,7 @@ OWN, BATCH, SERVED = 0, 1, 2
 @pytest.fixture(scope="module")
 def probe():
     lib = build_host_probe("graph_memory_probe.cu", "graph_memory_probe")
-    lib.probe_bytes.restype = ctypes.c_longlong
+    lib.probe_bytes.restype = lib.probe_group_partials.restype = ctypes.c_longlong
     return lib
 
 
@@ -94,3 +94,20 @@ def test_autotuner_ranks_what_the_launch_reads(probe, grid, o, v, fp32):
             assert order[0] == own
     if fp32:
         assert got == ranks(probe, c, 1, fp32)
+
+
+@pytest.mark.parametrize("fp32", [0, 1])
+@pytest.mark.parametrize("members", [1, 4, 16, 64])
+def test_grouped_split_partials_are_bounded(probe, fp32, members):
+    """Beyond what its FP32 sums need, one grouped launch has at most 4 x 8 x 152 split items (twice
+    the loads of half a mean CTA share), of at most 64 x 64 outputs."""
+    for grid, o, v in (((2, 2, 1), 6, 20), ((2, 2, 2), 8, 24), ((1, 1, 1), 4, 8)):
+        c = config(grid, o, v, 1 if fp32 else 0)
+        gemm, got = 0, 0
+        while got >= 0:
+            for shape in range(12):
+                least = ctypes.c_longlong(0)
+                got = probe.probe_group_partials(ctypes.byref(c), members, fp32, gemm, shape, ctypes.byref(least))
+                assert got <= 4 * 8 * 152 * 4096 + least.value, (grid, gemm, shape)
+            gemm += 1
+        assert gemm > 10
