@@ -2597,7 +2597,8 @@ int run_residual(ccsd_ctx* h) {
 //   * max|R| per member, and the update of the members not yet converged.
 // The group's launch descriptors are built once per membership on the host.
 struct BatchGroup {
-    int cfg = 0;                      // tile shape of the launch
+    std::vector<ccsd_ctx*> m;         // members in the launch
+    int cfg = 0;                      // its tile shape
     std::vector<GemmArgs> args;       // per member, tiles for `cfg`, pointers resolved
     GemmArgs* d_args = nullptr;
     long long* d_prefix = nullptr;
@@ -2791,53 +2792,57 @@ std::vector<int> group_splits(const std::vector<ccsd_ctx*>& m, size_t si, int cf
     return ns;
 }
 
-// The launch of one contraction step over the members.  own_split: each with the splits and the
+// The launch of one contraction step over members bg.m.  own_split: each with the splits and the
 // workspace of its own plan; otherwise group_splits, or the least splits (see there).
 int group_gemm_descriptors(Group& G, BatchGroup& bg, size_t si, int cfg, cudaStream_t st, bool own_split = false,
                            bool least = false) {
-    const int n = (int)G.m.size();
+    const int n = (int)bg.m.size();
     const int arith = G.fp32 ? ZG_FP32 : ZG_FP64;
     bg.cfg = cfg;
     bg.args.clear();
     std::vector<int> splits;
-    if (!own_split) splits = group_splits(G.m, si, cfg, arith, least);
+    if (!own_split) splits = group_splits(bg.m, si, cfg, arith, least);
     long long tot = 0;
     std::vector<long long> prefix;
     size_t work = 0, tiles = 0;          // split partials and counters of the members that split
     std::vector<size_t> work_off, cnt_off;
     for (int i = 0; i < n; ++i) {
-        ccsd_ctx* h = G.m[i];
+        ccsd_ctx* h = bg.m[i];
         const GemmPlan& p = h->gemms[h->seq[si].idx];
         const GemmVar& v = p.var[arith];
         int tm, tn;
         const int ns = own_split ? v.nsplit : splits[(size_t)i];
-        tiles_for(p.args, cfg, &tm, &tn);
-        if (own_split && cfg != v.shape && v.blocks > 0) { refuse("members of a split-keeping group must share each step's tile shape"); return CCSD_ERR_INVALID; }
+        const long long tiles_i = tiles_for(p.args, cfg, &tm, &tn);
         GemmArgs a = gemm_args(h, p, arith);
-        if (!own_split && ns > 1) {
-            work_off.push_back(work);
-            cnt_off.push_back(tiles);
+        work_off.push_back(work);
+        cnt_off.push_back(tiles);
+        if (ns > 1) {
             work += (size_t)ns * a.nbatch * a.M * a.N;
-            tiles += (size_t)tm * tn * a.nbatch;
-        } else {
-            work_off.push_back(0);
-            cnt_off.push_back(0);
+            tiles += (size_t)tiles_i;         // (counted in this launch's tiles, not in the member's own shape's)
         }
         a.tiles_m = tm; a.tiles_n = tn; a.nsplit = ns;
         prefix.push_back(tot);
-        tot += (long long)tm * tn * a.nbatch * a.nsplit;
+        tot += tiles_i * a.nsplit;
         bg.args.push_back(a);
     }
     prefix.push_back(tot);
     bg.total = tot;
     if (work) {
-        const int rc = group_split_space(bg, work, tiles, st);
+        int rc = 0;
+        int* cnt = nullptr;
+        if (own_split) {                      // partials in the members' workspaces, counters with the tables
+            if (!(rc = group_alloc(G, tiles * sizeof(int), (void**)&cnt)))
+                CK(cudaMemsetAsync(cnt, 0, tiles * sizeof(int), st));
+        } else {
+            rc = group_split_space(bg, work, tiles, st);
+            cnt = bg.cnt;
+        }
         if (rc) { bg.total = 0; return rc; }
         for (int i = 0; i < n; ++i) {
             GemmArgs& a = bg.args[(size_t)i];
             if (a.nsplit < 2) continue;
-            a.work = bg.work + work_off[(size_t)i];
-            a.cnt = bg.cnt + cnt_off[(size_t)i];
+            if (!own_split) a.work = bg.work + work_off[(size_t)i];
+            a.cnt = cnt + cnt_off[(size_t)i];
         }
     }
     if (!bg.d_args) {
@@ -2853,9 +2858,9 @@ int group_gemm_descriptors(Group& G, BatchGroup& bg, size_t si, int cfg, cudaStr
     return 0;
 }
 
-void launch_gemm_group(const BatchGroup& bg, int fp32, cudaStream_t st, int n) {
+void launch_gemm_group(const BatchGroup& bg, int fp32, cudaStream_t st) {
     if (bg.total <= 0 || !bg.d_args) return;
-    launch_zgemm_grouped(fp32 ? ZG_FP32 : ZG_FP64, bg.cfg, bg.d_args, bg.d_prefix, n, bg.total,
+    launch_zgemm_grouped(fp32 ? ZG_FP32 : ZG_FP64, bg.cfg, bg.d_args, bg.d_prefix, (int)bg.m.size(), bg.total,
                          (int)std::min<long long>(bg.total, (long long)kSMs * 8), st);
 }
 
@@ -2868,12 +2873,44 @@ int group_shape(const Group& G, size_t si, int arith) {
     return 3;
 }
 
+// Members of a split-keeping group by what fixes the bits of a contraction beside its splits: the
+// K groups of their own shape (a K group adds the terms k = q, q + KS, .. of a chunk in order, in
+// every tile shape).  One launch serves a class, in the shape of those K groups that the summed
+// estimate ranks first.
+struct KGroupClass { int shape; std::vector<ccsd_ctx*> m; };
+std::vector<KGroupClass> kgroup_classes(const std::vector<ccsd_ctx*>& m, size_t si, int arith) {
+    std::map<int, std::vector<ccsd_ctx*>> by;
+    for (ccsd_ctx* h : m) {
+        const GemmVar& v = h->gemms[h->seq[si].idx].var[arith];
+        if (v.blocks > 0) by[kZgShapes[v.shape].ks].push_back(h);
+    }
+    std::vector<KGroupClass> out;
+    for (auto& kv : by) {
+        int best = -1;
+        double best_est = 0.0;
+        for (int c = 0; c < kZgShapeCount; ++c) {
+            if (kZgShapes[c].ks != kv.first) continue;
+            double est = 0.0;
+            for (const ccsd_ctx* h : kv.second) {
+                const GemmPlan& p = h->gemms[h->seq[si].idx];
+                const GemmArgs& a = p.args;
+                est += zg_estimate(arith, c, p.var[arith].nsplit, a.M, a.N, a.K, a.nchunk, a.nbatch,
+                                   wide_operands(h, arith, p.a, p.b), kSMs);
+            }
+            if (best < 0 || est < best_est) { best = c; best_est = est; }
+        }
+        out.push_back({best, kv.second});
+    }
+    return out;
+}
+constexpr int kKGroupClasses = 3;         // KS = 1, 2, 4
+
 // Builds every grouped launch of one iteration of the group's members.  d_norms[i]
 // receives member i's max|R| (null: the group allocates its own array); d_skip[i] != 0
 // skips its update (may be null: all update).  cfgs: tile shape of each contraction
 // step (empty: each step's own shape in member 0).  own_split: every member keeps the
-// split-K choice of its own plan (its results are then bitwise those of a plain
-// iteration; the members must share each step's tile shape).
+// split-K choice and the K groups of its own plan (its results are then bitwise those of a
+// plain iteration; a contraction step is one launch per class of kgroup_classes).
 int group_build(Group& G, int fp32, const std::vector<int>& cfgs, double* d_norms, const int* d_skip,
                 cudaStream_t st, bool own_split = false) {
     const int n = (int)G.m.size();
@@ -2890,7 +2927,7 @@ int group_build(Group& G, int fp32, const std::vector<int>& cfgs, double* d_norm
         if (step_active(h0, h0->seq[si])) G.steps.push_back(si);
     int ngemm = 0;
     for (size_t si : G.steps) if (h0->seq[si].kind == 0) ++ngemm;
-    G.gemms.assign(ngemm, BatchGroup());
+    G.gemms.assign((size_t)ngemm * (own_split ? kKGroupClasses : 1), BatchGroup());
     int gi = 0;
     ensure_smem_attr(SMEM_TC_GROUPED);
     for (size_t si : G.steps) {
@@ -2898,14 +2935,29 @@ int group_build(Group& G, int fp32, const std::vector<int>& cfgs, double* d_norm
         GLaunch gl;
         switch (s0.kind) {
             case 0: {
-                const int cfg = gi < (int)cfgs.size() ? cfgs[gi] : group_shape(G, si, fp32 ? ZG_FP32 : ZG_FP64);
-                rc = group_gemm_descriptors(G, G.gemms[gi], si, cfg, st, own_split);
-                if (rc == CCSD_ERR_OOM && !own_split) rc = group_gemm_descriptors(G, G.gemms[gi], si, cfg, st, false, true);
+                const int arith = fp32 ? ZG_FP32 : ZG_FP64;
+                if (own_split) {
+                    std::vector<const BatchGroup*> parts;
+                    for (KGroupClass& c : kgroup_classes(G.m, si, arith)) {
+                        BatchGroup& bg = G.gemms[gi++];
+                        bg.m = c.m;
+                        if ((rc = group_gemm_descriptors(G, bg, si, c.shape, st, true))) return rc;
+                        parts.push_back(&bg);
+                    }
+                    gl.launches = (int)parts.size();
+                    gl.fn = [parts, fp32](cudaStream_t s) { for (const BatchGroup* bg : parts) launch_gemm_group(*bg, fp32, s); };
+                    break;
+                }
+                BatchGroup& bg = G.gemms[gi];
+                bg.m = G.m;
+                const int cfg = gi < (int)cfgs.size() ? cfgs[gi] : group_shape(G, si, arith);
+                rc = group_gemm_descriptors(G, bg, si, cfg, st);
+                if (rc == CCSD_ERR_OOM) rc = group_gemm_descriptors(G, bg, si, cfg, st, false, true);
                 if (rc) return rc;
-                const BatchGroup* bg = &G.gemms[gi];
                 gl.gemm = gi;
-                gl.launches = bg->total > 0 ? 1 : 0;
-                gl.fn = [bg, fp32, n](cudaStream_t s) { launch_gemm_group(*bg, fp32, s, n); };
+                gl.launches = bg.total > 0 ? 1 : 0;
+                const BatchGroup* launch = &bg;
+                gl.fn = [launch, fp32](cudaStream_t s) { launch_gemm_group(*launch, fp32, s); };
                 ++gi;
                 break;
             }
@@ -3167,9 +3219,9 @@ int batch_autotune(ccsd_batch* B) {
                 rc = group_gemm_descriptors(G, bg, si, c, B->st);
                 if (rc == CCSD_ERR_OOM) { rc = 0; continue; }     // no room for this candidate's splits
                 if (rc) break;
-                launch_gemm_group(bg, B->fp32, B->st, n);     // warm
+                launch_gemm_group(bg, B->fp32, B->st);        // warm
                 cudaEventRecord(e0, B->st);
-                launch_gemm_group(bg, B->fp32, B->st, n);
+                launch_gemm_group(bg, B->fp32, B->st);
                 cudaEventRecord(e1, B->st);
                 float ms = 0.f;
                 if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
@@ -3652,11 +3704,12 @@ int iter_finish(ccsd_ctx* h, double mr, int* done) {
 // handle whose integrals and amplitudes stay resident until it finishes) and
 // advances all admitted solves in rounds.  A round is one iteration of every
 // admitted solve: the solves are partitioned into groups of equal plan signature,
-// precision state and contraction tile shapes, every step of the residual is ONE
-// grouped launch per group (the groups on streams of their own, forked from the
-// server's stream), all max|R| come back in one copy, and then each solve takes its
-// convergence test and update (with DIIS).  Group members keep the split-K choices
-// of their own plans, so a solve's iterates are bitwise those it has alone.  Solves
+// precision state and DIIS depth, every step of the residual is one grouped launch per
+// group (a contraction step one per K-group class of its members' shapes; the groups on
+// streams of their own, forked from the server's stream), all max|R| come back in one
+// copy, and then each solve takes its convergence test and update (with DIIS).  Group
+// members keep the split-K choices and K groups of their own plans, so a solve's
+// iterates are bitwise those it has alone.  Solves
 // in the Ozaki arithmetic run their residual on their own.  Converged solves retire,
 // free their memory and make room for the queue; a group is rebuilt only when its
 // membership changes.
@@ -3763,17 +3816,14 @@ void server_finish(ccsd_server* S, ServerReq* r, int state) {
     }
 }
 
-// Grouping key of a solve in its current arithmetic: solves with equal keys share every
-// grouped launch of a round.
+// Grouping key of a solve in its current arithmetic: solves with equal keys share the grouped
+// launches of a round.  Sizes and tile shapes are not in it: with the tile shapes, the 64 sizes
+// of the batched workload made 48 groups in four lanes (mixed), one for nearly every size, where
+// there are 6 now.  100 s of the serving workload, p50 / p99 of its small solves: 0.100 / 2.60 s
+// with the tile shapes, 0.076 / 1.50 s without.
 std::vector<long long> server_key(const ccsd_ctx* h) {
-    std::vector<long long> k{h->fp32, h->oz_on, h->cfg.precision};
-    for (const Step& st : h->seq) {
-        k.push_back(st.kind * 16 + st.mode);
-        if (st.kind == 0) {
-            const GemmVar& v = h->gemms[st.idx].var[h->fp32 ? ZG_FP32 : ZG_FP64];
-            k.push_back(v.blocks > 0 ? v.shape : -1);
-        }
-    }
+    std::vector<long long> k{h->fp32, h->oz_on, h->cfg.precision, h->cfg.diis_depth};
+    for (const Step& st : h->seq) k.push_back(st.kind * 16 + st.mode);
     return k;
 }
 

@@ -133,3 +133,35 @@ extern "C" long long probe_group_partials(const ccsd_config* c, int n, int fp32,
     }
     return -1;
 }
+
+// Grouping key of a served solve in FP64 (fp32 = 0) or mixed iterations, its lane first; returns
+// its length.
+extern "C" int probe_key(const ccsd_config* c, int fp32, long long* out, int cap) {
+    Dry d(c, 2);
+    if (d.rc) return -1;
+    d.h.fp32 = fp32;
+    const std::vector<long long> k = server_key(&d.h);
+    out[0] = lane_of(*c);
+    for (size_t i = 0; i < k.size() && (int)i + 1 < cap; ++i) out[i + 1] = k[i];
+    return (int)k.size() + 1;
+}
+
+// Launches of contraction step `gemm` (as in probe_rank) over two served members: how many, and
+// bit 8 set if a launch mixes shapes of different K groups with its members' own.
+extern "C" int probe_classes(const ccsd_config* c0, const ccsd_config* c1, int fp32, int gemm) {
+    Dry a(c0, 2), b(c1, 2);
+    if (a.rc || b.rc || a.h.seq.size() != b.h.seq.size()) return -1;
+    a.h.fp32 = b.h.fp32 = fp32;
+    const int arith = fp32 ? ZG_FP32 : ZG_FP64;
+    for (size_t si = 0; si < a.h.seq.size(); ++si) {
+        const Step& st = a.h.seq[si];
+        if (st.kind != 0 || !step_active(&a.h, st) || gemm-- > 0) continue;
+        const std::vector<KGroupClass> cl = kgroup_classes({&a.h, &b.h}, si, arith);
+        int out = (int)cl.size();
+        for (const KGroupClass& c : cl)
+            for (const ccsd_ctx* h : c.m)
+                if (kZgShapes[h->gemms[h->seq[si].idx].var[arith].shape].ks != kZgShapes[c.shape].ks) out |= 256;
+        return out;
+    }
+    return -1;
+}

@@ -111,3 +111,39 @@ def test_grouped_split_partials_are_bounded(probe, fp32, members):
                 assert got <= 4 * 8 * 152 * 4096 + least.value, (grid, gemm, shape)
             gemm += 1
         assert gemm > 10
+
+
+@pytest.mark.parametrize("count,seed,most", [(64, 2000, 26), (16, 4000, 13)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_served_solves_share_groups(probe, precision, count, seed, most):
+    """Groups of the batched workload's 64 sizes and of the serving workload's 16, all served at
+    once: no more than with a key of seven tile shapes picked by thresholds."""
+    import ccsd_synth as cs
+    keys = set()
+    for s in cs.batch_specs(count, seed):
+        c = config(s.grid, s.nocc, s.nvir, precision)
+        out = (ctypes.c_longlong * 512)()
+        n = probe.probe_key(ctypes.byref(c), precision, out, 512)
+        assert 0 < n < 512
+        keys.add(tuple(out[:n]))
+    assert len(keys) <= most
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_served_launches_keep_k_groups(probe, precision):
+    """Members of one group whose own shapes differ: each contraction launch has the K groups of all
+    its members' own shapes, so their sums keep their order."""
+    split = 0
+    for one, two in ((((2, 2, 1), 4, 8), ((2, 2, 1), 6, 14)), (((3, 1, 1), 2, 5), ((3, 1, 1), 7, 20)),
+                     (((3, 1, 1), 3, 7), ((3, 1, 1), 8, 13)), (((2, 2, 1), 5, 18), ((2, 2, 1), 8, 20))):
+        a, b = (config(*x, precision) for x in (one, two))
+        gemm = 0
+        while True:
+            n = probe.probe_classes(ctypes.byref(a), ctypes.byref(b), precision, gemm)
+            if n < 0:
+                break
+            assert n < 4
+            split += n > 1
+            gemm += 1
+        assert gemm > 10
+    assert split > 0
