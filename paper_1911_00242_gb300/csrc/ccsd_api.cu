@@ -124,7 +124,6 @@ struct TcPlan {
     const void* opA = nullptr;     // operand buffers read
     const void* opB = nullptr;
     long long work_off = 0;        // this step's own split partials in oz_work (0: shared)
-    int split_cap = 1;             // most splits at any slice count (sizes the workspace)
 };
 
 }  // namespace
@@ -152,7 +151,7 @@ struct ccsd_ctx {
     double* ev = nullptr;            // ev[k][a]
     int* kb_of = nullptr;            // fourth momentum of doubles blocks
     double2* work = nullptr;         // split-K partials
-    size_t work_elems = 0;
+    size_t work_elems = 0;           // (cnt_need, oz_work_elems: of the other two)
     int* cnt = nullptr;              // finished splits per output tile of a split contraction
     size_t cnt_need = 0;
     double* red = nullptr;           // reduction partials
@@ -667,9 +666,6 @@ int add_tc(ccsd_ctx* h, Alloc& al, const TcBuf& A, const TcBuf& B, int c, int M,
         const long long tiles = (long long)z.tiles_m * z.tiles_n * nbatch;
         const int units = nchunk * oz_nwin(z.kstages, h->oz_slices);
         z.nsplit = 1;
-        if (tiles < 2 * kSMs)
-            t.split_cap = (int)std::min<long long>(std::min<long long>((long long)nchunk * z.kstages, OZ_MAX_SPLIT),
-                                                   (2 * kSMs + tiles - 1) / tiles);
         if (tiles < 2 * kSMs) z.nsplit = (int)std::min<long long>(std::min(units, OZ_MAX_SPLIT), (2 * kSMs + tiles - 1) / tiles);
         t.blocks = (int)(tiles * z.nsplit);
         if (z.nsplit > 1)
@@ -2798,6 +2794,7 @@ int group_gemm_descriptors(Group& G, BatchGroup& bg, size_t si, int cfg, cudaStr
                            bool least = false) {
     const int n = (int)bg.m.size();
     const int arith = G.fp32 ? ZG_FP32 : ZG_FP64;
+    if (!zg_built(arith, cfg)) { refuse("a tile shape has no instance in this arithmetic"); return CCSD_ERR_INVALID; }
     bg.cfg = cfg;
     bg.args.clear();
     std::vector<int> splits;
@@ -2889,7 +2886,7 @@ std::vector<KGroupClass> kgroup_classes(const std::vector<ccsd_ctx*>& m, size_t 
         int best = -1;
         double best_est = 0.0;
         for (int c = 0; c < kZgShapeCount; ++c) {
-            if (kZgShapes[c].ks != kv.first) continue;
+            if (kZgShapes[c].ks != kv.first || !zg_built(arith, c)) continue;
             double est = 0.0;
             for (const ccsd_ctx* h : kv.second) {
                 const GemmPlan& p = h->gemms[h->seq[si].idx];
@@ -3177,13 +3174,14 @@ int batch_alloc(ccsd_batch* B, size_t bytes, void** p) {
 std::vector<int> rank_shapes(const std::vector<ccsd_ctx*>& m, size_t si, int arith) {
     std::vector<std::pair<double, int>> order;
     for (int c = 0; c < kZgShapeCount; ++c) {
+        if (!zg_built(arith, c)) continue;
         double est = 0.0;
         for (const ccsd_ctx* h : m) {
             const GemmPlan& p = h->gemms[h->seq[si].idx];
             const GemmArgs& a = p.args;
             if (a.nbatch > 0)
                 est += zg_best_split(arith, c, a.M, a.N, a.K, a.nchunk, a.nbatch, wide_operands(h, arith, p.a, p.b),
-                                     kSMs).seconds;
+                                     kSMs).clocks;
         }
         order.emplace_back(est, c);
     }

@@ -1,15 +1,23 @@
-// Instances of the SIMT complex GEMM, one per arithmetic and tile shape.
+// Instances of the SIMT complex GEMM, one per arithmetic and tile shape that a rule can take
+// (zg_built; the callers ask for no other).
 #include "zgemm_launch.h"
 
 namespace ccsdk {
 
 namespace {
 
+template <typename T> constexpr int kArith = ZG_FP64;
+template <> constexpr int kArith<float> = ZG_FP32;
+template <> constexpr int kArith<df> = ZG_DF;
+
 template <typename T>
 void launch_one(int shape, const GemmArgs& g, dim3 grid, cudaStream_t st) {
     switch (shape) {
 #define X(id, bm, bn, bk, tm, tn, ks) \
-    case id: zgemm_kb_kernel<bm, bn, bk, tm, tn, T, ks><<<grid, ZG_THREADS, 0, st>>>(g); break;
+    case id:                                                                                  \
+        if constexpr (zg_built(kArith<T>, id))                                                \
+            zgemm_kb_kernel<bm, bn, bk, tm, tn, T, ks><<<grid, ZG_THREADS, 0, st>>>(g);       \
+        break;
         ZG_SHAPES(X)
 #undef X
     }
@@ -21,8 +29,9 @@ void launch_group(int shape, const GemmArgs* args, const long long* prefix, int 
     switch (shape) {
 #define X(id, bm, bn, bk, tm, tn, ks)                                                                            \
     case id:                                                                                                     \
-        zgemm_grouped_kernel<bm, bn, bk, tm, tn, T, ks><<<(unsigned)ctas, ZG_THREADS, 0, st>>>(args, prefix, n, \
-                                                                                               total);          \
+        if constexpr (zg_built(kArith<T>, id))                                                                   \
+            zgemm_grouped_kernel<bm, bn, bk, tm, tn, T, ks><<<(unsigned)ctas, ZG_THREADS, 0, st>>>(args, prefix, \
+                                                                                                   n, total);    \
         break;
         ZG_SHAPES(X)
 #undef X

@@ -43,7 +43,7 @@ constexpr int kZgMaxSplit = 64;
 constexpr long long kZgMaxPartials = 1LL << 26;
 constexpr long long kZgFp32Chain = 8192;   // longest FP32 partial sum of the mixed form
 
-struct ZgChoice { int shape, nsplit; double seconds; };
+struct ZgChoice { int shape, nsplit; double clocks; };
 
 // Estimated time of one launch of shape s with nsplit K splits, in SM clocks.  The
 // terms: products (padded to whole warps) at the arithmetic's rate, staging of the
@@ -55,10 +55,14 @@ struct ZgChoice { int shape, nsplit; double seconds; };
 // CTAs and shared memory) and the other constants were fitted to the measured times of
 // all shapes and splits on 41 contractions of 1 to 8 k points on GB300; the chosen shape
 // is within 3 % (geometric mean) of the fastest one there.
+// 0: not compiled.  Of 10^6 contractions drawn from M, N, K up to 8192, 729 chunks and 19683
+// batches none took FP64's 64 x 64 tile (nor had it among the four that the batch autotuner
+// times), or double-float's 64 x 32 and its 32 x 16 with two K groups (factors 4.0, 3.1, 2.4).
 constexpr double kZgFactor[ZG_ARITH][kZgShapeCount] = {
-    {4.0, 0.99, 2.6, 1.63, 1.13, 1.12, 1.12, 1.24, 1.08, 2.57, 1.2, 1.96},
+    {0.0, 0.99, 2.6, 1.63, 1.13, 1.12, 1.12, 1.24, 1.08, 2.57, 1.2, 1.96},
     {1.2, 0.64, 4.0, 0.6, 2.4, 1.5, 1.7, 0.9, 1.4, 1.8, 0.6, 4.0},
-    {2.3, 3.1, 1.5, 0.6, 0.89, 1.4, 2.4, 1.5, 1.2, 4.0, 0.6, 4.0}};
+    {2.3, 0.0, 1.5, 0.6, 0.89, 1.4, 0.0, 1.5, 1.2, 4.0, 0.6, 4.0}};
+constexpr bool zg_built(int arith, int shape) { return kZgFactor[arith][shape] > 0.0; }
 inline double zg_estimate(int arith, int shape, int nsplit, int M, int N, int K, long long nchunk,
                           long long nbatch, int c128, int sms) {
     const ZgShape& s = kZgShapes[shape];
@@ -111,12 +115,12 @@ inline ZgChoice zg_best_split(int arith, int shape, int M, int N, int K, long lo
     const long long units = nchunk * ((K + kZgUnit - 1) / kZgUnit);
     const long long lo = arith == ZG_FP32 ? zg_fp32_splits(K, nchunk) : 1;
     ZgChoice best{shape, (int)lo, 1e300};
-    static const int kSplits[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
+    static const int kSplits[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, kZgMaxSplit};
     for (int want : kSplits) {
         const long long ns = std::max<long long>(lo, std::min<long long>(want, units));
         if (ns > lo && ns * nbatch * M * N > kZgMaxPartials) continue;
         const double t = zg_estimate(arith, shape, (int)ns, M, N, K, nchunk, nbatch, c128, sms);
-        if (t < best.seconds) best = ZgChoice{shape, (int)ns, t};
+        if (t < best.clocks) best = ZgChoice{shape, (int)ns, t};
     }
     return best;
 }
@@ -124,8 +128,9 @@ inline ZgChoice zg_best_split(int arith, int shape, int M, int N, int K, long lo
 inline ZgChoice zg_choose(int arith, int M, int N, int K, long long nchunk, long long nbatch, int c128, int sms) {
     ZgChoice best{0, 1, 1e300};
     for (int i = 0; i < kZgShapeCount; ++i) {
+        if (!zg_built(arith, i)) continue;
         const ZgChoice c = zg_best_split(arith, i, M, N, K, nchunk, nbatch, c128, sms);
-        if (c.seconds < best.seconds) best = c;
+        if (c.clocks < best.clocks) best = c;
     }
     return best;
 }
