@@ -883,7 +883,8 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
         int KQ, kpl, kplp, kpr, kpo;
         long long epb;                       // bytes per operand element
         TcBuf la, lap, lb, ra, rb, b1, ha, hb, h2a, h2b;
-        TcBuf xb[2][2], wa[2], wb[2][2];     // packed hole-hole operands, by class (see pack_hh)
+        TcBuf xb[2][2], wa[2], wb[2][2];     // packed hole-hole operands, by class (see T.pack)
+        bool pack = false;                   // hole-hole packed by antisymmetry
         long long lb_floats;                 // ladder B capacity (elements per part / slice plane)
         long long lb_sc_rows;                // and its row scales (Ozaki): the (e < f) rows are shorter
         long long lad_max, lad_cap, pa, pb;  // sizes in elements per part / plane
@@ -902,11 +903,15 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
     // Hole-hole contractions on the tensor cores, packed by antisymmetry like the ladder: a
     // class of outputs and one of summed pairs, each (p < q) with all orbital pairs or (p = q)
     // with the ordered ones, a quarter of the products and of the tau operand.  The classes
-    // are up to four launches instead of one, so small problems (below kPackHhFlops) and the
-    // pooled layout keep the full sums.  At 2x2x2/o8/v32 the two steps take 3.6 ms instead of
-    // 8.2 (Ozaki) and 1.6 instead of 2.1 (mixed).
-    constexpr double kPackHhFlops = 4e9;
-    bool pack_hh = tcp && 8.0 * N * N * N * (double)N * oo * oo * vv >= kPackHhFlops;   // and not pooled (below)
+    // are up to four launches instead of one, so small problems and the pooled layout keep the
+    // full sums.  The lines, in the flops of the two contractions, by a residual's time packed over
+    // unpacked: Ozaki 1.32 at 0.07e9, 0.93..0.98 from 4e9 to 10e9, 0.87..0.95 above; mixed, whose
+    // GEMMs cost a sixth, by the number of classes: one (one k point) 0.98 at 4.8e9 and 0.91 at
+    // 12e9; two (2 k points along each axis at most) 1.18 at 4.8e9, 1.06 at 12e9, 0.98 at 24e9; four
+    // 1.14..1.39 at 5e9 to 8e9, 1.05 at 19e9, 1.02..1.04 at 33e9, 0.99..1.01 at 60e9, 0.98 above.  At
+    // 2x2x2/o8/v32 (137e9) the two steps take 3.6 ms instead of 8.2 (Ozaki) and 1.6 instead of 2.1
+    // (mixed).
+    const double hh_flops = 8.0 * N * N * N * (double)N * oo * oo * vv;
     struct PairClass { std::vector<std::pair<int, int>> pq; std::vector<std::vector<int>> in; };
     // pairs (p <= q) of class `diag` with the first members k of the summed pairs of class `diag_in`
     auto pair_class = [&](int diag, int diag_in) {
@@ -984,7 +989,10 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
             total_bytes += total * T.epb;
         }
         pooled = h->cfg.lean || total_bytes > (24LL << 30) * (long long)sets.size();
-        if (pooled) pack_hh = false;
+        int classes = 0;
+        for (int d = 0; d < 2; ++d) for (int e = 0; e < 2; ++e) classes += pair_class(d, e).pq.empty() ? 0 : 1;
+        const double mixed_line = classes <= 1 ? 4e9 : classes == 2 ? 1.6e10 : 6e10;
+        if (!pooled) for (TcSet& T : sets) T.pack = hh_flops >= (T.oz ? 4e9 : mixed_line);
         if (!pooled) {
             for (TcSet& T : sets) {
                 h->cur_oz = T.oz;
@@ -994,10 +1002,10 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
                     (rc = tc_alloc(h, al, T.lb, T.lb_floats / T.kpl + 1, T.kpl, T.lb_floats / std::max(T.kplp, T.KQ) + 1)) ||
                     (rc = tc_alloc(h, al, T.ra, N3l * ov, T.kpr)) || (rc = tc_alloc(h, al, T.rb, N3l * 2 * ov, T.kpr)) ||
                     (rc = tc_alloc(h, al, T.b1, N3l * 2 * ov, T.kpr)) ||
-                    (!pack_hh && ((rc = tc_alloc(h, al, T.ha, N3l * oo, T.kpl)) || (rc = tc_alloc(h, al, T.hb, N3l * 2 * oo, T.kpl)) ||
+                    (!T.pack && ((rc = tc_alloc(h, al, T.ha, N3l * oo, T.kpl)) || (rc = tc_alloc(h, al, T.hb, N3l * 2 * oo, T.kpl)) ||
                                   (rc = tc_alloc(h, al, T.h2a, N3l * oo, T.kpo)) || (rc = tc_alloc(h, al, T.h2b, N3l * 2 * vv, T.kpo)))))
                     return rc;
-                if (pack_hh) {
+                if (T.pack) {
                     const int kplt = (int)((2 * nlt_oo + T.KQ - 1) / T.KQ * T.KQ);
                     for (int d = 0; d < 2; ++d) for (int e = 0; e < 2; ++e) {
                         const long long blocks = class_blocks(pair_class(d, e));
@@ -1338,7 +1346,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
     std::vector<long long> so_lad;
     for (int S = 0; S < N; ++S) for (int ke = 0; ke < N; ++ke) for (int ki = 0; ki < N; ++ki)
         so_lad.push_back(blk(S2, ki, kg.k4(S, 0, ki), ke));
-    if (pack_hh) for (TcSet& T : sets) {
+    for (TcSet& T : sets) if (T.pack) {
         h->cur_oz = T.oz;
         // X packed: batches (km <= kn), rows (ki, ij) of tau (the ladder's operand), columns
         // the (m n) list of <mn||ef> (constant), K = (ke, ef list); mirror Whh(nm) = -Whh(mn)
@@ -1384,7 +1392,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
             }
         }
     }
-    if (!pack_hh) for (TcSet& T : sets) {
+    for (TcSet& T : sets) if (!T.pack) {
         h->cur_oz = T.oz;
         // X on tensor cores, one batch per momentum sum S = km + kn = ki + kj:
         // rows (km, mn) of <mn||ef> (constant operand), columns (ki, ij) of tau, K = (ke, ef)
@@ -1447,7 +1455,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
             if (tcp) h->seq.back().mode = 1;
         }
     }
-    if (pack_hh) for (TcSet& T : sets) {
+    for (TcSet& T : sets) if (T.pack) {
         h->cur_oz = T.oz;
         // R2 += tau_mn^ab Whh_mnij packed: batches (ka <= kb), rows (ki, ij) of Whh^T, columns
         // the (a b) list of tau, K = (km, mn list); mirror R2(ba) = -R2(ab)
@@ -1501,7 +1509,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
             }
         }
     }
-    if (!pack_hh) for (TcSet& T : sets) {
+    for (TcSet& T : sets) if (!T.pack) {
         h->cur_oz = T.oz;
         // R2 += 1/2 tau_mn^ab Whh_mnij on tensor cores, one batch per S = ki + kj:
         // rows (ki, ij) of Whh^T, columns (ka, ab) of tau, K = (km, mn)
@@ -1648,7 +1656,7 @@ int build_plan(ccsd_ctx* h, Alloc& al, size_t& work_need) {
             const std::vector<int>& efl = diag_ef ? lt_vv : full_vv;
             if (efl.empty()) continue;
             const TcBuf& A = diag_ef ? T.lap : T.la;
-            if (!pack_hh &&                  // (the packed X has embedded it)
+            if (!T.pack &&                   // (the packed X has embedded it)
                 (rc = add_embed(h, al, B_TAU, A, 0, (int)oo, (int)efl.size(), so_lad, tab({{(int)oo, vv}}), efl, false)))
                 return rc;
             for (int diag_ab = 0; diag_ab < 2; ++diag_ab) {

@@ -39,12 +39,36 @@ def test_packed_replay_equals_step_by_step(lib, grid, o, v, dtype, form):
     S.close()
 
 
+@pytest.mark.parametrize("grid,o,v,dtype", [((2, 2, 2), 14, 5, "c128"), ((2, 1, 1), 45, 6, "c64"), ((3, 1, 1), 40, 8, "c64"),
+                                            ((1, 1, 1), 49, 20, "c128")])
+def test_packed_mixed_residual(lib, grid, o, v, dtype):
+    """The mixed form from its own line on, against the FP64 form, replayed and step by step (bar as
+    for the parity tests: 1e-5 of max|R|)."""
+    from paper_1911_00242_gb300.binding import Solver
+    assert 8.0 * (grid[0] * grid[1] * grid[2]) ** 4 * o ** 4 * v ** 2 >= (6e10 if grid[0] == 3 else 1.6e10)
+    dev, t = problem(grid, o, v, dtype)
+    got = []
+    for precision in (0, 1):
+        S = Solver(grid, o, v, dev, precision=precision)
+        for trace in (False, True):
+            S.trace(trace)
+            r = [torch.full_like(x, float("nan")) for x in t]
+            S.residual(*t, *r)
+            torch.cuda.synchronize()
+            got.append(r)
+        S.close()
+    top = max(float(x.abs().max()) for x in got[0])
+    for x, y, z in zip(got[0], got[2], got[3]):
+        assert torch.equal(y, z)
+        assert float((x - y).abs().max()) < 1e-5 * top
+
+
 @pytest.mark.parametrize("precision", [0, 1])
 def test_batch_replays_agree(lib, precision):
     """Members on both sides of the packing rule (mixed), of uneven sizes, with DIIS."""
     import ctypes
     from paper_1911_00242_gb300 import binding
-    sizes = [((2, 2, 2), 10, 5), ((2, 1, 1), 3, 9), ((2, 2, 1), 5, 12), ((2, 1, 1), 33, 6), ((3, 1, 1), 4, 7)]
+    sizes = [((2, 2, 2), 14, 5), ((2, 1, 1), 3, 9), ((2, 2, 1), 5, 12), ((2, 1, 1), 45, 6), ((3, 1, 1), 4, 7)]
     probs = [problem(*s) for s in sizes]
     B = binding.BatchSolver([(g, o, v, d) for (g, o, v), (d, _) in zip(sizes, probs)], precision=precision, diis_depth=4,
                             conv_tol=0.0)
