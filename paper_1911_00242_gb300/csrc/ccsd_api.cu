@@ -52,6 +52,7 @@
 #include <new>
 #include <set>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 using namespace ccsdk;
@@ -4415,12 +4416,16 @@ int ccsd_set_precision(ccsd_t h, int precision) {
 int ccsd_energy(ccsd_t h, double* e_real, double* e_imag) {
     ApiScope api_scope_;
     if (!h) return CCSD_ERR_INVALID;
-    if (h->in32[B_OOVV])
-        energy_partial<<<h->red_blocks, 256, 0, h->st>>>(h->buf[B_T1], h->buf[B_T2], h->buf[B_FOV_IN], h->shadow[B_OOVV],
-                                                         h->N, h->o, h->v, h->cred);
-    else
-        energy_partial<<<h->red_blocks, 256, 0, h->st>>>(h->buf[B_T1], h->buf[B_T2], h->buf[B_FOV_IN], h->buf[B_OOVV],
-                                                         h->N, h->o, h->v, h->cred);
+    auto partial = [&](auto flat) {
+        if (h->in32[B_OOVV])
+            energy_partial<float2, decltype(flat)::value><<<h->red_blocks, 256, 0, h->st>>>(
+                h->buf[B_T1], h->buf[B_T2], h->buf[B_FOV_IN], h->shadow[B_OOVV], h->N, h->o, h->v, h->cred);
+        else
+            energy_partial<double2, decltype(flat)::value><<<h->red_blocks, 256, 0, h->st>>>(
+                h->buf[B_T1], h->buf[B_T2], h->buf[B_FOV_IN], h->buf[B_OOVV], h->N, h->o, h->v, h->cred);
+    };
+    if (energy_flat((long long)h->o * h->o * h->v * h->v)) partial(std::true_type{});
+    else partial(std::false_type{});
     final_csum<<<1, 32, 0, h->st>>>(h->cred, h->red_blocks, h->cred_out);
     CK(cudaMemcpyAsync(h->norm_host, h->cred_out, sizeof(double2), cudaMemcpyDeviceToHost, h->st));   // pinned
     CK(cudaStreamSynchronize(h->st));

@@ -272,58 +272,74 @@ __global__ void update_kernel(const UpdateOp op) { op.run(blockIdx.x, gridDim.x)
 
 // Energy partial sums: sum f_ia t_i^a + 1/4 sum <ij||ab> t_ij^ab
 //                    + 1/2 sum_{ki,kj} <i ki j kj||a ki b kj> t_i^a t_j^b.
-// A unit is 2048 elements of one momentum block (8 per thread, loaded together); the
-// element index is decoded only in the blocks with ka = ki, which have the t1 term.  The
+// A unit is 2048 elements (8 per thread, loaded together) of one momentum block, whose
+// element index is decoded only for ka = ki, where there is a t1 term; or, FLAT, of the
+// whole array, where every element finds its block first.  The
 // sum of <ij||ab> t_ij^ab is four FMAs per element, so the FP64 pipe (2 per clock and SM)
 // bounds it: at 2x2x2/o8/v32 0.21 ms, and 0.16 ms to read the 1.07 GB; ccsd_energy takes
 // 0.34 ms (0.68 ms with a pass that scaled t2, formed the product and decoded every element,
 // and one thread adding the blocks' sums).
 constexpr int kEnergyUnit = 2048;
-template <typename TS>
+// FLAT where the units of single blocks would be 15 % larger than the blocks.  By blocks and flat:
+// 3x3x3/o2/v6 (144 elements a block) 297 and 56 us, 3x3x2/o4/v18 (5184, 1.19) 300 and 277,
+// 3x2x1/o6/v20 (14400, 1.14) 64 and 74, 2x2x2/o8/v32 (65536, 1.0) 339 and 358.
+inline bool energy_flat(long long blk) {
+    return 20 * ((blk + kEnergyUnit - 1) / kEnergyUnit * kEnergyUnit) > 23 * blk;
+}
+
+// t += 2 t_i^a t_j^b (ki = ka) for element r = ((i o + j) v + a) v + b of a block.
+template <typename I>
+__device__ __forceinline__ void energy_t1_term(const double2* __restrict__ t1, I r, int ki, int kj, int o, int v, double2& t) {
+    const int b = (int)(r % (I)v); r /= (I)v;
+    const int a = (int)(r % (I)v); r /= (I)v;
+    const int j = (int)(r % (I)o), i = (int)(r / (I)o);
+    double2 x = t1[((long long)ki * o + i) * v + a];
+    const double2 y = t1[((long long)kj * o + j) * v + b];
+    x.x += x.x; x.y += x.y;
+    t.x = fma(x.x, y.x, t.x); t.x = fma(-x.y, y.y, t.x);
+    t.y = fma(x.x, y.y, t.y); t.y = fma(x.y, y.x, t.y);
+}
+
+template <typename TS, bool FLAT>
 __global__ void __launch_bounds__(256) energy_partial(
     const double2* __restrict__ t1, const double2* __restrict__ t2, const double2* __restrict__ fov,
     const TS* __restrict__ oovv, int N, int o, int v, double2* __restrict__ part)
 {
     __shared__ double2 sm[8];
     const long long n1 = (long long)N * o * v;
-    const long long blk = (long long)o * o * v * v;
-    const long long nseg = (blk + kEnergyUnit - 1) / kEnergyUnit;
+    const long long blk = (long long)o * o * v * v, n2 = blk * N * N * N;
+    const long long nseg = ((FLAT ? n2 : blk) + kEnergyUnit - 1) / kEnergyUnit;
     double d0[2] = {}, d1[2] = {}, d2[2] = {}, d3[2] = {};   // sum <ij||ab> (t_ij^ab + [t1 term])
     double sr = 0.0, si = 0.0;              // the f_ia t_i^a term
-    for (long long u = blockIdx.x; u < nseg * N * N * N; u += gridDim.x) {
-        const long long kk = u / nseg;
-        const long long e0 = (u - kk * nseg) * kEnergyUnit, base = kk * blk;
+    for (long long u = blockIdx.x; u < (FLAT ? nseg : nseg * N * N * N); u += gridDim.x) {
+        const long long kk = FLAT ? 0 : u / nseg;
+        const long long e0 = (u - kk * nseg) * kEnergyUnit, base = kk * blk, end = FLAT ? n2 : blk;
         const int ka = (int)(kk % N), kj = (int)((kk / N) % N), ki = (int)(kk / ((long long)N * N));
         double2 g[kEnergyUnit / 256], t[kEnergyUnit / 256];
 #pragma unroll
         for (int q = 0; q < kEnergyUnit / 256; ++q) {
             const long long e = e0 + q * 256 + threadIdx.x;
             g[q] = t[q] = make_double2(0.0, 0.0);
-            if (e < blk) { g[q] = ldz(oovv + base + e); t[q] = t2[base + e]; }
+            if (e < end) { g[q] = ldz(oovv + base + e); t[q] = t2[base + e]; }
         }
-        if (ka == ki) {
-            // t + 2 t_i^a t_j^b in place of t
+        if (FLAT) {
+            // blocks are short here (blk < 2^14), so block numbers and indices fit 32 bits
+#pragma unroll
+            for (int q = 0; q < kEnergyUnit / 256; ++q) {
+                const long long e = e0 + q * 256 + threadIdx.x;
+                if (e >= end) break;
+                const unsigned k = n2 < (1LL << 32) ? (unsigned)e / (unsigned)blk : (unsigned)(e / blk);
+                const int qa = (int)(k % (unsigned)N), qi = (int)(k / ((unsigned)N * (unsigned)N));
+                if (qa != qi) continue;
+                energy_t1_term(t1, (unsigned)(e - (long long)k * blk), qi, (int)(k / (unsigned)N % (unsigned)N), o, v, t[q]);
+            }
+        } else if (ka == ki) {
 #pragma unroll
             for (int q = 0; q < kEnergyUnit / 256; ++q) {
                 const long long e = e0 + q * 256 + threadIdx.x;
                 if (e >= blk) break;
-                int a, bb, i, j;
-                if (blk < (1LL << 31)) {
-                    unsigned r = (unsigned)e;
-                    bb = (int)(r % (unsigned)v); r /= (unsigned)v;
-                    a = (int)(r % (unsigned)v); r /= (unsigned)v;
-                    j = (int)(r % (unsigned)o); i = (int)(r / (unsigned)o);
-                } else {
-                    long long r = e;
-                    bb = (int)(r % v); r /= v;
-                    a = (int)(r % v); r /= v;
-                    j = (int)(r % o); i = (int)(r / o);
-                }
-                double2 x = t1[((long long)ki * o + i) * v + a];
-                const double2 y = t1[((long long)kj * o + j) * v + bb];
-                x.x += x.x; x.y += x.y;
-                t[q].x = fma(x.x, y.x, t[q].x); t[q].x = fma(-x.y, y.y, t[q].x);
-                t[q].y = fma(x.x, y.y, t[q].y); t[q].y = fma(x.y, y.x, t[q].y);
+                if (blk < (1LL << 31)) energy_t1_term(t1, (unsigned)e, ki, kj, o, v, t[q]);
+                else energy_t1_term(t1, e, ki, kj, o, v, t[q]);
             }
         }
 #pragma unroll
