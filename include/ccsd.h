@@ -121,7 +121,12 @@ typedef struct {
 /* Creates a solver for one problem.  `stream` is a cudaStream_t (NULL = the
  * legacy default stream) on the current device.  The amplitudes start at zero,
  * so the first update produces t0 = f(0) (paper Sec. 3.2.2).  Allocates all
- * work memory up front; returns CCSD_ERR_OOM if it does not fit. */
+ * work memory up front; returns CCSD_ERR_OOM if it does not fit.  Handles of up
+ * to 2^24 t2 elements build a CUDA graph of the residual in their first
+ * ccsd_residual and their first ccsd_iterate in each arithmetic (0.1 to 0.4 ms
+ * on the host, once) and replay it; where it cannot be built, and in calls made
+ * while the handle's stream is captured, the steps are launched one by one, with
+ * the same results. */
 int ccsd_create(const ccsd_config* cfg, const ccsd_inputs* in, void* stream, ccsd_t* out);
 
 /* Bytes of device memory ccsd_create allocates for this config when
@@ -252,7 +257,10 @@ int ccsd_destroy(ccsd_t h);
  * with its history, Gram matrix and Pulay solve kept in device memory -- is
  * replayed as one CUDA graph.  Members stop updating once their max|R| < conv_tol.
  * The problem data follow the rules of ccsd_create (device inputs borrowed).  Each
- * member extrapolates with its own handle's DIIS history, as ccsd_iterate does. */
+ * member extrapolates with its own handle's DIIS history, as ccsd_iterate does.  The
+ * first ccsd_batch_iterate may allocate workspace for split sums; launches for which
+ * there is no room run unsplit.  A member's own ccsd_residual and ccsd_iterate launch
+ * its steps one by one. */
 typedef struct ccsd_batch* ccsd_batch_t;
 int ccsd_batch_create(int n, const ccsd_config* cfgs, const ccsd_inputs* inputs, ccsd_batch_t* out);
 /* Up to n_iter iterations; done[i] / max_resid[i] per member (arrays of n, may be NULL). */
@@ -268,15 +276,15 @@ int ccsd_batch_destroy(ccsd_batch_t b);
 
 /* ---------------------------------------------------------------- serving form
  * A request loop on its own host thread.  Submitted solves wait in FIFO order
- * until their device-memory footprint fits in hbm_budget_bytes and one of
- * max_slots slots is free; each admitted solve gets a handle whose integrals and
+ * until the memory of their handle (at most ccsd_footprint) fits in hbm_budget_bytes
+ * and one of max_slots slots is free; each admitted solve gets a handle whose integrals and
  * amplitudes stay resident until it finishes.  Admitted solves advance in rounds,
  * one iteration each per round, in lanes by the order of magnitude of their
  * iteration's work: every lane has a stream of its own and runs its rounds at its own
  * pace, so small solves do not wait for the iterations of large ones.  Within a
- * lane's round, solves with the same plan signature, arithmetic and contraction tile
- * shapes form a group, and every step of their residual is one grouped launch (the
- * groups run concurrently); all max|R| come back in one copy, each solve takes its
+ * lane's round, solves with the same plan signature, arithmetic and DIIS depth form a
+ * group, and every step of their residual is one grouped launch, a contraction one to
+ * three (the groups run concurrently); all max|R| come back in one copy, each solve takes its
  * convergence test, and one grouped update (with DIIS) advances the solves that go
  * on.  A solve's iterates are bitwise those it has alone.  Converged solves retire
  * and free their memory for the queue.  A solve runs like ccsd_solve (mixed

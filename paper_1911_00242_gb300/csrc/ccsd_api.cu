@@ -304,12 +304,14 @@ struct GemmSpec {
 const int kSMs = 152;
 // Largest t2 (elements, 16 bytes each) of a problem whose residual is replayed as a graph.
 // A replay saves about 2 us of host time per launch and runs independent steps side by
-// side: a chain of 4 k points (n2 = 65 k) takes 0.72 ms step by step and 0.35 ms replayed,
-// one Ozaki iteration at 2x2x1/o8/v32 (n2 = 4 M) 9.0 and 8.1 ms, with equal bits.  At
-// 2x2x2/o8/v32 (n2 = 34 M) each step fills the chip (87.9 and 87.8 ms), and ccsd_residual's
-// arguments, copied in and out, cost memory and time.
+// side: a chain of 4 k points (n2 = 65 k) takes 0.72 ms step by step and 0.35 ms replayed.
+// Residuals step by step and replayed, FP64, mixed and Ozaki, with equal bits: 2x2x1/o8/v32
+// (4.2 M) 78.8 and 77.5, 3.3 and 2.4, 7.2 and 6.5 ms; 2x2x2/o6/v24 (10.6 M) 239 and 236, 6.5 and
+// 5.6, 18.8 and 17.7; 2x2x2/o8/v25 (20.5 M) 567 and 562, 11.0 and 10.1, 35.6 and 34.5; 2x2x2/o8/v32
+// (34 M) Ozaki 87.9 and 87.8.  Above the line the gain is some per cent, and the staged copies
+// of ccsd_residual's arguments and the regions of concurrent steps take gigabytes.
 const long long kGraphElems = 1LL << 24;
-const size_t kGraphWorkBytes = 1ull << 30;    // split partials (all steps') above which launches fill the chip
+const size_t kGraphWorkBytes = 1ull << 30;    // most split partials of all steps of a replayed residual
 // What a replay may take beside the step-by-step workspace (the split partials of steps that run
 // side by side, and the staged amplitudes): at most half of the handle's other memory.
 const size_t kGraphShare = 2;
