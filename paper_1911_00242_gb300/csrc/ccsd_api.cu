@@ -3386,7 +3386,7 @@ size_t place_regions(const std::vector<Region>& rs, const std::vector<std::vecto
 // replay would take more than its share of memory, and in handles that never replay (batch
 // members; grouped iterations of served solves), every step uses the front of one workspace,
 // one after another.  The regions a graph needs are some 1.0 to 1.3 times the largest step's: a
-// region each, as large as their sum, took 273 MB instead of 133 MB at 2x2x1/o6/v20 (FP64).
+// region each, as large as their sum, took 273 MB instead of 141 MB at 2x2x1/o6/v20 (FP64).
 void lay_out_graph(ccsd_ctx* h, size_t& work_need) {
     if (h->use == HandleUse::batch || h->n2 > kGraphElems) return;
     const int fp32 = h->fp32, oz_on = h->oz_on;
